@@ -69,7 +69,7 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     // every per-query cache is rebuilt for this query's coins
     ws.fl_on = 0;
     if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
-    SG_TRY(ensure_mask_cache(g, ws, co.W, st, co.lt != 0));
+    SG_TRY(ensure_mask_cache(g, ws, co, st));
 
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     struct EvGuard {

@@ -171,6 +171,7 @@ void free_graph_buffers(sg_graph *g, cudaStream_t st)
     dbuf_free(g->cin, st);
     dbuf_free(g->tmi, st);
     dbuf_free(g->fw, st);
+    dbuf_free(g->esrc, st);
     dbuf_free(g->hid_out, st);
     dbuf_free(g->hrow_out, st);
     dbuf_free(g->hpref_out, st);
@@ -216,11 +217,15 @@ sg_status finish_load(int64_t n, sgh::hvec<int32_t> &rp, sgh::hvec<int32_t> &col
     sgh::build_csc(n, rp, col, crp, cin);
     static_assert(sizeof(sgh::Arc2) == sizeof(int2), "CSC entries upload as int2");
     std::vector<uint32_t> tmi((size_t)n);
+    std::atomic<int64_t> n_in{0};
     sgh::parallel_rows(n, [&](int64_t a, int64_t b) {
+        int64_t in = 0;
         for (int64_t v = a; v < b; ++v) {
             const int64_t d = crp[(size_t)v + 1] - crp[(size_t)v];
             tmi[(size_t)v] = d > 0 ? (uint32_t)((1ull << 32) / (uint64_t)d - 1ull) : 0xffffffffu;
+            in += d > 0;
         }
+        n_in += in;
     });
     sg_graph *g = new (std::nothrow) sg_graph();
     if (!g) {
@@ -229,6 +234,7 @@ sg_status finish_load(int64_t n, sgh::hvec<int32_t> &rp, sgh::hvec<int32_t> &col
     }
     g->n = n;
     g->m = m;
+    g->n_in = n_in;
     sg_status rc = SG_OK;
     if (cudaGetDevice(&g->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) {
@@ -303,7 +309,7 @@ sg_status finish_load(int64_t n, sgh::hvec<int32_t> &rp, sgh::hvec<int32_t> &col
         delete g;
         return rc;
     }
-    if ((rc = ensure_wic(g, st)) != SG_OK) {
+    if ((rc = ensure_wic(g, st)) != SG_OK || (rc = build_arc_sources(g, st)) != SG_OK) {
         free_graph_buffers(g, st);
         delete g;
         return rc;
@@ -330,10 +336,19 @@ bool is_pageable(const void *p)
 
 }  // namespace
 
-void free_workspace(sg_workspace &ws, cudaStream_t st)
+static void free_core(sg_workspace &ws, cudaStream_t st)
 {
     dbuf_free(ws.s, st);
     dbuf_free(ws.cov, st);
+    dbuf_free(ws.ctl, st);
+    dbuf_free(ws.am_gain, st);
+    dbuf_free(ws.am_id, st);
+    ws.core_w = 0;
+}
+
+// The tiered engines' arrays and caches.
+static void free_tiers(sg_workspace &ws, cudaStream_t st)
+{
     dbuf_free(ws.nbits, st);
     dbuf_free(ws.pendf, st);
     dbuf_free(ws.fq_a, st);
@@ -395,14 +410,18 @@ void free_workspace(sg_workspace &ws, cudaStream_t st)
     dbuf_free(ws.slot_vis, st);
     dbuf_free(ws.slot_qa, st);
     dbuf_free(ws.slot_touched, st);
-    dbuf_free(ws.ctl, st);
-    dbuf_free(ws.am_gain, st);
-    dbuf_free(ws.am_id, st);
+    ws.wcap = 0;
+    ws.nslots = 0;
+}
+
+void free_workspace(sg_workspace &ws, cudaStream_t st)
+{
+    free_core(ws, st);
+    free_tiers(ws, st);
+    dbuf_free(ws.snap, st);
     dbuf_free(ws.out_seeds, st);
     dbuf_free(ws.out_gains, st);
-    ws.wcap = 0;
     ws.kcap = 0;
-    ws.nslots = 0;
 }
 
 GraphView view_of(const sg_graph *g, const sg_workspace &ws, int heavy_on)
@@ -444,14 +463,24 @@ static bool mask_cache_fits(const sg_graph *g, int32_t W)
     return g_mask_cache && g->m > 0 && mask_cache_bytes(g, W) <= ((size_t)16 << 30);
 }
 
-sg_status ensure_mask_cache(sg_graph *g, sg_workspace &ws, int32_t W, cudaStream_t st, bool required)
+// The linear threshold model's draws are per node, so every route keeps
+// them as masks.
+sg_status check_lt_masks(const sg_graph *g, const Coins &co)
 {
-    ws.lm_on = 0;
-    if (required && g->m > 0 && mask_cache_bytes(g, W) > ((size_t)16 << 30)) {
+    if (co.lt && g->m > 0 && mask_cache_bytes(g, co.W) > ((size_t)16 << 30)) {
         set_error("the linear threshold model needs the live-mask cache (2 x W x m x 8 = %zu bytes > 16 GiB)",
-                  mask_cache_bytes(g, W));
+                  mask_cache_bytes(g, co.W));
         return SG_ENOMEM;
     }
+    return SG_OK;
+}
+
+sg_status ensure_mask_cache(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st)
+{
+    const int32_t W = co.W;
+    const bool required = co.lt != 0;
+    ws.lm_on = 0;
+    SG_TRY(check_lt_masks(g, co));
     if (!required && !mask_cache_fits(g, W)) return SG_OK;
     if (g->m == 0) return SG_OK;
     if (ws.lm_cap < W) {
@@ -533,13 +562,19 @@ size_t tier3_budget(int64_t n)
     return std::min<size_t>(cap, std::max<size_t>((size_t)64 << 20, b));
 }
 
+size_t core_bytes(const sg_graph *g, int32_t W, int32_t k)
+{
+    const size_t n = (size_t)g->n;
+    return 8 * n + 8 * n * (size_t)W + (size_t)g->num_sms * 2 * 12 + (size_t)k * 12 + 4096;  // s, cov, partials, outputs
+}
+
 // Device bytes a workspace for (W, k) takes, as ensure_workspace /
 // ensure_heavy_index / ensure_snapshot_lists allocate them (upper bound).
 size_t workspace_bytes(const sg_graph *g, int32_t W, int32_t k)
 {
     const size_t n = (size_t)g->n, nw = n * (size_t)W, W64 = (size_t)64 * W;
-    size_t b = 8 * n;                                  // s
-    b += 8 * nw * 4;                                   // cov, nbits, pendf, bottom-up frontier
+    size_t b = core_bytes(g, W, k);
+    b += 8 * nw * 3;                                   // nbits, pendf, bottom-up frontier
     b += 4 * nw * (size_t)std::max(8, knobs().walk_groups) * 2;  // forward queues
     b += 4 * nw;                                       // du_x
     b += 4 * (nw + W64 + 64) * 2;                      // task lists
@@ -552,7 +587,6 @@ size_t workspace_bytes(const sg_graph *g, int32_t W, int32_t k)
     const size_t per_slot = n * 20 + (size_t)qcap * 4;
     const size_t slots = std::max<size_t>(1, std::min<size_t>((size_t)g->num_sms * SG_DENSE_BLOCKS, tier3_budget(g->n) / per_slot));
     b += slots * per_slot;
-    b += (size_t)g->num_sms * 2 * 12 + (size_t)k * 12 + 4096;
     if (heavy_index_enabled(g, W)) {
         b += (size_t)(g->hsum_out + g->hsum_in) * W * 12 + (size_t)(g->nh_out + g->nh_in) * W * 4;
         b += (size_t)g->n * W * 32;  // forward row descriptors
@@ -570,18 +604,41 @@ size_t workspace_bytes(const sg_graph *g, int32_t W, int32_t k)
     return b;
 }
 
+sg_status ensure_core(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, cudaStream_t st)
+{
+    if (ws.core_w < W) {
+        free_core(ws, st);
+        SG_TRY(dbuf_alloc(ws.s, (size_t)g->n, st));
+        SG_TRY(dbuf_alloc(ws.cov, (size_t)g->n * (size_t)W, st));
+        SG_TRY(dbuf_alloc(ws.ctl, 1, st));
+        ws.am_blocks = g->num_sms * 2;
+        SG_TRY(dbuf_alloc(ws.am_gain, (size_t)ws.am_blocks, st));
+        SG_TRY(dbuf_alloc(ws.am_id, (size_t)ws.am_blocks, st));
+        ws.n = g->n;
+        ws.core_w = W;
+    }
+    if (ws.kcap < k) {
+        dbuf_free(ws.out_seeds, st);
+        dbuf_free(ws.out_gains, st);
+        ws.kcap = 0;
+        SG_TRY(dbuf_alloc(ws.out_seeds, (size_t)k, st));
+        SG_TRY(dbuf_alloc(ws.out_gains, (size_t)k, st));
+        ws.kcap = k;
+    }
+    return SG_OK;
+}
+
 sg_status ensure_workspace(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, cudaStream_t st)
 {
     const int64_t n = g->n;
+    SG_TRY(ensure_core(g, ws, W, k, st));
     if (ws.wcap < W) {
-        free_workspace(ws, st);
+        free_tiers(ws, st);
         const size_t nw = (size_t)n * (size_t)W;
-        SG_TRY(dbuf_alloc(ws.s, (size_t)n, st));
-        SG_TRY(dbuf_alloc(ws.cov, nw, st));
         SG_TRY(dbuf_alloc(ws.nbits, nw, st));
         SG_TRY(dbuf_alloc(ws.pendf, nw, st));
         // one level queue per (word, walk group)
-        ws.fq_groups = std::max(8, knobs().walk_groups);
+        ws.fq_groups = std::max(8, std::max(knobs().walk_groups, g_walk_groups));
         SG_TRY(dbuf_alloc(ws.fq_a, nw * (size_t)ws.fq_groups, st));
         SG_TRY(dbuf_alloc(ws.fq_b, nw * (size_t)ws.fq_groups, st));
         SG_TRY(dbuf_alloc(ws.du_x, nw, st));
@@ -605,7 +662,6 @@ sg_status ensure_workspace(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, 
         SG_TRY(dbuf_alloc(ws.lmk_H, ((size_t)64 * W) << 8, st));
         SG_TRY(dbuf_alloc(ws.lmk_E, ((size_t)64 * W) << 8, st));
         SG_TRY(dbuf_alloc(ws.lmk_HE, ((size_t)64 * W) << 8, st));
-        SG_TRY(dbuf_alloc(ws.ctl, 1, st));
 
         SG_CUDA_TRY(cudaMemsetAsync(ws.nbits.p, 0, ws.nbits.bytes, st));
         SG_CUDA_TRY(cudaMemsetAsync(ws.pendf.p, 0, ws.pendf.bytes, st));
@@ -623,19 +679,8 @@ sg_status ensure_workspace(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, 
         SG_CUDA_TRY(cudaMemsetAsync(ws.slot_vis.p, 0, ws.slot_vis.bytes, st));
         SG_CUDA_TRY(cudaMemsetAsync(ws.slot_qa.p, 0xff, ws.slot_qa.bytes, st));
         ws.slot_qmask = qcap - 1;
-        ws.am_blocks = g->num_sms * 2;
-        SG_TRY(dbuf_alloc(ws.am_gain, (size_t)ws.am_blocks, st));
-        SG_TRY(dbuf_alloc(ws.am_id, (size_t)ws.am_blocks, st));
         ws.nslots = slots;
         ws.wcap = W;
-        ws.n = n;
-    }
-    if (ws.kcap < k) {
-        dbuf_free(ws.out_seeds, st);
-        dbuf_free(ws.out_gains, st);
-        SG_TRY(dbuf_alloc(ws.out_seeds, (size_t)k, st));
-        SG_TRY(dbuf_alloc(ws.out_gains, (size_t)k, st));
-        ws.kcap = k;
     }
     return SG_OK;
 }
@@ -1030,7 +1075,7 @@ sg_status cc_select_impl(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t
 {
     SG_TRY(cc_prepare_graph(g, st));
     const int launches0 = g_launches;
-    SG_TRY(ensure_workspace(g, ws, co.W, k, st));
+    SG_TRY(ensure_core(g, ws, co.W, k, st));
     SG_TRY(cc_ensure(g, ws, co.R, st));
     if (prepare_only) return SG_OK;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -1102,16 +1147,23 @@ sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_ca
         return cc_select_impl(g, ws, co, k, st, out_seeds, out_gains, stats, prepare_only);
     const int model = c.model == SG_WIC ? MODEL_WIC : MODEL_UIC;
     const int launches0 = g_launches;
-    SG_TRY(ensure_workspace(g, ws, co.W, k, st));
     // the linear threshold model reads every coin from the live-mask cache
     const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
-    if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
-    ws.slists_on = 0;
-    if (heavy_on && g_snapshot_lists) SG_TRY(ensure_snapshot_lists(g, ws, co, c.p, model, st));
-    ws.fl_on = 0;
-    if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
-    SG_TRY(ensure_mask_cache(g, ws, co.W, st, co.lt != 0));
-    ws.walk_groups = std::min(knobs().walk_groups, ws.fq_groups);
+    SG_TRY(check_lt_masks(g, co));
+    const bool snap = snap_route(g, co, model);
+    if (snap) {
+        SG_TRY(ensure_core(g, ws, co.W, k, st));
+        SG_TRY(ensure_snap(g, ws, co, model, st));
+    } else {
+        SG_TRY(ensure_workspace(g, ws, co.W, k, st));
+        if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
+        ws.slists_on = 0;
+        if (heavy_on && g_snapshot_lists) SG_TRY(ensure_snapshot_lists(g, ws, co, c.p, model, st));
+        ws.fl_on = 0;
+        if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
+        SG_TRY(ensure_mask_cache(g, ws, co, st));
+        ws.walk_groups = std::min(knobs().walk_groups, ws.fq_groups);
+    }
     if (prepare_only) return SG_OK;
     // events: 0 start, 1 after index, 2 after init tier 1, 3 after init,
     // 4 end; per round: after forward update
@@ -1142,25 +1194,32 @@ sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_ca
         for (auto &e : e_fwd) e = mark();
         SG_CUDA_TRY(cudaEventRecord(e_start, st));
     }
-    SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, (size_t)g->n * sizeof(long long), st));
     SG_CUDA_TRY(cudaMemsetAsync(ws.cov.p, 0, (size_t)g->n * (size_t)co.W * 8, st));
-    SG_CUDA_TRY(cudaMemsetAsync(ws.anc.p, 0, (size_t)g->n * (size_t)co.W * 8, st));
-    SG_CUDA_TRY(cudaMemsetAsync(ws.anc_cnt.p, 0, (size_t)co.W * (size_t)ws.fq_groups * 4, st));
     SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
-    if (heavy_on) {
-        SG_TRY(run_heavy_index(g, ws, co, model, st));
-        if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
-        SG_TRY(run_row_desc(g, ws, co, st));
-        ws.rd_on = 1;
+    if (snap) {
+        SG_TRY(run_snap_build(g, ws, co, model, st));
+    } else {
+        SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, (size_t)g->n * sizeof(long long), st));
+        SG_CUDA_TRY(cudaMemsetAsync(ws.anc.p, 0, (size_t)g->n * (size_t)co.W * 8, st));
+        SG_CUDA_TRY(cudaMemsetAsync(ws.anc_cnt.p, 0, (size_t)co.W * (size_t)ws.fq_groups * 4, st));
+        if (heavy_on) {
+            SG_TRY(run_heavy_index(g, ws, co, model, st));
+            if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
+            SG_TRY(run_row_desc(g, ws, co, st));
+            ws.rd_on = 1;
+        }
+        if (ws.slists_on) SG_TRY(run_snapshot_lists(g, ws, co, st));
+        if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
     }
-    if (ws.slists_on) SG_TRY(run_snapshot_lists(g, ws, co, st));
-    if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
     if (stats) SG_CUDA_TRY(cudaEventRecord(e_index, st));
-    SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st, stats ? &tev : nullptr));
+    if (snap) SG_TRY(run_snap_init(g, ws, co, model, stats != nullptr, st, stats ? &tev : nullptr));
+    else SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st, stats ? &tev : nullptr));
     if (stats) SG_CUDA_TRY(cudaEventRecord(e_init, st));
     for (int32_t i = 0; i < k; ++i) {
         if (stats) SG_CUDA_TRY(cudaEventRecord(e_round[(size_t)i], st));
-        SG_TRY(run_round(g, ws, co, model, heavy_on, i, st, stats ? e_fwd[(size_t)i] : nullptr));
+        const cudaEvent_t fwd = stats ? e_fwd[(size_t)i] : nullptr;
+        if (snap) SG_TRY(run_snap_round(g, ws, co, model, i, st, fwd));
+        else SG_TRY(run_round(g, ws, co, model, heavy_on, i, st, fwd));
     }
     SG_TRY(plant_injected_flags(ws, st));
     SG_TRY(run_poison(g, ws, ws.out_seeds.p, ws.out_gains.p, k, st));
@@ -1187,7 +1246,7 @@ sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_ca
         stats->status_flags = h.flags;
         stats->kernel_launches = g_launches - launches0;
         stats->heavy_index = heavy_on;
-        stats->mask_cache = ws.lm_on;
+        stats->mask_cache = snap ? (co.lt ? 1 : 0) : ws.lm_on;
         memcpy(stats->work_keys, h.work_keys, sizeof(h.work_keys));
         memcpy(stats->work_elems, h.work_elems, sizeof(h.work_elems));
         memcpy(stats->list_elems, h.list_elems, sizeof(h.list_elems));
@@ -1300,8 +1359,17 @@ sg_status sg_workspace_create(const sg_graph *g, int32_t R_max, int32_t k_max, v
     }
     sg_graph *gm = const_cast<sg_graph *>(g);
     const int32_t W = (R_max + 63) / 64;
-    sg_status rc = ensure_workspace(gm, *ws, W, k_max, st);
-    if (rc == SG_OK && heavy_index_enabled(g, W)) rc = ensure_heavy_index(gm, *ws, W, st);
+    // sized for a weighted-cascade query on the default route; another
+    // cascade or route adds what it needs when it first runs
+    Coins co;
+    sg_status rc = make_coins(sg_cascade{SG_WIC, 0.0}, 0, R_max, &co);
+    if (rc == SG_OK && snap_route(g, co, MODEL_WIC)) {
+        rc = ensure_core(gm, *ws, W, k_max, st);
+        if (rc == SG_OK) rc = ensure_snap(gm, *ws, co, MODEL_WIC, st);
+    } else if (rc == SG_OK) {
+        rc = ensure_workspace(gm, *ws, W, k_max, st);
+        if (rc == SG_OK && heavy_index_enabled(g, W)) rc = ensure_heavy_index(gm, *ws, W, st);
+    }
     if (rc == SG_OK && cudaStreamSynchronize(st) != cudaSuccess) {
         set_error("sg_workspace_create: %s", cudaGetErrorString(cudaGetLastError()));
         rc = SG_ECUDA;
@@ -1344,7 +1412,11 @@ sg_status sg_workspace_bytes(const sg_graph *g, int32_t R_max, int32_t k_max, si
         set_error("R_max must satisfy 1 <= R_max < 2^24");
         return SG_EINVAL;
     }
-    *bytes = workspace_bytes(g, (R_max + 63) / 64, k_max);
+    // enough for either route
+    const int32_t W = (R_max + 63) / 64;
+    Coins co;
+    SG_TRY(make_coins(sg_cascade{SG_WIC, 0.0}, 0, R_max, &co));
+    *bytes = std::max(workspace_bytes(g, W, k_max), core_bytes(g, W, k_max) + snap_bytes(g, co, MODEL_WIC));
     return SG_OK;
 }
 
@@ -1394,7 +1466,7 @@ sg_status sg_spread(sg_graph *g, int32_t R, sg_cascade c, uint64_t seed, const i
     if (rc == SG_OK && s_count > 0) {
         if (c.model == SG_UIC_UNDIRECTED) {
             rc = cc_prepare_graph(g, st);
-            if (rc == SG_OK) rc = ensure_workspace(g, g->ws, co.W, 1, st);
+            if (rc == SG_OK) rc = ensure_core(g, g->ws, co.W, 1, st);
             if (rc == SG_OK) rc = cc_ensure(g, g->ws, co.R, st);
             if (rc == SG_OK)
                 rc = cc_spread(g, g->ws, co, dS.p, s_count, dc.p, reinterpret_cast<unsigned long long *>(dc.p + 1),
@@ -1431,8 +1503,8 @@ sg_status sg_init_gains(sg_graph *g, int32_t R, sg_cascade c, uint64_t seed, voi
     cudaStream_t st = (cudaStream_t)stream;
     const int model = c.model == SG_WIC ? MODEL_WIC : MODEL_UIC;
     sg_workspace &ws = g->ws;
-    SG_TRY(ensure_workspace(g, ws, co.W, 1, st));
     if (c.model == SG_UIC_UNDIRECTED) {
+        SG_TRY(ensure_core(g, ws, co.W, 1, st));
         SG_TRY(cc_prepare_graph(g, st));
         SG_TRY(cc_ensure(g, ws, co.R, st));
         SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, (size_t)g->n * sizeof(long long), st));
@@ -1447,22 +1519,32 @@ sg_status sg_init_gains(sg_graph *g, int32_t R, sg_cascade c, uint64_t seed, voi
         if (init_edges) *init_edges = h.init_edges;
         return flags_status(h.flags);
     }
-    const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
-    if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
-    ws.slists_on = 0;
-    ws.fl_on = 0;
-    if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
-    SG_TRY(ensure_mask_cache(g, ws, co.W, st, co.lt != 0));
-    SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, (size_t)g->n * sizeof(long long), st));
-    SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
-    if (heavy_on) {
-        SG_TRY(run_heavy_index(g, ws, co, model, st));
-        if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
-        SG_TRY(run_row_desc(g, ws, co, st));
-        ws.rd_on = 1;
+    SG_TRY(check_lt_masks(g, co));
+    if (snap_route(g, co, model)) {
+        SG_TRY(ensure_core(g, ws, co.W, 1, st));
+        SG_TRY(ensure_snap(g, ws, co, model, st));
+        SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
+        SG_TRY(run_snap_build(g, ws, co, model, st));
+        SG_TRY(run_snap_init(g, ws, co, model, init_edges != nullptr, st, nullptr));
+    } else {
+        SG_TRY(ensure_workspace(g, ws, co.W, 1, st));
+        const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
+        if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
+        ws.slists_on = 0;
+        ws.fl_on = 0;
+        if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
+        SG_TRY(ensure_mask_cache(g, ws, co, st));
+        SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, (size_t)g->n * sizeof(long long), st));
+        SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
+        if (heavy_on) {
+            SG_TRY(run_heavy_index(g, ws, co, model, st));
+            if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
+            SG_TRY(run_row_desc(g, ws, co, st));
+            ws.rd_on = 1;
+        }
+        if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
+        SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st));
     }
-    if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
-    SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st));
     SG_TRY(plant_injected_flags(ws, st));
     SG_TRY(run_poison(g, ws, nullptr, ws.s.p, g->n, st));
     SG_CUDA_TRY(cudaMemcpyAsync(out_s, ws.s.p, (size_t)g->n * 8, cudaMemcpyDefault, st));

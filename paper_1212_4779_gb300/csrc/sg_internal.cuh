@@ -230,6 +230,56 @@ struct Ctl {
     long long du_total;   // reverse tasks of the current round
 };
 
+// One snapshot's compact graph (sg_snap_kernels.cuh).
+struct SnapInfo {
+    int32_t nI;        // internal nodes: a live out-arc
+    int32_t C;         // joins
+    int32_t L;         // live arcs
+    int32_t JA;        // arcs to joins
+    int32_t t0, t1;    // closure tasks, from the front / back of the task list
+    int32_t f0, f1;    // initial gains: sources that need a walk of their own, likewise
+    int32_t lmk_cnt, lmk_deg;  // nodes the landmark reaches, their out-degree sum
+    int32_t nrel;      // relevant joins of the round
+    int32_t bad;       // the snapshot has more live arcs than reserved
+};
+
+// Compact snapshot graphs of one query.  Strides: cap live arcs, icap
+// internal nodes, jcap joins, tcap tree nodes per snapshot; iw / jw / n32 /
+// m32 words of the bitmaps over internal nodes / joins / nodes / arcs.
+struct SnapView {
+    int32_t n, R, W, cap, icap, jcap, tcap, iw, jw;
+    int32_t wwarps;    // warps of a closure-walk launch
+    long long m, n32, m32;
+    const int32_t *rp, *col, *esrc, *crp;
+    const int2 *cin;
+    unsigned long long *any, *join, *oany;  // [W][n] snapshots with a live in-arc, several, a live out-arc
+    uint32_t *lb;                           // [R][m32] live arcs
+    uint32_t *outb, *joinb;                 // [R][n32] internal nodes, joins ...
+    int32_t *outp, *joinp;                  // ... and set bits before each word
+    SnapInfo *info;
+    int2 *arc;                              // [R][cap] live arcs in CSR order: (internal source, destination)
+    int32_t *inode, *par, *pend, *share, *jid;  // [R][icap] node id, tree parent, scratch, child with the
+                                                // same join range, join id
+    uint32_t *deg, *cnt;                    // [R][icap] out-degree sum of T(v); current marginal count
+    unsigned long long *acc;                // [R][icap] (arcs from T(v) to joins, |T(v)|)
+    unsigned long long *pj, *pn;            // [R][icap] (~root, first position in jarc) / (~root, ... in tn)
+    unsigned long long *cv;                 // [R][icap] closure totals of a walked range
+    int32_t *task, *fb, *ilist;             // [R][icap]
+    int4 *rec;                              // [R][jcap] join: |T|, out-degree sum, first join arc, join arcs
+    int32_t *jnode, *jint, *jlist;          // [R][jcap] node, internal node (-1: none), queue
+    int32_t *inoff;                         // [R][jcap + 1] in-arcs of a join in jin
+    uint32_t *jarc;                         // [R][cap] join arcs: target join, top bit set for a leaf
+    int32_t *jin;                           // [R][cap] in-arcs of joins (internal sources)
+    int32_t *tn;                            // [R][tcap] nodes of the trees, T(v) contiguous
+    uint32_t *covi, *marki;                 // [R][iw] covered / marked internal nodes
+    uint32_t *covj, *rel, *lmr;             // [R][jw] covered joins, a round's relevant ones, landmark's reach
+    uint2 *rel2;                            // [R][jw] word of rel, set bits before it
+    int4 *rrec;                             // [R][jcap] relevant joins by rank: weight, first join arc, join arcs
+    int32_t *cstart, *cnext, *arrive;       // chunk starts [2R + 1], most bits a walk needs, chunk size; counters
+    int32_t *wq;                            // walk queues
+    uint32_t *gbm;                          // [blocks][jw] visited bits too large for shared memory
+};
+
 }  // namespace sgi
 
 // Workspace owned by a graph handle and reused by every call on it.
@@ -238,6 +288,8 @@ struct sg_workspace {
     int device = 0;
     int64_t n = 0;
     int32_t wcap = 0;     // words of capacity of the [W][n] arrays
+    int32_t core_w = 0;   // words of capacity of cov
+    sgi::DBuf<unsigned char> snap;  // compact snapshot graphs, laid out per query
     int32_t nslots = 0;   // tier-3 (CTA engine) slots
     int32_t fq_groups = 0;    // forward-walk blocks per word the queues fq_a/fq_b were sized for
     int32_t walk_groups = 8;  // forward/landmark walk blocks per word for the current query
@@ -306,6 +358,8 @@ struct sg_graph {
     sgi::DBuf<int2> cin;
     sgi::DBuf<uint32_t> tmi;
     sgi::DBuf<uint2> fw;      // built on first WIC query
+    sgi::DBuf<int32_t> esrc;  // source of every arc
+    int64_t n_in = 0;         // nodes with an in-arc
     int32_t lmk_nodes[8] = {-1, -1, -1, -1, -1, -1, -1, -1};  // landmarks: largest out-degrees (>= 32)
     int32_t lmk_count = 0;
     // heavy rows (static)
@@ -326,11 +380,15 @@ namespace sgi {
 
 GraphView view_of(const sg_graph *g, const sg_workspace &ws, int heavy_on);
 sg_status ensure_wic(sg_graph *g, cudaStream_t st);
+// What every route of a query needs: gains, coverage, counters, outputs.
+sg_status ensure_core(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, cudaStream_t st);
+// ensure_core and the tiered engines' arrays.
 sg_status ensure_workspace(sg_graph *g, sg_workspace &ws, int32_t W, int32_t k, cudaStream_t st);
 sg_status ensure_heavy_index(sg_graph *g, sg_workspace &ws, int32_t W, cudaStream_t st);
 void free_workspace(sg_workspace &ws, cudaStream_t st);
 sg_status make_coins(const sg_cascade &c, uint64_t seed, int32_t R, Coins *out);
 bool heavy_index_enabled(const sg_graph *g, int32_t W);
+sg_status check_lt_masks(const sg_graph *g, const Coins &co);
 
 
 // kernels launched by this thread since the counter was last reset
@@ -394,6 +452,23 @@ extern int g_mask_cache;
 // nonzero: queries build and use forward per-snapshot live lists when they fit
 extern int g_fwd_lists;
 
+// events recorded around the initial-gain launches (any may be null): the
+// three engine tiers, or walks / counts / remaining walks
+struct TierEvents {
+    cudaEvent_t start = nullptr, t1 = nullptr, t2 = nullptr, t3 = nullptr;
+};
+
+// compact snapshot graphs (sg_snap.cu)
+bool snap_route(const sg_graph *g, const Coins &co, int model);
+size_t snap_bytes(const sg_graph *g, const Coins &co, int model);
+sg_status build_arc_sources(sg_graph *g, cudaStream_t st);
+sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
+sg_status run_snap_build(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
+sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, cudaStream_t st,
+                        const TierEvents *ev);
+sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t round, cudaStream_t st,
+                         cudaEvent_t after_cover);
+
 // kernels (sg_kernels.cu)
 sg_status run_heavy_index(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
 sg_status run_snapshot_lists(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st);
@@ -421,14 +496,12 @@ sg_status run_spread(sg_graph *g, const Coins &co, int model, const int32_t *d_S
 sg_status run_walk(sg_graph *g, const sg_workspace &ws, const Coins &co, int model, int heavy_on,
                    const int32_t *d_S, int32_t ns, unsigned long long *vis, unsigned long long *pend, int32_t *qa,
                    int32_t *qb, long long *d_total, unsigned long long *d_edges, cudaStream_t st);
-sg_status ensure_mask_cache(sg_graph *g, sg_workspace &ws, int32_t W, cudaStream_t st, bool required = false);
+sg_status ensure_mask_cache(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st);
 size_t mask_cache_bytes(const sg_graph *g, int32_t W);
 sg_status ensure_snapshot_lists(sg_graph *g, sg_workspace &ws, const Coins &co, double p_uic, int model,
                                 cudaStream_t st);
-// events recorded around the initial-gain tier launches (any may be null)
-struct TierEvents {
-    cudaEvent_t start = nullptr, t1 = nullptr, t2 = nullptr, t3 = nullptr;
-};
+sg_status run_lt_masks(sg_graph *g, const Coins &co, int w0, int words, unsigned long long *lm_in,
+                       unsigned long long *lm_out, unsigned long long *arc_major, int aW, cudaStream_t st);
 sg_status run_init_gains(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int heavy_on, cudaStream_t st,
                          const TierEvents *ev = nullptr);
 sg_status run_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int heavy_on, int32_t round,
@@ -440,7 +513,8 @@ sg_status run_live_masks(sg_graph *g, const Coins &co, int model, uint64_t *out,
 // Device flags (Ctl::flags) a query can leave: FLAG_NO_CANDIDATE, the argmax
 // found no candidate; FLAG_WAIT, a bounded device-side wait gave up;
 // FLAG_UNION_FIND, the union-find ran out of hooking retries.
-enum { FLAG_NO_CANDIDATE = 1, FLAG_WAIT = 2, FLAG_UNION_FIND = 8 };
+// FLAG_SNAPSHOT, a snapshot did not fit the compact graphs' reserve.
+enum { FLAG_NO_CANDIDATE = 1, FLAG_WAIT = 2, FLAG_UNION_FIND = 8, FLAG_SNAPSHOT = 16 };
 // SG_OK for flags 0; SG_ETIMEOUT when FLAG_WAIT is set; SG_EINTERNAL for
 // any other flag.  Sets the thread's error text on failure.
 sg_status flags_status(int32_t flags);
@@ -455,6 +529,7 @@ sg_status run_poison(const sg_graph *g, sg_workspace &ws, int32_t *seeds, long l
 sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_cascade c, uint64_t seed, void *stream,
                       int32_t *out_seeds, int64_t *out_gains, sg_stats *stats, bool prepare_only);
 sg_status check_query(const sg_graph *g, int32_t R, int32_t k);
+size_t core_bytes(const sg_graph *g, int32_t W, int32_t k);
 size_t workspace_bytes(const sg_graph *g, int32_t W, int32_t k);
 
 struct DeviceGuard {

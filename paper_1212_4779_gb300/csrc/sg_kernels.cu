@@ -2678,10 +2678,11 @@ sg_status init_gains_t(sg_graph *g, sg_workspace &ws, const Coins &co, int heavy
     return launch_tiers<DIR_FWD, MODEL, TASK_INIT>(g, ws, a, st, ev);
 }
 
-sg_status launch_argmax(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t round, cudaStream_t st)
+// For the routes that keep no per-word counts of newly covered nodes.
+sg_status launch_argmax(sg_graph *g, sg_workspace &ws, int32_t round, cudaStream_t st)
 {
     argmax_kernel<<<ws.am_blocks, AM_T, 0, st>>>(ws.s.p, (int)g->n, ws.ctl.p, ws.am_gain.p, ws.am_id.p,
-                                                 ws.out_seeds.p, ws.out_gains.p, round, ws.du_cnt.p, co.W);
+                                                 ws.out_seeds.p, ws.out_gains.p, round, nullptr, 0);
     SG_CUDA_TRY(cudaGetLastError());
     ++g_launches;
     return SG_OK;
@@ -2960,7 +2961,8 @@ sg_status run_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, i
 
 sg_status run_argmax(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t round, cudaStream_t st)
 {
-    return launch_argmax(g, ws, co, round, st);
+    (void)co;
+    return launch_argmax(g, ws, round, st);
 }
 
 sg_status run_live_masks(sg_graph *g, const Coins &co, int model, uint64_t *out, cudaStream_t st,

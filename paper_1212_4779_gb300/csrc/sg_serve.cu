@@ -228,18 +228,32 @@ void srv_retire(sg_server *s)
     }
 }
 
-// An idle workspace for (g, W), creating one within the memory budget
+// An idle workspace for a request, creating one within the memory budget
 // (releasing least recently used idle ones if needed).  -1: none now.
 // *fresh: the workspace was created now; its set-up (allocations and
 // clears) is queued on the setup stream and marked by setup_ev.  Nothing
 // here waits on the host.
-int srv_workspace(sg_server *s, sg_graph *g, int32_t W, bool *impossible, bool *fresh)
+int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fresh)
 {
     *impossible = false;
     *fresh = false;
+    sg_graph *g = rq->g;
+    const int32_t W = (rq->R + 63) / 64;
+    const int model = rq->c.model == SG_WIC ? MODEL_WIC : MODEL_UIC;
+    Coins co;
+    if (make_coins(rq->c, rq->seed, rq->R, &co) != SG_OK) {
+        *impossible = true;
+        return -1;
+    }
+    // the compact graphs' size depends on the cascade, the tiered engines'
+    // arrays only on the graph and W
+    const bool cc = rq->c.model == SG_UIC_UNDIRECTED;
+    const bool snap = !cc && snap_route(g, co, model);
+    const size_t core = core_bytes(g, W, s->cfg.k_cap);
+    const size_t need = cc ? core + cc_workspace_bytes(g, rq->R)
+                           : (snap ? core + snap_bytes(g, co, model) : workspace_bytes(g, W, s->cfg.k_cap));
     for (size_t i = 0; i < s->pool.size(); ++i)
-        if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W) return (int)i;
-    const size_t need = workspace_bytes(g, W, s->cfg.k_cap);
+        if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W && s->pool[i].bytes >= need) return (int)i;
     while (s->used + need > s->budget) {
         int lru = -1;
         for (size_t i = 0; i < s->pool.size(); ++i)
@@ -264,8 +278,9 @@ int srv_workspace(sg_server *s, sg_graph *g, int32_t W, bool *impossible, bool *
     sg_workspace *w = new (std::nothrow) sg_workspace();
     if (!w) return -1;
     cudaStream_t st = s->setup_st;
-    if (ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK ||
-        (heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
+    if (ensure_core(g, *w, W, s->cfg.k_cap, st) != SG_OK || (snap && ensure_snap(g, *w, co, model, st) != SG_OK) ||
+        (!snap && !cc && ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK) ||
+        (!snap && !cc && heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
         cudaEventRecord(s->setup_ev, st) != cudaSuccess) {
         free_workspace(*w, st);
         delete w;
@@ -295,9 +310,8 @@ void srv_admit(sg_server *s, std::unique_lock<std::mutex> &lock)
             }
         if (!free_slot) return;
         SrvRequest *r = s->queue.front();
-        const int32_t W = (r->R + 63) / 64;
         bool impossible = false, fresh = false;
-        const int wi = srv_workspace(s, r->g, W, &impossible, &fresh);
+        const int wi = srv_workspace(s, r, &impossible, &fresh);
         if (wi < 0) {
             if (!impossible) return;  // wait for memory
             s->queue.pop_front();

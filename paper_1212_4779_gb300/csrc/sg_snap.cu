@@ -1,0 +1,274 @@
+// sg_snap.cu -- the compact snapshot graphs: when a query takes them, their
+// device memory, and the launches (kernels in sg_snap_kernels.cuh).
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "sg_snap_kernels.cuh"
+
+namespace sgi {
+
+namespace {
+
+constexpr size_t SNAP_BYTES_MAX = (size_t)64 << 30;
+constexpr int WALK_BLOCKS = 2;                // closure-walk blocks per SM
+// Their shared memory for bitmaps and queues: over all joins (initial
+// gains), over the relevant ones (rounds, which leave more of the SM to L1
+// for the relevance bitmaps).
+constexpr int WALK_SMEM = 108 << 10;
+constexpr int ROUND_SMEM = 48 << 10;
+
+// Live arcs reserved per snapshot.  Their number is a sum of independent
+// coins: the mean plus 16 standard deviations (and a constant for small
+// means) is passed with a probability below e^-120; a snapshot that does
+// pass it is reported (FLAG_SNAPSHOT), never truncated.  LT keeps at most
+// one in-arc per node.
+int64_t live_cap(const sg_graph *g, const Coins &co, int model)
+{
+    double mean;
+    if (co.lt) return std::max<int64_t>(1, std::min(g->m, g->n_in));
+    if (model == MODEL_WIC) mean = (double)g->n_in;
+    else mean = co.none_live ? 0.0 : (double)g->m * (((double)co.uic_tm1 + 1.0) / 4294967296.0);
+    const double c = mean + 16.0 * std::sqrt(mean) + 256.0;
+    return std::max<int64_t>(1, std::min<int64_t>(g->m, (int64_t)c));
+}
+
+struct Carve {
+    unsigned char *base;
+    size_t off = 0;
+    template <class T>
+    void take(T *&p, size_t count)
+    {
+        off = (off + 255) & ~(size_t)255;
+        p = base ? reinterpret_cast<T *>(base + off) : nullptr;
+        off += count * sizeof(T);
+    }
+};
+
+// Lays the arrays out from `base` (NULL: sizes only); returns the bytes.
+// `clear` / `clear_bytes`: the leading part a query starts from zero.
+size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base, SnapView &v,
+             unsigned long long **lm, size_t *clear_bytes)
+{
+    v = SnapView{};
+    v.n = (int32_t)g->n;
+    v.m = g->m;
+    v.R = co.R;
+    v.W = co.W;
+    v.cap = (int32_t)live_cap(g, co, model);
+    v.icap = (int32_t)std::min<int64_t>(g->n, v.cap);
+    v.jcap = v.icap;
+    v.tcap = (int32_t)std::min<int64_t>(g->n, 2 * (int64_t)v.cap);
+    v.iw = (v.icap + 31) / 32;
+    v.jw = (v.jcap + 127) / 128 * 4;  // copied 16 bytes at a time
+    v.n32 = (g->n + 255) / 256 * 8;
+    v.m32 = (g->m + 255) / 256 * 8;
+    v.wwarps = g->num_sms * WALK_BLOCKS * WK_W;
+    v.rp = g->rp.p;
+    v.col = g->col.p;
+    v.esrc = g->esrc.p;
+    v.crp = g->crp.p;
+    v.cin = g->cin.p;
+    const size_t R = (size_t)co.R, nw = (size_t)g->n * co.W;
+    const size_t ri = R * v.icap, rj = R * v.jcap, rc = R * v.cap;
+    const size_t wb = (size_t)g->num_sms * WALK_BLOCKS;
+    Carve c{base};
+    c.take(v.cnext, 1);
+    c.take(v.arrive, 1);
+    c.take(v.any, nw);
+    c.take(v.join, nw);
+    c.take(v.oany, nw);
+    c.take(v.covi, R * v.iw);
+    c.take(v.covj, R * v.jw);
+    if (clear_bytes) *clear_bytes = c.off;
+    c.take(v.lb, R * v.m32);
+    c.take(v.outb, R * v.n32);
+    c.take(v.joinb, R * v.n32);
+    c.take(v.outp, R * v.n32);
+    c.take(v.joinp, R * v.n32);
+    c.take(v.info, R);
+    c.take(v.arc, rc);
+    c.take(v.inode, ri);
+    c.take(v.par, ri);
+    c.take(v.pend, ri);
+    c.take(v.share, ri);
+    c.take(v.jid, ri);
+    c.take(v.deg, ri);
+    c.take(v.cnt, ri);
+    c.take(v.acc, ri);
+    c.take(v.pj, ri);
+    c.take(v.pn, ri);
+    c.take(v.cv, ri);
+    c.take(v.task, ri);
+    c.take(v.fb, ri);
+    c.take(v.ilist, ri);
+    c.take(v.rec, rj);
+    c.take(v.jnode, rj);
+    c.take(v.jint, rj);
+    c.take(v.jlist, rj);
+    c.take(v.inoff, R * ((size_t)v.jcap + 1));
+    c.take(v.jarc, rc);
+    c.take(v.jin, rc);
+    c.take(v.tn, R * v.tcap);
+    c.take(v.marki, R * v.iw);
+    c.take(v.rel, R * v.jw);
+    c.take(v.rel2, R * v.jw);
+    c.take(v.lmr, R * v.jw);
+    c.take(v.rrec, rj);
+    c.take(v.cstart, 2 * R + 3);
+    c.take(v.wq, wb * WK_W * WK_QG);
+    c.take(v.gbm, wb * v.jw);
+    unsigned long long *masks = nullptr;
+    if (co.lt) c.take(masks, (size_t)g->m * co.W);
+    if (lm) *lm = masks;
+    return c.off;
+}
+
+__global__ void __launch_bounds__(256) arc_sources_kernel(int n, const int32_t *rp, int32_t *esrc)
+{
+    // one warp per row
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long u = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; u < n; u += nw)
+        for (int e = __ldg(rp + u) + lane; e < __ldg(rp + u + 1); e += 32) esrc[e] = (int32_t)u;
+}
+
+}  // namespace
+
+// The compact snapshot graphs serve every directed cascade and LT.  The
+// tiered engines remain for the calls that set one of their knobs (whoever
+// asks for a tier, a landmark count or a cache gets it), for graphs without
+// arcs, and where the graphs would pass SNAP_BYTES_MAX (dense cascades on
+// large graphs: about 100 bytes per live arc and snapshot).
+bool snap_route(const sg_graph *g, const Coins &co, int model)
+{
+    const Knobs k = knobs();
+    if (k.walk_groups != 64 || k.bu_mode != 1 || k.bu_div != 4 || k.t1_keys != 64 || k.t2_keys != 2048 ||
+        k.landmarks != 8 || k.scc != 1 || k.fwd_lists != 1 || k.word_major != 1 || k.t1_direct != 16)
+        return false;
+    if (g_mask_cache || !g_snapshot_lists || g->heavy_min_deg != 2 || g->m == 0) return false;
+    return snap_bytes(g, co, model) <= SNAP_BYTES_MAX;
+}
+
+size_t snap_bytes(const sg_graph *g, const Coins &co, int model)
+{
+    SnapView v;
+    return carve(g, co, model, nullptr, v, nullptr, nullptr);
+}
+
+sg_status build_arc_sources(sg_graph *g, cudaStream_t st)
+{
+    if (g->esrc.p || g->m == 0) return SG_OK;
+    SG_TRY(dbuf_alloc(g->esrc, (size_t)g->m, st));
+    const int blocks = (int)std::min<long long>((g->n * 32 + 255) / 256, (long long)g->num_sms * 16);
+    arc_sources_kernel<<<blocks, 256, 0, st>>>((int)g->n, g->rp.p, g->esrc.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    ++g_launches;
+    return SG_OK;
+}
+
+sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st)
+{
+    const size_t need = snap_bytes(g, co, model);
+    if (ws.snap.bytes < need) {
+        dbuf_free(ws.snap, st);
+        SG_TRY(dbuf_alloc(ws.snap, need, st));
+    }
+    return SG_OK;
+}
+
+namespace {
+
+template <int MODE, bool EDGES>
+sg_status launch_walk(sg_graph *g, sg_workspace &ws, const SnapView &v, cudaStream_t st)
+{
+    auto kern = snap_walk_kernel<MODE, EDGES>;
+    constexpr int smem = MODE == 2 ? ROUND_SMEM : WALK_SMEM;
+    SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kern<<<g->num_sms * WALK_BLOCKS, WK_T, smem, st>>>(v, ws.ctl.p, ws.s.p, smem);
+    SG_CUDA_TRY(cudaGetLastError());
+    ++g_launches;
+    return SG_OK;
+}
+
+}  // namespace
+
+// Threads of the kernels that give each snapshot one block.
+static int snap_threads(const SnapView &v) { return v.cap >= 8192 ? 1024 : 256; }
+
+// Coins and compact graphs of every snapshot.
+sg_status run_snap_build(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st)
+{
+    SnapView v;
+    unsigned long long *lm = nullptr;
+    size_t clear = 0;
+    carve(g, co, model, ws.snap.p, v, &lm, &clear);
+    SG_CUDA_TRY(cudaMemsetAsync(ws.snap.p, 0, clear, st));
+    const int tiles = (int)std::min<long long>((v.m + SN_TILE - 1) / SN_TILE, (long long)g->num_sms * 8);
+    if (co.lt) {
+        SG_CUDA_TRY(cudaMemsetAsync(lm, 0, (size_t)g->m * co.W * 8, st));
+        SG_TRY(run_lt_masks(g, co, 0, co.W, nullptr, lm, nullptr, 0, st));
+        snap_coins_kernel<2><<<tiles, SN_TILE, 0, st>>>(v, co, nullptr, lm);
+    } else if (model == MODEL_WIC) {
+        snap_coins_kernel<1><<<tiles, SN_TILE, 0, st>>>(v, co, g->fw.p, nullptr);
+    } else {
+        snap_coins_kernel<0><<<tiles, SN_TILE, 0, st>>>(v, co, nullptr, nullptr);
+    }
+    SG_CUDA_TRY(cudaGetLastError());
+    const int ntiles = (int)std::min<long long>(((long long)v.n + SN_TILE - 1) / SN_TILE, (long long)g->num_sms * 8);
+    snap_nodes_kernel<<<ntiles, SN_TILE, 0, st>>>(v, ws.ctl.p, ws.s.p);
+    snap_compact_kernel<<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p);
+    snap_trees_kernel<<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p);
+    snap_place_kernel<<<v.R, snap_threads(v), 0, st>>>(v);
+    SG_CUDA_TRY(cudaGetLastError());
+    g_launches += 5;
+    return SG_OK;
+}
+
+// Initial gains into ws.s; their edge count only if `edges`.
+sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, cudaStream_t st,
+                        const TierEvents *ev)
+{
+    SnapView v;
+    carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
+    if (ev && ev->start) SG_CUDA_TRY(cudaEventRecord(ev->start, st));
+    // blocks per snapshot of the kernels that give each internal node a thread
+    const int per = (int)std::max<long long>(1, std::min<long long>((v.icap + 1023) / 1024, (8LL * g->num_sms + v.R - 1) / v.R));
+    if (edges) snap_small_kernel<true><<<v.R * per, 256, 0, st>>>(v);
+    else snap_small_kernel<false><<<v.R * per, 256, 0, st>>>(v);
+    SG_CUDA_TRY(cudaGetLastError());
+    if (edges) SG_TRY((launch_walk<0, true>(g, ws, v, st)));
+    else SG_TRY((launch_walk<0, false>(g, ws, v, st)));
+    if (ev && ev->t1) SG_CUDA_TRY(cudaEventRecord(ev->t1, st));
+    if (edges) snap_resolve_kernel<true><<<v.R * per, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+    else snap_resolve_kernel<false><<<v.R * per, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    g_launches += 2;
+    if (ev && ev->t2) SG_CUDA_TRY(cudaEventRecord(ev->t2, st));
+    if (edges) SG_TRY((launch_walk<1, true>(g, ws, v, st)));
+    else SG_TRY((launch_walk<1, false>(g, ws, v, st)));
+    // the landmark marks give way to the rounds' marks
+    SG_CUDA_TRY(cudaMemsetAsync(v.marki, 0, (size_t)v.R * v.iw * 4, st));
+    if (ev && ev->t3) SG_CUDA_TRY(cudaEventRecord(ev->t3, st));
+    return SG_OK;
+}
+
+// One selection round: argmax, cover, update.
+sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t round, cudaStream_t st,
+                         cudaEvent_t after_cover)
+{
+    SnapView v;
+    carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
+    SG_TRY(run_argmax(g, ws, co, round, st));
+    const int T = snap_threads(v), lists = SW_CAP * T * 4;
+    SG_CUDA_TRY(cudaFuncSetAttribute(snap_cover_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lists));
+    snap_cover_kernel<<<v.R, T, lists, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    ++g_launches;
+    if (after_cover) SG_CUDA_TRY(cudaEventRecord(after_cover, st));
+    return launch_walk<2, false>(g, ws, v, st);
+}
+
+}  // namespace sgi

@@ -1,0 +1,1689 @@
+// sg_snap_kernels.cuh -- device kernels of the compact snapshot graphs (the
+// default route of a selection; sg_snap.cu launches them).
+//
+// Every snapshot's live graph is laid out once per query and contracted to
+// what reachability counts need.  In snapshot r:
+//   internal node   a node with a live out-arc (others reach only themselves)
+//   join            a node with two or more live in-arcs, or the lowest node
+//                   of a cycle of nodes with one live in-arc each
+//   tree            every other node has at most one live in-arc, so below
+//                   each join (and each node without in-arcs) hangs a tree;
+//                   T(v) is the subtree of v in it
+// T(v) is entered only through v, so |R(v)| = |T(v)| + the sizes |T(j)| of
+// the joins j reachable from v.  Tree nodes are laid out so that the arcs
+// leaving T(v) towards joins are one contiguous range J(v) of the snapshot's
+// join-arc list; a count is a closure walk over join ids alone, with one
+// visited bit per join.
+// On R-MAT 20 under the weighted cascade a snapshot's 450 K live arcs leave
+// 80 K joins (62 K of them with no join arc of their own), 179 K join arcs
+// and 28 K ranges to walk, 3 M arc visits in all, where walking the nodes
+// themselves visits 22 M; the snapshot takes about 4 MB, so the walks of a
+// few snapshots at a time stay in L2 and their visited bits in shared
+// memory.
+//
+// A selection round covers R(v*) in each snapshot (closed under
+// reachability, so later walks skip covered joins), marks the uncovered
+// nodes that reach a newly covered join, and subtracts from each of them
+// the newly covered nodes it reaches: all of them for the ancestors of v*,
+// else a closure walk restricted to the marked and newly covered joins.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "sg_internal.cuh"
+
+namespace sgi {
+namespace {
+
+constexpr unsigned SN_FULL = 0xffffffffu;
+constexpr int SN_T = 1024;      // most threads of the one-block-per-snapshot kernels
+constexpr int SN_TILE = 256;    // arcs or nodes per block pass of the bit transposes
+constexpr int WK_T = 512;       // threads of the closure walks
+constexpr int WK_W = WK_T / 32;
+constexpr int WK_QS = 128;      // queue entries of a walk in shared memory
+constexpr int WK_QG = 8192;     // ... and in global memory
+constexpr int WK_TS = 128;      // visited joins remembered for a cheap undo
+constexpr int WK_CH = 16;       // most tasks a warp claims at a time
+constexpr int SW_CAP = 16;      // joins a one-thread walk may visit
+constexpr int SW_ARCS = 96;     // ... and arcs it may scan
+constexpr int WK_U = 4;         // arcs in flight per lane
+constexpr uint32_t CV_CYCLE = 0x80000000u;
+constexpr uint32_t ARC_LEAF = 0x80000000u;  // jarc: the join has no live out-arc (weight 1, nothing below)
+
+__device__ __forceinline__ uint64_t sn_word_mask(int word, int R)
+{
+    const int rem = R - word * 64;
+    return rem >= 64 ? ~0ull : ((1ull << rem) - 1ull);
+}
+
+__device__ __forceinline__ bool sn_bit(const uint32_t *b, int i) { return (b[i >> 5] >> (i & 31)) & 1u; }
+
+// number of set bits of bitmap b below position i (p: exclusive prefix per word)
+__device__ __forceinline__ int sn_rank(const uint32_t *b, const int32_t *p, int i)
+{
+    return p[i >> 5] + __popc(b[i >> 5] & ((1u << (i & 31)) - 1u));
+}
+
+// (j+1)-th lowest set bit of m, j < popc(m)
+__device__ __forceinline__ int sn_nth_bit(uint32_t m, int j)
+{
+    int pos = 0;
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+        const int c = __popc(m & ((1u << w) - 1u));
+        if (j >= c) {
+            j -= c;
+            m >>= w;
+            pos += w;
+        }
+    }
+    return pos;
+}
+
+__device__ __forceinline__ int sn_warp_incl(int v, int lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(SN_FULL, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long sn_pack(int hi, uint32_t lo)
+{
+    return ((unsigned long long)(uint32_t)hi << 32) | lo;
+}
+__device__ __forceinline__ int sn_hi(unsigned long long w) { return (int)(w >> 32); }
+__device__ __forceinline__ uint32_t sn_lo(unsigned long long w) { return (uint32_t)w; }
+__device__ __forceinline__ unsigned long long sn_vol(const unsigned long long *p)
+{
+    return *(const volatile unsigned long long *)p;
+}
+__device__ __forceinline__ int sn_vol(const int32_t *p) { return *(const volatile int32_t *)p; }
+
+// Exclusive block scan of v; sh[33].
+__device__ __forceinline__ int sn_block_excl(int v, int *sh, int &total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int inc = sn_warp_incl(v, lane);
+    __syncthreads();
+    if (lane == 31) sh[wid] = inc;
+    __syncthreads();
+    const int wi = sn_warp_incl(lane < nw ? sh[lane] : 0, lane);
+    total = __shfl_sync(SN_FULL, wi, 31);
+    const int before = __shfl_sync(SN_FULL, wi, (wid + 31) & 31);
+    return (wid ? before : 0) + inc - v;
+}
+
+// Exclusive offset of one int per warp; sh[33].
+__device__ __forceinline__ int sn_warp_offset(int v, int *sh, int &total)
+{
+    const int lane = threadIdx.x & 31;
+    const int ex = sn_block_excl(lane == 0 ? v : 0, sh, total);
+    return __shfl_sync(SN_FULL, ex, 0);
+}
+
+// Ranges of queue entries [q0, q1), spread evenly over the block: range(q)
+// gives (first, length) of an entry, body(q, k) is called for each of its
+// elements k.  Few entries hold most elements (hubs), so one warp per entry
+// left most of the block idle.  Ends with a barrier.
+struct ExpandShared {
+    int sh[33];
+    int ex[SN_T];
+    int first[SN_T];
+};
+template <class Range, class Body>
+__device__ __forceinline__ void sn_expand(ExpandShared &S, int q0, int q1, Range range, Body body)
+{
+    const int tid = threadIdx.x, T = blockDim.x;
+    for (int b = q0; b < q1; b += T) {
+        int first = 0, len = 0, total;
+        if (b + tid < q1) range(b + tid, first, len);
+        const int ex = sn_block_excl(len, S.sh, total);
+        S.ex[tid] = ex;
+        S.first[tid] = first;
+        __syncthreads();
+        const int n = min(T, q1 - b);
+        for (int a = tid; a < total; a += T) {
+            int lo = 0, hi = n - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (S.ex[mid] <= a) lo = mid;
+                else hi = mid - 1;
+            }
+            body(b + lo, S.first[lo] + a - S.ex[lo]);
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------- coins to bitmaps
+
+// Live bits of arcs, transposed to one bitmap over the arcs per snapshot,
+// and per (word, node) the snapshots with a live out-arc (oany), a live
+// in-arc (any) and two or more (join).  FROM 0: uniform coins, 1: weighted
+// coins, 2: masks already drawn (lm [W][m]).  Each warp evaluates 32 arcs
+// of one word, 64 coins per lane, and turns the 64 x 32 bits with ballots;
+// rows leave the block 32 bytes at a time.  Bound by the coins' integer
+// arithmetic; they are drawn once for both directions.
+template <int FROM>
+__global__ void __launch_bounds__(SN_TILE) snap_coins_kernel(SnapView v, Coins co, const uint2 *fw,
+                                                             const unsigned long long *lm)
+{
+    __shared__ uint32_t tile[64][SN_TILE / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const long long tiles = (v.m + SN_TILE - 1) / SN_TILE;
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const long long e = t * SN_TILE + tid;
+        const bool in = e < v.m;
+        int y = 0, x = 0;
+        uint32_t tm1 = co.uic_tm1;
+        if (in) {
+            x = __ldg(v.esrc + e);
+            if (FROM == 1) {
+                const uint2 a = __ldg(fw + e);
+                y = (int)a.x;
+                tm1 = a.y;
+            } else {
+                y = __ldg(v.col + e);
+            }
+        }
+        const uint64_t base = co.seed ^ (uint64_t)e;
+        for (int w = 0; w < v.W; ++w) {
+            uint64_t mk = 0;
+            if (in) {
+                if (FROM == 2) {
+                    mk = __ldg(lm + (long long)w * v.m + e);
+                } else if (!co.none_live) {
+                    const int nb = min(64, v.R - 64 * w);
+                    uint32_t lo = 0, hi = 0;
+#pragma unroll 8
+                    for (int b = 0; b < min(32, nb); ++b)
+                        lo |= (uint32_t)(coin_hi32(base, (uint32_t)(64 * w + b)) <= tm1) << b;
+#pragma unroll 8
+                    for (int b = 32; b < nb; ++b)
+                        hi |= (uint32_t)(coin_hi32(base, (uint32_t)(64 * w + b)) <= tm1) << (b - 32);
+                    mk = ((uint64_t)hi << 32) | lo;
+                }
+                if (mk) {
+                    const size_t o = (size_t)w * (size_t)v.n;
+                    atomicOr(&v.oany[o + x], (unsigned long long)mk);
+                    const uint64_t dup = mk & atomicOr(&v.any[o + y], (unsigned long long)mk);
+                    if (dup) atomicOr(&v.join[o + y], (unsigned long long)dup);
+                }
+            }
+            uint32_t r0 = 0, r1 = 0;
+            const uint32_t ml = (uint32_t)mk, mh = (uint32_t)(mk >> 32);
+#pragma unroll
+            for (int b = 0; b < 32; ++b) {
+                const uint32_t b0 = __ballot_sync(SN_FULL, (ml >> b) & 1u), b1 = __ballot_sync(SN_FULL, (mh >> b) & 1u);
+                if (lane == b) {
+                    r0 = b0;
+                    r1 = b1;
+                }
+            }
+            tile[lane][wid] = r0;
+            tile[lane + 32][wid] = r1;
+            __syncthreads();
+            for (int i = tid; i < 64 * (SN_TILE / 32); i += SN_TILE) {
+                const int b = i / (SN_TILE / 32), k = i % (SN_TILE / 32);
+                const int r = 64 * w + b;
+                if (r < v.R) v.lb[(size_t)r * v.m32 + (size_t)t * (SN_TILE / 32) + k] = tile[b][k];
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Node bitmaps per snapshot (internal nodes, joins) from the bit-sliced
+// words, and the part of the initial gains and of their edge count that
+// needs no walk: a node without a live out-arc reaches itself.
+__global__ void __launch_bounds__(SN_TILE) snap_nodes_kernel(SnapView v, Ctl *ctl, long long *s)
+{
+    __shared__ uint32_t to[64][SN_TILE / 32], tj[64][SN_TILE / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tiles = (v.n + SN_TILE - 1) / SN_TILE;
+    unsigned long long ed = 0;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int x = t * SN_TILE + tid;  // t * SN_TILE <= n < 2^31
+        const bool in = x < v.n && x >= 0;
+        long long own = 0;
+        for (int w = 0; w < v.W; ++w) {
+            uint64_t o = 0, j = 0;
+            if (in) {
+                o = v.oany[(size_t)w * (size_t)v.n + x];
+                j = v.join[(size_t)w * (size_t)v.n + x];
+                own += __popcll(sn_word_mask(w, v.R) & ~o);
+            }
+            uint32_t o0 = 0, o1 = 0, j0 = 0, j1 = 0;
+#pragma unroll
+            for (int b = 0; b < 32; ++b) {
+                const uint32_t a0 = __ballot_sync(SN_FULL, (o >> b) & 1ull), a1 = __ballot_sync(SN_FULL, (o >> (b + 32)) & 1ull);
+                const uint32_t c0 = __ballot_sync(SN_FULL, (j >> b) & 1ull), c1 = __ballot_sync(SN_FULL, (j >> (b + 32)) & 1ull);
+                if (lane == b) {
+                    o0 = a0;
+                    o1 = a1;
+                    j0 = c0;
+                    j1 = c1;
+                }
+            }
+            to[lane][wid] = o0;
+            to[lane + 32][wid] = o1;
+            tj[lane][wid] = j0;
+            tj[lane + 32][wid] = j1;
+            __syncthreads();
+            for (int i = tid; i < 64 * (SN_TILE / 32); i += SN_TILE) {
+                const int b = i / (SN_TILE / 32), k = i % (SN_TILE / 32);
+                const int r = 64 * w + b;
+                if (r < v.R) {
+                    const size_t q = (size_t)r * v.n32 + (size_t)t * (SN_TILE / 32) + k;
+                    v.outb[q] = to[b][k];
+                    v.joinb[q] = tj[b][k];
+                }
+            }
+            __syncthreads();
+        }
+        if (in) {
+            s[x] = own;
+            ed += (unsigned long long)own * (unsigned long long)(__ldg(v.rp + x + 1) - __ldg(v.rp + x));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ed += __shfl_xor_sync(SN_FULL, ed, o);
+    if (lane == 0 && ed) atomicAdd(&ctl->init_edges, ed);
+}
+
+// ---------------------------------------------------------- per snapshot
+
+// Set bits of a bitmap: totals per warp chunk of words.  Chunks are
+// contiguous and a multiple of 32 words, so the order is kept.
+__device__ __forceinline__ void sn_chunk(long long words, long long &lo, long long &hi)
+{
+    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long per = ((words + nw - 1) / nw + 31) / 32 * 32;
+    lo = min((long long)wid * per, words);
+    hi = min(lo + per, words);
+}
+
+__device__ __forceinline__ int sn_chunk_count(const uint32_t *b, long long lo, long long hi)
+{
+    const int lane = threadIdx.x & 31;
+    int c = 0;
+    for (long long i = lo + lane; i < hi; i += 32) c += __popc(b[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(SN_FULL, c, o);
+    return c;
+}
+
+// Internal nodes and live arcs of one snapshot, in node and arc order, with
+// the direct counts of every internal node: itself and its leaf children
+// (low half of acc), its arcs to joins (high half), their out-degrees, and
+// the parent of every internal tree node.
+__global__ void __launch_bounds__(SN_T) snap_compact_kernel(SnapView v, Ctl *ctl)
+{
+    __shared__ int sh[33];
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const uint32_t *outb = v.outb + (size_t)r * v.n32, *joinb = v.joinb + (size_t)r * v.n32;
+    const uint32_t *lb = v.lb + (size_t)r * v.m32;
+    int32_t *outp = v.outp + (size_t)r * v.n32;
+    const size_t io = (size_t)r * v.icap;
+    SnapInfo *info = v.info + r;
+    long long lo, hi, alo, ahi;
+    sn_chunk(v.n32, lo, hi);
+    sn_chunk(v.m32, alo, ahi);
+    int nI, L;
+    int off = sn_warp_offset(sn_chunk_count(outb, lo, hi), sh, nI);
+    int aoff = sn_warp_offset(sn_chunk_count(lb, alo, ahi), sh, L);
+    const bool bad = nI > v.icap || L > v.cap;
+    if (tid == 0) {
+        SnapInfo z{};
+        z.nI = bad ? 0 : nI;
+        z.L = bad ? 0 : L;
+        z.bad = bad;
+        *info = z;
+        if (bad) atomicOr(&ctl->flags, FLAG_SNAPSHOT);
+    }
+    for (long long i0 = lo; i0 < hi; i0 += 32) {
+        const long long i = i0 + lane;
+        uint32_t b = i < hi ? outb[i] : 0u;
+        const int c = __popc(b);
+        const int inc = sn_warp_incl(c, lane);
+        int p = off + inc - c;
+        if (i < hi) outp[i] = p;
+        off += __shfl_sync(SN_FULL, inc, 31);
+        while (b && !bad) {
+            const int x = (int)(i * 32) + __ffs(b) - 1;
+            b &= b - 1;
+            v.inode[io + p] = x;
+            v.acc[io + p] = 1ull;
+            v.deg[io + p] = (uint32_t)(__ldg(v.rp + x + 1) - __ldg(v.rp + x));
+            v.par[io + p] = -1;
+            v.pend[io + p] = 1;
+            v.share[io + p] = -1;
+            v.jid[io + p] = -1;
+            v.cv[io + p] = 0;
+            ++p;
+        }
+    }
+    if (bad) return;
+    __syncthreads();
+    // live arcs: 32 words (1024 arcs) per warp step, spread over the lanes
+    int2 *arc = v.arc + (size_t)r * v.cap;
+    for (long long i0 = alo; i0 < ahi; i0 += 32) {
+        const long long i = i0 + lane;
+        const uint32_t b = i < ahi ? lb[i] : 0u;
+        const int c = __popc(b);
+        const int inc = sn_warp_incl(c, lane);
+        const int total = __shfl_sync(SN_FULL, inc, 31), ex = inc - c;
+        for (int j0 = 0; j0 < total; j0 += 32) {
+            const int j = j0 + lane;
+            int k = 0;
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1)
+                if (__shfl_sync(SN_FULL, ex, k + step) <= j) k += step;  // k + step <= 31
+            const uint32_t wb = __shfl_sync(SN_FULL, b, k);
+            const int wex = __shfl_sync(SN_FULL, ex, k);
+            if (j < total) {
+                const long long e = (i0 + k) * 32 + sn_nth_bit(wb, j - wex);
+                const int y = __ldg(v.col + e);
+                const int x = __ldg(v.esrc + e);
+                const int xi = sn_rank(outb, outp, x);
+                arc[aoff + j] = make_int2(xi, y);
+                if (sn_bit(joinb, y)) {
+                    atomicAdd(&v.acc[io + xi], 1ull << 32);
+                } else if (sn_bit(outb, y)) {
+                    v.par[io + sn_rank(outb, outp, y)] = xi;
+                } else {
+                    atomicAdd(&v.acc[io + xi], 1ull);
+                    atomicAdd(&v.deg[io + xi], (uint32_t)(__ldg(v.rp + y + 1) - __ldg(v.rp + y)));
+                }
+            }
+        }
+        aoff += total;
+    }
+}
+
+// Trees of one snapshot: cycles of one-parent nodes are cut at their lowest
+// node (which becomes a join), subtree totals are summed towards the roots,
+// and every node gets its absolute positions in the join-arc and node lists.
+__global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
+{
+    __shared__ int sh[33];
+    __shared__ int changed, ncut;
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
+    SnapInfo *info = v.info + r;
+    if (info->bad) return;
+    const int nI = info->nI;
+    const size_t io = (size_t)r * v.icap;
+    const int32_t *inode = v.inode + io;
+    int32_t *par = v.par + io, *pend = v.pend + io, *share = v.share + io;
+    unsigned long long *acc = v.acc + io, *pj = v.pj + io, *pn = v.pn + io;
+    uint32_t *deg = v.deg + io;
+    uint32_t *joinb = v.joinb + (size_t)r * v.n32;
+    int32_t *cut = v.jin + (size_t)r * v.cap;  // scratch here
+    // Pointer doubling: pj = (an ancestor, lowest index on the path up to
+    // it).  A round without a change leaves exactly the nodes above which
+    // lies a cycle unrooted, each with the cycle's lowest index.
+    for (int i = tid; i < nI; i += T) pj[i] = sn_pack(par[i] >= 0 ? par[i] : i, (uint32_t)i);
+    if (tid == 0) ncut = 0;
+    int rounds = 0;
+    while (true) {
+        __syncthreads();
+        if (tid == 0) changed = 0;
+        __syncthreads();
+        for (int i = tid; i < nI; i += T) {
+            if (par[i] < 0) continue;
+            const unsigned long long w = pj[i];
+            const int p = sn_hi(w);
+            if (par[p] < 0) continue;  // rooted
+            const unsigned long long q = sn_vol(pj + p);
+            const uint32_t mn = min(sn_lo(w), sn_lo(q));
+            *(volatile unsigned long long *)(pj + i) = sn_pack(sn_hi(q), mn);
+            if (mn != sn_lo(w) || par[sn_hi(q)] < 0) changed = 1;
+        }
+        __syncthreads();
+        if (!changed) break;
+        if (++rounds > 64) {
+            if (tid == 0) atomicOr(&ctl->flags, FLAG_SNAPSHOT);
+            break;
+        }
+    }
+    for (int i = tid; i < nI; i += T) {
+        if (par[i] < 0) continue;
+        const int p = sn_hi(pj[i]);
+        if (par[p] < 0) continue;
+        const int c = (int)sn_lo(pj[p]);
+        const int x = inode[c];
+        const uint32_t bit = 1u << (x & 31);
+        if (!(atomicOr(&joinb[x >> 5], bit) & bit)) cut[atomicAdd(&ncut, 1)] = c;
+    }
+    __syncthreads();
+    for (int k = tid; k < ncut; k += T) {
+        const int c = cut[k];
+        atomicAdd(&acc[par[c]], 1ull << 32);  // its in-arc leads to a join now
+    }
+    __syncthreads();
+    for (int k = tid; k < ncut; k += T) par[cut[k]] = -1;
+    __syncthreads();
+    for (int i = tid; i < nI; i += T)
+        if (par[i] >= 0) atomicAdd(&pend[par[i]], 1);
+    __syncthreads();
+    // Subtree sums: the last of a node's own thread and its children's
+    // carries on upwards; what the parent had before is the child's offset.
+    for (int i = tid; i < nI; i += T) {
+        int c = i;
+        while (atomicSub(&pend[c], 1) == 1) {
+            const int p = par[c];
+            if (p < 0) break;
+            __threadfence_block();
+            const unsigned long long a = sn_vol(acc + c);
+            const uint32_t d = *(volatile uint32_t *)(deg + c);
+            const unsigned long long old = atomicAdd(&acc[p], a);
+            pj[c] = sn_pack(p, (uint32_t)sn_hi(old));
+            pn[c] = sn_pack(p, sn_lo(old));
+            atomicAdd(&deg[p], d);
+            __threadfence_block();
+            c = p;
+        }
+    }
+    __syncthreads();
+    // roots in index order
+    {
+        const int nw = T >> 5, per = ((nI + nw - 1) / nw + 31) / 32 * 32;
+        const int lo = min(wid * per, nI), hi = min(lo + per, nI);
+        int cj = 0, cn = 0;
+        for (int i = lo + lane; i < hi; i += 32)
+            if (par[i] < 0) {
+                cj += sn_hi(acc[i]);
+                cn += (int)sn_lo(acc[i]);
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            cj += __shfl_xor_sync(SN_FULL, cj, o);
+            cn += __shfl_xor_sync(SN_FULL, cn, o);
+        }
+        int JA, N;
+        int oj = sn_warp_offset(cj, sh, JA), on = sn_warp_offset(cn, sh, N);
+        for (int i0 = lo; i0 < hi; i0 += 32) {
+            const int i = i0 + lane;
+            const bool root = i < hi && par[i] < 0;
+            const int a = root ? sn_hi(acc[i]) : 0, b = root ? (int)sn_lo(acc[i]) : 0;
+            const int ia = sn_warp_incl(a, lane), ib = sn_warp_incl(b, lane);
+            if (root) {
+                pj[i] = sn_pack(~i, (uint32_t)(oj + ia - a));
+                pn[i] = sn_pack(~i, (uint32_t)(on + ib - b));
+            }
+            oj += __shfl_sync(SN_FULL, ia, 31);
+            on += __shfl_sync(SN_FULL, ib, 31);
+        }
+        if (tid == 0) info->JA = JA;
+    }
+    // absolute positions: (ancestor or ~root, offset below it)
+    rounds = 0;
+    while (true) {
+        __syncthreads();
+        if (tid == 0) changed = 0;
+        __syncthreads();
+        for (int i = tid; i < nI; i += T) {
+            const unsigned long long a = pj[i], b = pn[i];
+            if (sn_hi(a) >= 0) {
+                const unsigned long long q = sn_vol(pj + sn_hi(a));
+                *(volatile unsigned long long *)(pj + i) = sn_pack(sn_hi(q), sn_lo(a) + sn_lo(q));
+                changed = 1;
+            }
+            if (sn_hi(b) >= 0) {
+                const unsigned long long q = sn_vol(pn + sn_hi(b));
+                *(volatile unsigned long long *)(pn + i) = sn_pack(sn_hi(q), sn_lo(b) + sn_lo(q));
+                changed = 1;
+            }
+        }
+        __syncthreads();
+        if (!changed) break;
+        if (++rounds > 64) {
+            if (tid == 0) atomicOr(&ctl->flags, FLAG_SNAPSHOT);
+            break;
+        }
+    }
+    // a child with its parent's whole range shares the parent's closure
+    for (int i = tid; i < nI; i += T) {
+        const int p = par[i], sj = sn_hi(acc[i]);
+        if (p >= 0 && sj > 0 && sj == sn_hi(acc[p])) share[p] = i;
+    }
+    // joins in node order
+    int32_t *joinp = v.joinp + (size_t)r * v.n32;
+    long long lo, hi;
+    sn_chunk(v.n32, lo, hi);
+    int C;
+    int off = sn_warp_offset(sn_chunk_count(joinb, lo, hi), sh, C);
+    if (tid == 0) info->C = C;
+    for (long long i0 = lo; i0 < hi; i0 += 32) {
+        const long long i = i0 + lane;
+        uint32_t b = i < hi ? joinb[i] : 0u;
+        const int c = __popc(b);
+        const int inc = sn_warp_incl(c, lane);
+        int p = off + inc - c;
+        if (i < hi) joinp[i] = p;
+        off += __shfl_sync(SN_FULL, inc, 31);
+        while (b) {
+            v.jnode[(size_t)r * v.jcap + p] = (int)(i * 32) + __ffs(b) - 1;
+            b &= b - 1;
+            ++p;
+        }
+    }
+}
+
+// The chunks of tasks of every snapshot's two task segments, in order, and
+// the most bits a walk needs (one block; cnt(r, seg) gives the lengths,
+// ids(r) the bits).  A chunk is WK_CH tasks, fewer when there would not be
+// several chunks for each walking warp.
+template <class F, class G>
+__device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, F cnt, G ids)
+{
+    const int tid = threadIdx.x, T = blockDim.x;
+    __shared__ int most;
+    __shared__ unsigned long long all;
+    if (tid == 0) {
+        most = 0;
+        all = 0;
+    }
+    __syncthreads();
+    for (int r = tid; r < v.R; r += T) {
+        const int c = cnt(r, 0) + cnt(r, 1);
+        if (c > 0) {
+            atomicAdd(&all, (unsigned long long)c);
+            atomicMax(&most, ids(r));
+        }
+    }
+    __syncthreads();
+    const int ch = (int)max(1ull, min((unsigned long long)WK_CH, all / (unsigned long long)(8 * v.wwarps)));
+    int carry = 0;
+    for (int base = 0; base < 2 * v.R; base += T) {
+        const int q = base + tid;
+        int total;
+        const int ex = sn_block_excl(q < 2 * v.R ? (cnt(q >> 1, q & 1) + ch - 1) / ch : 0, sh, total);
+        if (q < 2 * v.R) v.cstart[q] = carry + ex;
+        carry += total;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        v.cstart[2 * v.R] = carry;
+        v.cstart[2 * v.R + 1] = most;
+        v.cstart[2 * v.R + 2] = ch;
+        *v.cnext = 0;
+    }
+}
+
+// Join-arc, join in-arc and node lists and join records of one snapshot,
+// then its landmark: a join x with many arcs below it and
+// many above.  Every node that reaches x reaches all of R(x), so those
+// walks start from a copy of R(x)'s bits and total.
+__global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
+{
+    __shared__ ExpandShared S;
+    __shared__ int tail;
+    __shared__ unsigned long long best;
+    __shared__ unsigned int lc, ld;
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
+    SnapInfo *info = v.info + r;
+    const int nI = info->nI, L = info->L, C = info->C;
+    const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap, ao = (size_t)r * v.cap;
+    const uint32_t *outb = v.outb + (size_t)r * v.n32, *joinb = v.joinb + (size_t)r * v.n32;
+    const int32_t *outp = v.outp + (size_t)r * v.n32, *joinp = v.joinp + (size_t)r * v.n32;
+    const unsigned long long *acc = v.acc + io, *pj = v.pj + io, *pn = v.pn + io;
+    unsigned long long *fill = v.cv + io;
+    int32_t *inoff = v.inoff + (size_t)r * (v.jcap + 1);
+    uint32_t *jarc = v.jarc + ao;
+    int32_t *jin = v.jin + ao, *tn = v.tn + (size_t)r * v.tcap;
+    int4 *rec = v.rec + jo;
+    for (int c = tid; c <= C; c += T) inoff[c] = 0;
+    if (tid == 0) {
+        best = 0;
+        lc = 0;
+        ld = 0;
+        tail = 0;
+    }
+    for (int i = tid; i < nI; i += T) tn[sn_lo(pn[i])] = v.inode[io + i];
+    __syncthreads();
+    for (int j = tid; j < L; j += T) {
+        const int2 a = v.arc[ao + j];
+        const bool out = sn_bit(outb, a.y);
+        if (sn_bit(joinb, a.y)) {
+            const int c = sn_rank(joinb, joinp, a.y);
+            const int k = sn_hi(atomicAdd(&fill[a.x], 1ull << 32));
+            jarc[sn_lo(pj[a.x]) + k] = (uint32_t)c | (out ? 0u : ARC_LEAF);
+            atomicAdd(&inoff[c + 1], 1);
+        } else if (!out) {
+            const int k = (int)sn_lo(atomicAdd(&fill[a.x], 1ull));
+            tn[sn_lo(pn[a.x]) + 1 + k] = a.y;
+        }
+    }
+    __syncthreads();
+    // inoff[c + 1] = in-arcs of join c -> its start (shifted by one: the
+    // fill below moves each to the join's end, the next one's start)
+    {
+        const int nw = T >> 5, per = ((C + nw - 1) / nw + 31) / 32 * 32;
+        const int lo = min(wid * per, C), hi = min(lo + per, C);
+        int s = 0, all;
+        for (int c = lo + lane; c < hi; c += 32) s += inoff[c + 1];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(SN_FULL, s, o);
+        int off = sn_warp_offset(s, S.sh, all);
+        for (int c0 = lo; c0 < hi; c0 += 32) {
+            const int c = c0 + lane;
+            const int x = c < hi ? inoff[c + 1] : 0;
+            const int inc = sn_warp_incl(x, lane);
+            if (c < hi) inoff[c + 1] = off + inc - x;
+            off += __shfl_sync(SN_FULL, inc, 31);
+        }
+    }
+    for (int c = tid; c < C; c += T) {
+        const int y = v.jnode[jo + c];
+        if (sn_bit(outb, y)) {
+            const int i = sn_rank(outb, outp, y);
+            v.jint[jo + c] = i;
+            v.jid[io + i] = c;
+            rec[c] = make_int4((int)sn_lo(acc[i]), (int)v.deg[io + i], (int)sn_lo(pj[i]), sn_hi(acc[i]));
+        } else {
+            v.jint[jo + c] = -1;
+            rec[c] = make_int4(1, __ldg(v.rp + y + 1) - __ldg(v.rp + y), 0, 0);
+        }
+    }
+    __syncthreads();
+    for (int j = tid; j < L; j += T) {
+        const int2 a = v.arc[ao + j];
+        if (sn_bit(joinb, a.y)) jin[atomicAdd(&inoff[sn_rank(joinb, joinp, a.y) + 1], 1)] = a.x;
+    }
+    __syncthreads();
+    // landmark: join arcs below times in-arcs up to two steps above
+    for (int c = tid; c < C; c += T) {
+        const int w = rec[c].w;
+        if (w < 2) continue;
+        unsigned long long up = 0;
+        for (int k = inoff[c]; k < inoff[c + 1]; ++k) {
+            const int j = v.jid[io + ~sn_hi(pj[jin[k]])];
+            up += 1ull + (j >= 0 ? (unsigned long long)(inoff[j + 1] - inoff[j]) : 0ull);
+        }
+        const unsigned long long sc = min(up * (unsigned long long)w, (1ull << 31) - 1ull);
+        atomicMax(&best, (sc << 32) | (uint32_t)c);
+    }
+    __syncthreads();
+    const int x = best ? (int)(uint32_t)best : -1;
+    const int cw = (C + 31) >> 5, iw = (nI + 31) >> 5;
+    uint32_t *lr = v.lmr + (size_t)r * v.jw, *lu = v.marki + (size_t)r * v.iw;
+    int32_t *ql = v.jlist + jo, *qi = v.ilist + io;
+    for (int i = tid; i < cw; i += T) lr[i] = 0;
+    for (int i = tid; i < iw; i += T) lu[i] = 0;
+    __syncthreads();
+    if (x >= 0) {
+        if (tid == 0) {
+            lr[x >> 5] = 1u << (x & 31);
+            ql[0] = x;
+            tail = 1;
+        }
+        __syncthreads();
+        for (int h = 0;;) {  // R(x): joins
+            const int t = tail;
+            __syncthreads();
+            if (h >= t) break;
+            sn_expand(
+                S, h, t,
+                [&](int q, int &first, int &len) {
+                    const int4 e = rec[ql[q]];
+                    atomicAdd(&lc, (unsigned)e.x);
+                    atomicAdd(&ld, (unsigned)e.y);
+                    first = e.z;
+                    len = e.w;
+                },
+                [&](int, int k) {
+                    const int j = (int)(jarc[k] & ~ARC_LEAF);
+                    const uint32_t bit = 1u << (j & 31);
+                    if (!(atomicOr(&lr[j >> 5], bit) & bit)) ql[atomicAdd(&tail, 1)] = j;
+                });
+            h = t;
+        }
+        __syncthreads();
+        if (tid == 0) tail = 0;
+        __syncthreads();
+        // U(x): internal nodes that reach x
+        auto mark = [&](int i) {
+            const uint32_t bit = 1u << (i & 31);
+            if (!(atomicOr(&lu[i >> 5], bit) & bit)) qi[atomicAdd(&tail, 1)] = i;
+        };
+        for (int k = inoff[x] + tid; k < inoff[x + 1]; k += T) mark(jin[k]);
+        __syncthreads();
+        for (int h = 0;;) {
+            const int t = tail;
+            __syncthreads();
+            if (h >= t) break;
+            sn_expand(
+                S, h, t,
+                [&](int q, int &first, int &len) {
+                    const int i = qi[q];
+                    const int p = v.par[io + i], j = v.jid[io + i];
+                    if (p >= 0) {
+                        mark(p);
+                    } else if (j >= 0) {
+                        first = inoff[j];
+                        len = inoff[j + 1] - first;
+                    }
+                },
+                [&](int, int k) { mark(jin[k]); });
+            h = t;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        info->lmk_cnt = (int)lc;
+        info->lmk_deg = (int)ld;
+    }
+}
+
+// ------------------------------------------------------------- the walks
+
+// One thread's closure walk, for the many ranges that reach only a few
+// joins (on R-MAT 20 three in four): the visited joins are a short list,
+// looked through only when a 64-bit filter says that one may be there.
+// skip: joins left out (NULL: none).  REL: only joins in rel are entered, and
+// only covered ones (covj) count.  Returns false, with the totals
+// meaningless, when the walk is too large; n: visited joins.
+template <bool REL, bool EDGES>
+__device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uint32_t *jarc, const int4 *rec,
+                                           const uint32_t *skip, const uint32_t *rel, const uint32_t *covj, int pos,
+                                           int wd, unsigned int &cnt, unsigned int &deg, int &n)
+{
+    n = 0;
+    int h = 0, p = pos, e = pos + wd, scanned = 0;
+    unsigned long long seen = 0;
+    if (wd > SW_ARCS) return false;
+    while (true) {
+        if (p < e) {
+            const uint32_t a = jarc[p++];
+            const int j = (int)(a & ~ARC_LEAF);
+            if (REL && !sn_bit(rel, j)) continue;
+            if (skip && sn_bit(skip, j)) continue;
+            const unsigned long long f = 1ull << (((uint32_t)j * 2654435761u) >> 26);
+            if (seen & f) {
+                bool found = false;
+                for (int k = 0; k < n; ++k) found |= list[k * stride] == a;
+                if (found) continue;
+            }
+            if (n == SW_CAP) return false;
+            seen |= f;
+            list[n * stride] = a;
+            ++n;
+            if (a & ARC_LEAF) {
+                cnt += 1u;
+                if (EDGES) deg += (unsigned)rec[j].y;
+            }
+        } else {
+            while (h < n && (list[h * stride] & ARC_LEAF)) ++h;
+            if (h == n) return true;
+            const int j = (int)list[h * stride];
+            ++h;
+            const int4 r = rec[j];
+            if (!REL || sn_bit(covj, j)) cnt += (unsigned)r.x;
+            if (EDGES) deg += (unsigned)r.y;
+            scanned += r.w;
+            if (scanned > SW_ARCS) return false;
+            p = r.z;
+            e = p + r.w;
+        }
+    }
+}
+
+// The initial gains' ranges by one thread each; those that are too large go
+// to the task lists of the warp walks (in place of all tasks).
+template <bool EDGES>
+__global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
+{
+    __shared__ uint32_t list[SW_CAP][256];
+    __shared__ int sh[33];
+    __shared__ int last;
+    const int tid = threadIdx.x;
+    const int per = gridDim.x / v.R > 0 ? gridDim.x / v.R : 1;  // blocks per snapshot
+    for (int b = blockIdx.x; b < per * v.R; b += gridDim.x) {
+        const int r = b / per, part = b - r * per;
+        SnapInfo *info = v.info + r;
+        const int nI = info->nI;
+        const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
+        const uint32_t *lu = v.marki + (size_t)r * v.iw, *lmr = v.lmr + (size_t)r * v.jw;
+        for (int i = part * 256 + tid; i < nI; i += per * 256) {
+            const int wd = sn_hi(v.acc[io + i]);
+            if (wd < 2 || v.share[io + i] >= 0) continue;
+            const unsigned long long pj = v.pj[io + i];
+            const bool l = sn_bit(lu, i);
+            unsigned int c = l ? (unsigned)info->lmk_cnt : 0u, d = l ? (unsigned)info->lmk_deg : 0u;
+            int n;
+            if (small_walk<false, EDGES>(&list[0][tid], 256, v.jarc + (size_t)r * v.cap, v.rec + jo, l ? lmr : nullptr,
+                                         nullptr, nullptr, (int)sn_lo(pj), wd, c, d, n)) {
+                const int rj = v.jid[io + ~sn_hi(pj)];
+                bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
+                for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
+                v.cv[io + i] = sn_pack((int)(c | (cyc ? CV_CYCLE : 0u)), d);
+            } else if (l) {
+                v.task[io + v.icap - 1 - atomicAdd(&info->t1, 1)] = i;
+            } else {
+                v.task[io + atomicAdd(&info->t0, 1)] = i;
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(v.arrive, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sn_plan(v, sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); },
+            [&](int q) { return sn_vol(&v.info[q].C); });
+    if (tid == 0) *v.arrive = 0;
+}
+
+// One warp's closure walk over join ids.  A join found for the first time
+// adds its totals and, with join arcs of its own, is queued.  Each lane
+// keeps WK_U arcs in flight: the walk is a chain of dependent loads from
+// L2 (arc, record), so loads in flight set its rate.  The queue's first
+// entries lie in shared memory; entries past its end are dropped and the
+// walk then re-expands every join it visited (which changes nothing for
+// those already expanded) until no entry was dropped.
+//   REL false  ids are join ids, vis one bit per join, rec their records
+//   REL true   a round: only the relevant joins (rel: bitmap word and set
+//              bits before it) are entered, under their rank among them; vis
+//              and rec (weight, first arc, arcs) are by that rank, so a late
+//              round's few relevant joins take a few words per warp
+template <bool REL>
+struct Walk {
+    uint32_t *vis;
+    int32_t *qs, *ts;    // shared queue and undo list
+    int32_t *qg;         // global queue
+    const uint32_t *jarc;
+    const int4 *rec;
+    const uint2 *rel;    // REL
+    int count;           // ids
+    int qt, nt, na;      // queued, visited, arcs scanned
+    bool lost;
+    unsigned int cnt, deg;
+
+    __device__ __forceinline__ static int first_of(const int4 &e) { return REL ? e.y : e.z; }
+    __device__ __forceinline__ static int arcs_of(const int4 &e) { return REL ? e.z : e.w; }
+
+    // arcs a[u] of this lane, valid where act[u]
+    template <bool EDGES, int U>
+    __device__ __forceinline__ void arcs(const uint32_t (&a)[U], const bool (&act)[U], int lane)
+    {
+        int id[U];
+        bool fresh[U], push[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            id[u] = (int)(a[u] & ~ARC_LEAF);
+            fresh[u] = act[u];
+            if (REL && fresh[u]) {
+                const uint2 w = rel[id[u] >> 5];
+                const uint32_t bit = 1u << (id[u] & 31);
+                fresh[u] = (w.x & bit) != 0;
+                id[u] = (int)w.y + __popc(w.x & (bit - 1u));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (fresh[u]) {
+                const uint32_t bit = 1u << (id[u] & 31);
+                fresh[u] = !(atomicOr(&vis[id[u] >> 5], bit) & bit);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            push[u] = false;
+            if (!fresh[u]) continue;
+            if (!EDGES && (a[u] & ARC_LEAF)) {
+                cnt += 1u;
+            } else {
+                const int4 e = rec[id[u]];
+                cnt += (unsigned)e.x;
+                if (EDGES) deg += (unsigned)e.y;
+                push[u] = arcs_of(e) > 0;
+            }
+        }
+        const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned bf = __ballot_sync(SN_FULL, fresh[u]);
+            if (!bf) continue;
+            if (fresh[u]) {
+                const int p = nt + __popc(bf & lt);
+                if (p < WK_TS) ts[p] = id[u];
+            }
+            nt += __popc(bf);
+            const unsigned bp = __ballot_sync(SN_FULL, push[u]);
+            if (push[u]) {
+                const int p = qt + __popc(bp & lt);
+                if (p < WK_QS) qs[p] = id[u];
+                else if (p < WK_QS + WK_QG) qg[p - WK_QS] = id[u];
+            }
+            qt += __popc(bp);
+        }
+        if (qt > WK_QS + WK_QG) {
+            qt = WK_QS + WK_QG;
+            lost = true;
+        }
+    }
+
+    // arcs a0 + 32u + lane of the batch of ranges (pos, ex) the lanes hold
+    template <bool EDGES, int U>
+    __device__ __forceinline__ void spread(int a0, int total, int pos, int ex, int lane)
+    {
+        uint32_t a[U];
+        bool act[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = a0 + 32 * u + lane;
+            int k = 0;
+            if (U == 1 || a0 + 32 * u < total) {  // the same for the whole warp
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1)
+                    if (__shfl_sync(SN_FULL, ex, k + step) <= t) k += step;
+                const int kp = __shfl_sync(SN_FULL, pos, k), kx = __shfl_sync(SN_FULL, ex, k);
+                k = kp + t - kx;
+            }
+            act[u] = t < total;
+            a[u] = act[u] ? jarc[k] : 0u;
+        }
+        arcs<EDGES, U>(a, act, lane);
+    }
+
+    template <bool EDGES, int U>
+    __device__ __forceinline__ void straight(int pos, int left, int lane)
+    {
+        uint32_t a[U];
+        bool act[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            act[u] = 32 * u + lane < left;
+            a[u] = act[u] ? jarc[pos + 32 * u + lane] : 0u;
+        }
+        arcs<EDGES, U>(a, act, lane);
+    }
+
+    template <bool EDGES>
+    __device__ __forceinline__ void queue(int lane)
+    {
+        int qh = 0;
+        __syncwarp();
+        while (qh < qt) {
+            const int nb = min(32, qt - qh);
+            int pos = 0, wd = 0;
+            if (lane < nb) {
+                const int p = qh + lane;
+                const int4 e = rec[p < WK_QS ? qs[p] : qg[p - WK_QS]];
+                pos = first_of(e);
+                wd = arcs_of(e);
+            }
+            qh += nb;
+            const int inc = sn_warp_incl(wd, lane);
+            const int total = __shfl_sync(SN_FULL, inc, 31), ex = inc - wd;
+            na += total;
+            if (qh == qt && qt > WK_QS) {  // drained: start over at the front
+                __syncwarp();
+                qh = 0;
+                qt = 0;
+            }
+            for (int a0 = 0; a0 < total;) {
+                if (total - a0 > 32) {
+                    spread<EDGES, WK_U>(a0, total, pos, ex, lane);
+                    a0 += 32 * WK_U;
+                } else {
+                    spread<EDGES, 1>(a0, total, pos, ex, lane);
+                    a0 += 32;
+                }
+            }
+            __syncwarp();
+        }
+        qt = 0;
+    }
+
+    // Closure of the join-arc range [pos, pos + wd); base: bits set in vis
+    // before the walk (NULL: none).
+    template <bool EDGES>
+    __device__ __forceinline__ void range(int pos, int wd, const uint32_t *base, int lane)
+    {
+        qt = 0;
+        nt = 0;
+        na = wd;
+        lost = false;
+        cnt = 0;
+        deg = 0;
+        for (int a0 = 0; a0 < wd;) {
+            if (wd - a0 > 32) {
+                straight<EDGES, WK_U>(pos + a0, wd - a0, lane);
+                a0 += 32 * WK_U;
+            } else {
+                straight<EDGES, 1>(pos + a0, wd - a0, lane);
+                a0 += 32;
+            }
+        }
+        queue<EDGES>(lane);
+        while (lost) {
+            lost = false;
+            const int words = (count + 31) >> 5;
+            for (int i = 0; i < words; ++i) {
+                const uint32_t b = *(volatile uint32_t *)&vis[i] & ~(base ? base[i] : 0u);
+                const int j = i * 32 + lane;
+                const bool act = ((b >> lane) & 1u) && j < count && arcs_of(rec[j]) > 0;
+                const unsigned bp = __ballot_sync(SN_FULL, act);
+                if (!bp) continue;
+                if (act) qs[__popc(bp & ((1u << lane) - 1u))] = j;  // at most 32 <= WK_QS
+                qt = __popc(bp);
+                queue<EDGES>(lane);
+            }
+        }
+    }
+
+    // vis back to the base
+    __device__ __forceinline__ void undo(const uint32_t *base, int lane)
+    {
+        __syncwarp();
+        if (nt <= WK_TS) {
+            for (int t = lane; t < nt; t += 32) atomicAnd(&vis[ts[t] >> 5], ~(1u << (ts[t] & 31)));
+            __syncwarp();
+        } else {
+            load(base, lane);
+        }
+    }
+
+    __device__ __forceinline__ void load(const uint32_t *base, int lane)
+    {
+        const int words = (count + 31) >> 5;
+        // vis areas and bases are 16-byte aligned and padded to 16 bytes
+        int4 *d = reinterpret_cast<int4 *>(vis);
+        const int4 *b = reinterpret_cast<const int4 *>(base);
+#pragma unroll 4
+        for (int i = lane; i < (words + 3) >> 2; i += 32) d[i] = base ? b[i] : make_int4(0, 0, 0, 0);
+        __syncwarp();
+    }
+};
+
+// Internal node i and the tree ancestors that share its range lose c;
+// returns the reverse edges.
+__device__ __forceinline__ unsigned long long snap_lose(const SnapView &v, long long *s, size_t io, int i,
+                                                        unsigned int c)
+{
+    unsigned long long edges = 0;
+    for (int u = i;;) {
+        const int x = v.inode[io + u];
+        v.cnt[io + u] -= c;
+        atomicAdd((unsigned long long *)&s[x], (unsigned long long)(-(long long)c));
+        edges += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + x + 1) - __ldg(v.crp + x));
+        const int p = v.par[io + u];
+        if (p < 0 || v.share[io + p] != u) return edges;
+        u = p;
+    }
+}
+
+__device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t)
+{
+    int lo = 0, hi = count - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (start[mid] <= t) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// MODE 0: initial gains, the distinct ranges (result kept in cv).
+// MODE 1: initial gains, sources whose count needs their own walk.
+// MODE 2: a round's marked ranges: the newly covered nodes each reaches,
+//         subtracted from it and from the tree ancestors that share its range.
+// EDGES: also the out-degree sums (MODE 0 and 1).
+// Warps claim chunks of tasks in snapshot order, so the graphs of the few
+// snapshots in flight stay in L2.  (Chunks claimed per block, with a barrier
+// after each, left warps waiting for the block's longest walk 40 % of the
+// time.)  Each warp keeps its bits in shared memory (in global memory, one
+// warp per block, when they are more than that holds) and undoes a small
+// walk's bits one by one instead of clearing all.
+template <int MODE, bool EDGES>
+__global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl, long long *s, int smem_bytes)
+{
+    constexpr bool REL = MODE == 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int total = v.cstart[2 * v.R], most = v.cstart[2 * v.R + 1], per = v.cstart[2 * v.R + 2];
+    Walk<REL> w;
+    const int area = ((((most + 31) >> 5) * 4 + 15) & ~15) + (WK_QS + WK_TS) * 4;
+    const int nact = smem_bytes / area;
+    if (wid >= max(1, nact)) return;
+    w.qs = reinterpret_cast<int32_t *>(smem_raw + (size_t)wid * (nact ? area : 0));
+    w.ts = w.qs + WK_QS;
+    w.vis = nact ? reinterpret_cast<uint32_t *>(w.ts + WK_TS) : v.gbm + (size_t)blockIdx.x * v.jw;
+    w.qg = v.wq + ((size_t)blockIdx.x * WK_W + wid) * WK_QG;
+    int q = -1, qbeg = 0, qend = 0;  // (snapshot, segment) at hand: its base is in vis
+    int cnt = 0, lcnt = 0, ldeg = 0;
+    size_t io = 0;
+    const uint32_t *base = nullptr;
+    const int32_t *list = nullptr;
+    unsigned long long edges = 0, arcs = 0, joins = 0;
+    while (true) {
+        int ch = 0;
+        if (lane == 0) ch = atomicAdd(v.cnext, 1);
+        ch = __shfl_sync(SN_FULL, ch, 0);
+        if (ch >= total) break;
+        if (ch >= qend) {
+            q = find_chunk(v.cstart, 2 * v.R, ch);
+            qbeg = v.cstart[q];
+            qend = v.cstart[q + 1];
+            const int r = q >> 1, seg = q & 1;
+            const SnapInfo *in = v.info + r;
+            cnt = MODE == 1 ? (seg ? in->f1 : in->f0) : (seg ? in->t1 : in->t0);
+            lcnt = seg ? in->lmk_cnt : 0;
+            ldeg = seg ? in->lmk_deg : 0;
+            io = (size_t)r * v.icap;
+            w.count = REL ? in->nrel : in->C;
+            w.jarc = v.jarc + (size_t)r * v.cap;
+            w.rec = (REL ? v.rrec : v.rec) + (size_t)r * v.jcap;
+            w.rel = v.rel2 + (size_t)r * v.jw;
+            base = seg ? v.lmr + (size_t)r * v.jw : nullptr;
+            list = (MODE == 1 ? v.fb : v.task) + io;
+            w.load(base, lane);
+        }
+        const int k0 = (ch - qbeg) * per, nk = min(cnt - k0, per);
+        int ti = 0, tp = 0, tw = 0, tr = 0;  // the chunk's tasks, one per lane
+        if (lane < nk) {
+            ti = list[(q & 1) ? v.icap - 1 - (k0 + lane) : k0 + lane];
+            const unsigned long long pj = v.pj[io + ti];
+            tp = (int)sn_lo(pj);
+            tw = sn_hi(v.acc[io + ti]);
+            if (!REL) tr = v.jid[io + ~sn_hi(pj)];
+        }
+        for (int k = 0; k < nk; ++k) {
+            const int i = __shfl_sync(SN_FULL, ti, k), rj = __shfl_sync(SN_FULL, tr, k);
+            w.template range<EDGES>(__shfl_sync(SN_FULL, tp, k), __shfl_sync(SN_FULL, tw, k), base, lane);
+            unsigned int c = w.cnt, d = w.deg;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                c += __shfl_xor_sync(SN_FULL, c, o);
+                if (EDGES) d += __shfl_xor_sync(SN_FULL, d, o);
+            }
+            if (lane == 0) {
+                c += (unsigned)lcnt;
+                d += (unsigned)ldeg;
+                if (MODE != 2) {
+                    const bool cyc = rj >= 0 && (*(volatile uint32_t *)&w.vis[rj >> 5] >> (rj & 31) & 1u);
+                    if (MODE == 0) {
+                        v.cv[io + i] = sn_pack((int)(c | (cyc ? CV_CYCLE : 0u)), d);
+                    } else {
+                        if (!cyc) {
+                            c += sn_lo(v.acc[io + i]);
+                            d += v.deg[io + i];
+                        }
+                        v.cnt[io + i] = c;
+                        atomicAdd((unsigned long long *)&s[v.inode[io + i]], (unsigned long long)c);
+                        edges += d;
+                    }
+                } else {
+                    edges += snap_lose(v, s, io, i, c);
+                }
+            }
+            arcs += (unsigned long long)w.na;
+            joins += (unsigned long long)w.nt;
+            w.undo(base, lane);
+        }
+    }
+    if (lane == 0 && edges) atomicAdd(MODE == 2 ? &ctl->rev_edges : &ctl->init_edges, edges);
+    if (lane == 0 && arcs) {
+        atomicAdd(&ctl->work_elems[MODE == 2 ? 1 : 0][MODE == 0 ? 0 : 2], arcs);
+        atomicAdd(&ctl->work_keys[MODE == 2 ? 1 : 0][MODE == 0 ? 0 : 2], joins);
+    }
+}
+
+// Counts of all internal nodes from the walked ranges.  A node's closure is
+// that of the lowest tree node with the same range; a range of one join arc
+// is followed to the join's own closure.  Where that closure runs through a
+// cycle (so that it might hold the node's own tree) the node gets a walk of
+// its own, by this thread or, when too large, by a warp (list fb, planned
+// for MODE 1 by the last block).
+template <bool EDGES>
+__global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl, long long *s)
+{
+    __shared__ uint32_t list[SW_CAP][256];
+    __shared__ int sh[33];
+    __shared__ int last;
+    const int tid = threadIdx.x, lane = tid & 31;
+    unsigned long long edges = 0;
+    const int per = gridDim.x / v.R > 0 ? gridDim.x / v.R : 1;  // blocks per snapshot
+    for (int b = blockIdx.x; b < per * v.R; b += gridDim.x) {
+        const int r = b / per, part = b - r * per;
+        SnapInfo *info = v.info + r;
+        const int nI = info->nI;
+        const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
+        const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
+        const uint32_t *lu = v.marki + (size_t)r * v.iw, *lmr = v.lmr + (size_t)r * v.jw;
+        for (int i = part * 256 + tid; i < nI; i += per * 256) {
+            const unsigned long long a = v.acc[io + i];
+            unsigned int c = sn_lo(a), d = v.deg[io + i];
+            bool walk = false;
+            if (sn_hi(a) > 0) {
+                int o = i;
+                while (v.share[io + o] >= 0) o = v.share[io + o];
+                int wd = sn_hi(a), pos = (int)sn_lo(v.pj[io + o]), before = -1;
+                for (int step = 0;; ++step) {
+                    if (wd >= 2) {
+                        const unsigned long long cv = v.cv[io + o];
+                        if ((uint32_t)sn_hi(cv) & CV_CYCLE) {
+                            if (step > 0) {
+                                walk = true;
+                                break;
+                            }
+                            c = 0;  // its own tree is among the joins found
+                            d = 0;
+                        }
+                        c += (uint32_t)sn_hi(cv) & ~CV_CYCLE;
+                        d += sn_lo(cv);
+                        break;
+                    }
+                    const int j = (int)(jarc[pos] & ~ARC_LEAF);
+                    const int4 e = v.rec[jo + j];
+                    c += (unsigned)e.x;
+                    d += (unsigned)e.y;
+                    if (e.w == 0) break;
+                    if (step >= 32 || j == before) {  // a cycle of one-arc joins, or perhaps one
+                        walk = true;
+                        break;
+                    }
+                    before = j;
+                    o = v.jint[jo + j];
+                    while (v.share[io + o] >= 0) o = v.share[io + o];
+                    wd = e.w;
+                    pos = e.z;
+                }
+            }
+            if (walk) {
+                const unsigned long long pj = v.pj[io + i];
+                const bool l = sn_bit(lu, i);
+                c = l ? (unsigned)info->lmk_cnt : 0u;
+                d = l ? (unsigned)info->lmk_deg : 0u;
+                int n;
+                if (small_walk<false, EDGES>(&list[0][tid], 256, jarc, v.rec + jo, l ? lmr : nullptr, nullptr, nullptr,
+                                             (int)sn_lo(pj), sn_hi(a), c, d, n)) {
+                    const int rj = v.jid[io + ~sn_hi(pj)];
+                    bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
+                    for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
+                    if (!cyc) {
+                        c += sn_lo(a);
+                        d += v.deg[io + i];
+                    }
+                    walk = false;
+                }
+            }
+            if (walk) {
+                if (sn_bit(lu, i)) v.fb[io + v.icap - 1 - atomicAdd(&info->f1, 1)] = i;
+                else v.fb[io + atomicAdd(&info->f0, 1)] = i;
+            } else {
+                v.cnt[io + i] = c;
+                atomicAdd((unsigned long long *)&s[v.inode[io + i]], (unsigned long long)c);
+                edges += d;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) edges += __shfl_xor_sync(SN_FULL, edges, o);
+    if (lane == 0 && edges) atomicAdd(&ctl->init_edges, edges);
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(v.arrive, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sn_plan(v, sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].f1 : &v.info[q].f0); },
+            [&](int q) { return sn_vol(&v.info[q].C); });
+    if (tid == 0) *v.arrive = 0;
+}
+
+// ------------------------------------------------------------- a round
+
+// Cover R(v*) in one snapshot, subtract from the ancestors of v*, and list
+// the ranges whose counts need a walk (Algorithm 2, inner loops), with the
+// joins such a walk may enter: the newly covered ones and the marked ones
+// above them.  With many newly covered joins one of them serves as the
+// round's landmark, as in the initial gains.
+__global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, long long *s, unsigned long long *cov)
+{
+    extern __shared__ uint32_t smem_list[];  // [SW_CAP][T]
+    __shared__ ExpandShared S;
+    __shared__ int tail, itail, nnew, tnew, nt0, nt1, last, pleaf;
+    __shared__ unsigned int lw;
+    __shared__ unsigned long long best;
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+    SnapInfo *info = v.info + r;
+    const int x = sn_vol(&ctl->vstar);
+    const int C = info->C;
+    const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
+    const uint32_t *outb = v.outb + (size_t)r * v.n32, *joinb = v.joinb + (size_t)r * v.n32;
+    const int32_t *outp = v.outp + (size_t)r * v.n32, *joinp = v.joinp + (size_t)r * v.n32;
+    const uint32_t *lb = v.lb + (size_t)r * v.m32;
+    unsigned long long *covw = cov + (size_t)(r >> 6) * (size_t)v.n;
+    const unsigned long long cbit = 1ull << (r & 63);
+    const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
+    const int32_t *jin = v.jin + (size_t)r * v.cap;
+    const int32_t *inoff = v.inoff + (size_t)r * (v.jcap + 1);
+    const int32_t *tn = v.tn + (size_t)r * v.tcap, *par = v.par + io, *jid = v.jid + io;
+    const int4 *rec = v.rec + jo;
+    uint32_t *covj = v.covj + (size_t)r * v.jw, *rel = v.rel + (size_t)r * v.jw, *lmr = v.lmr + (size_t)r * v.jw;
+    uint2 *rel2 = v.rel2 + (size_t)r * v.jw;
+    uint32_t *covi = v.covi + (size_t)r * v.iw, *mk = v.marki + (size_t)r * v.iw;
+    int32_t *ql = v.jlist + jo, *qi = v.ilist + io;
+    const int cw = (C + 31) >> 5;
+    unsigned long long fwd = 0, rev = 0;
+    const bool run = x >= 0 && !info->bad && !(covw[x] & cbit);
+    int nrel = 0;
+    if (tid == 0) {
+        tail = 0;
+        itail = 0;
+        nnew = 0;
+        tnew = 0;
+        nt0 = 0;
+        nt1 = 0;
+        pleaf = -1;
+        lw = 0;
+        best = 0;
+    }
+    __syncthreads();
+    if (run) {
+        const bool internal = sn_bit(outb, x), isj = sn_bit(joinb, x);
+        const int xi = internal ? sn_rank(outb, outp, x) : -1;
+        const int xj = isj ? sn_rank(joinb, joinp, x) : -1;
+        for (int i = tid; i < cw; i += T) rel[i] = 0;
+        __syncthreads();
+        // newly covered joins: closure from v* over uncovered joins
+        auto cover = [&](int j) {
+            const uint32_t bit = 1u << (j & 31);
+            if (!(atomicOr(&covj[j >> 5], bit) & bit)) {
+                ql[atomicAdd(&tail, 1)] = j;
+                atomicOr(&rel[j >> 5], bit);
+            }
+        };
+        if (isj) {
+            if (tid == 0) cover(xj);
+        } else if (internal) {
+            const int p0 = (int)sn_lo(v.pj[io + xi]), wd = sn_hi(v.acc[io + xi]);
+            for (int k = tid; k < wd; k += T) cover((int)(jarc[p0 + k] & ~ARC_LEAF));
+        }
+        __syncthreads();
+        for (int h = 0;;) {
+            const int t = tail;
+            __syncthreads();
+            if (h >= t) break;
+            sn_expand(
+                S, h, t,
+                [&](int q, int &first, int &len) {
+                    const int4 e = rec[ql[q]];
+                    first = e.z;
+                    len = e.w;
+                },
+                [&](int, int k) { cover((int)(jarc[k] & ~ARC_LEAF)); });
+            h = t;
+        }
+        const int nd = tail;
+        // Uncovered internal nodes above something: marks, and all above
+        // qi[from ..).  Covered (covi) means before this round until the
+        // newly covered nodes are entered below.
+        auto mark = [&](int i) {
+            const uint32_t bit = 1u << (i & 31);
+            if (covi[i >> 5] & bit) return;
+            if (!(atomicOr(&mk[i >> 5], bit) & bit)) qi[atomicAdd(&itail, 1)] = i;
+        };
+        auto up = [&](int from) -> int {
+            int h = from;
+            while (true) {
+                __syncthreads();
+                const int t = itail;
+                __syncthreads();
+                if (h >= t) return t;
+                sn_expand(
+                    S, h, t,
+                    [&](int q, int &first, int &len) {
+                        const int i = qi[q];
+                        const int p = par[i], j = jid[i];
+                        if (p >= 0) {
+                            mark(p);
+                        } else if (j >= 0) {
+                            first = inoff[j];
+                            len = inoff[j + 1] - first;
+                        }
+                    },
+                    [&](int, int k) { mark(jin[k]); });
+                h = t;
+            }
+        };
+        // Ancestors of v*, through newly covered nodes too (v* may lie in a
+        // component with them).  A leaf keeps no parent: its live in-arc is
+        // looked up among its canonical ones.
+        if (isj) {
+            for (int k = inoff[xj] + tid; k < inoff[xj + 1]; k += T) mark(jin[k]);
+        } else if (internal) {
+            if (tid == 0 && par[xi] >= 0) {
+                pleaf = par[xi];
+                mark(par[xi]);
+            }
+        } else {
+            for (int k = __ldg(v.crp + x) + tid; k < __ldg(v.crp + x + 1); k += T) {
+                const int2 a = __ldg(v.cin + k);
+                if ((lb[(uint32_t)a.y >> 5] >> (a.y & 31)) & 1u) {
+                    const int i = sn_rank(outb, outp, a.x);
+                    pleaf = i;
+                    mark(i);
+                }
+            }
+        }
+        const int na = up(0);
+        // newly covered nodes: the trees of those joins and T(v*)
+        auto node = [&](int y) -> int {
+            if (atomicOr(&covw[y], cbit) & cbit) return 0;
+            unsigned int c = 1;
+            if (sn_bit(outb, y)) {
+                const int i = sn_rank(outb, outp, y);
+                atomicOr(&covi[i >> 5], 1u << (i & 31));
+                c = v.cnt[io + i];
+                v.cnt[io + i] = 0;
+            }
+            atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)c));
+            fwd += (unsigned long long)(__ldg(v.rp + y + 1) - __ldg(v.rp + y));
+            rev += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
+            return 1;
+        };
+        int got = 0, gott = 0;
+        if (!isj) {
+            if (internal) {
+                const int p0 = (int)sn_lo(v.pn[io + xi]), len = (int)sn_lo(v.acc[io + xi]);
+                for (int k = tid; k < len; k += T) gott += node(tn[p0 + k]);
+            } else if (tid == 0) {
+                gott += node(x);
+            }
+        }
+        sn_expand(
+            S, 0, nd,
+            [&](int q, int &first, int &len) {
+                const int j = ql[q], i = v.jint[jo + j];
+                if (i < 0) {
+                    got += node(v.jnode[jo + j]);
+                } else {
+                    first = (int)sn_lo(v.pn[io + i]);
+                    len = (int)sn_lo(v.acc[io + i]);
+                }
+            },
+            [&](int, int k) { got += node(tn[k]); });
+        if (gott) atomicAdd(&tnew, gott);
+        if (got + gott) atomicAdd(&nnew, got + gott);
+        __syncthreads();
+        const int N = nnew;
+        for (int q = tid; q < na; q += T) {
+            const int i = qi[q];
+            if (covi[i >> 5] >> (i & 31) & 1u) continue;
+            const int y = v.inode[io + i];
+            v.cnt[io + i] -= (unsigned)N;
+            atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)N));
+            rev += (unsigned long long)N * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
+        }
+        if (tid == 0 && pleaf >= 0 && tnew) {
+            // the tree v* hangs in lost T(v*)
+            const int j = jid[~sn_hi(v.pj[io + pleaf])];
+            if (j >= 0 && !(covj[j >> 5] >> (j & 31) & 1u)) v.rec[jo + j].x -= tnew;
+        }
+        // The round's landmark: the newly covered join with the most arcs
+        // below times in-arcs from uncovered non-ancestors, two steps up.
+        int nu = na;
+        const bool lmk = nd >= 64;
+        if (lmk) {
+            for (int i = tid; i < cw; i += T) lmr[i] = 0;
+            for (int q = tid; q < nd; q += T) {
+                const int j = ql[q], w = rec[j].w;
+                if (w < 2) continue;
+                unsigned long long a = 0;
+                for (int k = inoff[j]; k < inoff[j + 1]; ++k) {
+                    const int i = jin[k];
+                    if ((covi[i >> 5] | mk[i >> 5]) >> (i & 31) & 1u) continue;
+                    const int rj = jid[~sn_hi(v.pj[io + i])];
+                    a += 1ull + (rj >= 0 ? (unsigned long long)(inoff[rj + 1] - inoff[rj]) : 0ull);
+                }
+                if (a) atomicMax(&best, (min(a * (unsigned long long)w, (1ull << 31) - 1ull) << 32) | (uint32_t)j);
+            }
+            __syncthreads();
+            const int lj = best ? (int)(uint32_t)best : -1;
+            if (lj >= 0) {
+                int32_t *qr = v.fb + io;  // free between the initial gains' last walk and the next query
+                if (tid == 0) {
+                    lmr[lj >> 5] = 1u << (lj & 31);
+                    qr[0] = lj;
+                    tail = 1;
+                }
+                __syncthreads();
+                for (int h = 0;;) {
+                    const int t = tail;
+                    __syncthreads();
+                    if (h >= t) break;
+                    sn_expand(
+                        S, h, t,
+                        [&](int q, int &first, int &len) {
+                            const int4 e = rec[qr[q]];
+                            atomicAdd(&lw, (unsigned)e.x);
+                            first = e.z;
+                            len = e.w;
+                        },
+                        [&](int, int k) {
+                            const int j = (int)(jarc[k] & ~ARC_LEAF);
+                            const uint32_t bit = 1u << (j & 31);
+                            if (!(rel[j >> 5] & bit)) return;  // covered before
+                            if (!(atomicOr(&lmr[j >> 5], bit) & bit)) qr[atomicAdd(&tail, 1)] = j;
+                        });
+                    h = t;
+                }
+                for (int k = inoff[lj] + tid; k < inoff[lj + 1]; k += T) mark(jin[k]);
+                nu = up(na);
+            }
+        }
+        __syncthreads();
+        // the other nodes that reach a newly covered join
+        sn_expand(
+            S, 0, nd,
+            [&](int q, int &first, int &len) {
+                const int j = ql[q];
+                first = inoff[j];
+                len = inoff[j + 1] - first;
+            },
+            [&](int, int k) { mark(jin[k]); });
+        const int ni = up(nu);
+        // marked joins are relevant too
+        for (int q = na + tid; q < ni; q += T) {
+            const int j = jid[qi[q]];
+            if (j >= 0) atomicOr(&rel[j >> 5], 1u << (j & 31));
+        }
+        for (int q = tid; q < ni; q += T) atomicAnd(&mk[qi[q] >> 5], ~(1u << (qi[q] & 31)));
+        __syncthreads();
+        // what each marked node loses: small walks here, the others as tasks
+        int32_t *task = v.task + io;
+        for (int q = na + tid; q < ni; q += T) {
+            const int i = qi[q];
+            if (v.share[io + i] >= 0) continue;  // with the child that has its range
+            unsigned int c = q < nu ? lw : 0u, d = 0;
+            int n;
+            if (!small_walk<true, false>(smem_list + tid, T, jarc, rec, q < nu ? lmr : nullptr, rel, covj,
+                                         (int)sn_lo(v.pj[io + i]), sn_hi(v.acc[io + i]), c, d, n)) {
+                if (q < nu) task[v.icap - 1 - atomicAdd(&nt1, 1)] = i;
+                else task[atomicAdd(&nt0, 1)] = i;
+                continue;
+            }
+            rev += snap_lose(v, s, io, i, c);
+        }
+        __syncthreads();
+        if (nt0 + nt1) {
+            // ranks and records of the relevant joins
+            for (int b = 0; b < cw; b += T) {
+                const int i = b + tid;
+                int tot;
+                const uint32_t w = i < cw ? rel[i] : 0u;
+                const int ex = sn_block_excl(__popc(w), S.sh, tot);
+                if (i < cw) rel2[i] = make_uint2(w, (unsigned)(nrel + ex));
+                nrel += tot;
+                __syncthreads();
+            }
+            int4 *rrec = v.rrec + jo;
+            auto rank = [&](int j) {
+                const uint2 w = rel2[j >> 5];
+                return (int)w.y + __popc(w.x & ((1u << (j & 31)) - 1u));
+            };
+            for (int q = tid; q < nd; q += T) {
+                const int j = ql[q];
+                const int4 e = rec[j];
+                rrec[rank(j)] = make_int4(e.x, e.z, e.w, 0);
+            }
+            for (int q = na + tid; q < ni; q += T) {
+                const int j = jid[qi[q]];
+                if (j < 0) continue;
+                const int4 e = rec[j];
+                rrec[rank(j)] = make_int4(0, e.z, e.w, 0);
+            }
+            if (nt1) {
+                // the landmark's reach by rank, in place of the join bitmap
+                int32_t *qr = v.fb + io;
+                const int nl = tail;
+                for (int i = tid; i < cw; i += T) lmr[i] = 0;
+                __syncthreads();
+                for (int q = tid; q < nl; q += T) {
+                    const int k = rank(qr[q]);
+                    atomicOr(&lmr[k >> 5], 1u << (k & 31));
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        fwd += __shfl_xor_sync(SN_FULL, fwd, o);
+        rev += __shfl_xor_sync(SN_FULL, rev, o);
+    }
+    if (lane == 0 && fwd) atomicAdd(&ctl->fwd_edges, fwd);
+    if (lane == 0 && rev) atomicAdd(&ctl->rev_edges, rev);
+    __syncthreads();
+    if (tid == 0) {
+        info->t0 = nt0;
+        info->t1 = nt1;
+        info->nrel = nrel;
+        info->lmk_cnt = (int)lw;
+        if (nt0 + nt1) atomicAdd(&ctl->rev_tasks, (unsigned long long)(nt0 + nt1));
+        if (nnew) atomicAdd(&ctl->du_entries, (unsigned long long)nnew);
+        __threadfence();
+        last = atomicAdd(v.arrive, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sn_plan(v, S.sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); },
+            [&](int q) { return sn_vol(&v.info[q].nrel); });
+    if (tid == 0) *v.arrive = 0;
+}
+
+}  // namespace
+}  // namespace sgi
