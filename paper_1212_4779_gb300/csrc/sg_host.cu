@@ -1218,7 +1218,7 @@ sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_ca
     for (int32_t i = 0; i < k; ++i) {
         if (stats) SG_CUDA_TRY(cudaEventRecord(e_round[(size_t)i], st));
         const cudaEvent_t fwd = stats ? e_fwd[(size_t)i] : nullptr;
-        if (snap) SG_TRY(run_snap_round(g, ws, co, model, i, st, fwd));
+        if (snap) SG_TRY(run_snap_round(g, ws, co, model, stats != nullptr, i, st, fwd));
         else SG_TRY(run_round(g, ws, co, model, heavy_on, i, st, fwd));
     }
     SG_TRY(plant_injected_flags(ws, st));

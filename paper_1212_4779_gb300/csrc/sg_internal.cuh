@@ -236,6 +236,7 @@ struct SnapInfo {
     int32_t C;         // joins
     int32_t L;         // live arcs
     int32_t JA;        // arcs to joins
+    int32_t N;         // nodes of the trees under internal roots
     int32_t t0, t1;    // closure tasks, from the front / back of the task list
     int32_t f0, f1;    // initial gains: sources that need a walk of their own, likewise
     int32_t lmk_cnt, lmk_deg;  // nodes the landmark reaches, their out-degree sum
@@ -248,6 +249,7 @@ struct SnapInfo {
 // m32 words of the bitmaps over internal nodes / joins / nodes / arcs.
 struct SnapView {
     int32_t n, R, W, cap, icap, jcap, tcap, iw, jw;
+    int32_t aw;        // words of the bitmaps over join arcs
     int32_t wwarps;    // warps of a closure-walk launch
     long long m, n32, m32;
     const int32_t *rp, *col, *esrc, *crp;
@@ -263,19 +265,28 @@ struct SnapView {
     uint32_t *deg, *cnt;                    // [R][icap] out-degree sum of T(v); current marginal count
     unsigned long long *acc;                // [R][icap] (arcs from T(v) to joins, |T(v)|)
     unsigned long long *pj, *pn;            // [R][icap] (~root, first position in jarc) / (~root, ... in tn)
+    int2 *up;                               // [R][icap] what lies above: (first, count) in jin, or (~parent, 1)
+    int2 *rrange;                           // [R][icap] a round's tasks: (first, count) in rarc
     unsigned long long *cv;                 // [R][icap] closure totals of a walked range
     int32_t *task, *fb, *ilist;             // [R][icap]
     int4 *rec;                              // [R][jcap] join: |T|, out-degree sum, first join arc, join arcs
-    int32_t *jnode, *jint, *jlist;          // [R][jcap] node, internal node (-1: none), queue
+    int32_t *jnode, *jlist;                 // [R][jcap] node, queue
+    int2 *jtn;                              // [R][jcap] T(j) in tn: (first, count)
     int32_t *inoff;                         // [R][jcap + 1] in-arcs of a join in jin
     uint32_t *jarc;                         // [R][cap] join arcs: target join, top bit set for a leaf
-    int32_t *jin;                           // [R][cap] in-arcs of joins (internal sources)
-    int32_t *tn;                            // [R][tcap] nodes of the trees, T(v) contiguous
+    int2 *jin;                              // [R][cap] in-arcs of joins: (internal source, position in jarc)
+    int32_t *apos;                          // [R][cap] position in jarc of each live arc to a join
+    int2 *tn;                               // [R][tcap] nodes of the trees, T(v) contiguous: (node, internal or -1)
     uint32_t *covi, *marki;                 // [R][iw] covered / marked internal nodes
-    uint32_t *covj, *rel, *lmr;             // [R][jw] covered joins, a round's relevant ones, landmark's reach
+    uint32_t *covj, *rel;                   // [R][jw] covered joins, a round's relevant ones
+    uint32_t *lmr, *lmc;                    // [R][jw] landmark's reach, the same by rank among the relevant
     uint2 *rel2;                            // [R][jw] word of rel, set bits before it
-    int4 *rrec;                             // [R][jcap] relevant joins by rank: weight, first join arc, join arcs
-    int32_t *cstart, *cnext, *arrive;       // chunk starts [2R + 1], most bits a walk needs, chunk size; counters
+    int4 *rrec;                             // [R][jcap] relevant joins by rank: weight, -, first arc, arcs
+    uint32_t *rarc;                         // [R][cap] arcs to relevant joins, in jarc's order, by rank
+    uint32_t *abit;                         // [R][aw] their positions in jarc ...
+    uint2 *abit2;                           // ... and word of abit, set bits before it
+    int32_t *cstart, *cnext, *arrive;       // chunk starts [2R + 1], most bits a walk needs, chunk size,
+                                            // whether a round's tasks all go to warps; counters
     int32_t *wq;                            // walk queues
     uint32_t *gbm;                          // [blocks][jw] visited bits too large for shared memory
 };
@@ -466,8 +477,8 @@ sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model,
 sg_status run_snap_build(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
 sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, cudaStream_t st,
                         const TierEvents *ev);
-sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t round, cudaStream_t st,
-                         cudaEvent_t after_cover);
+sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, int32_t round,
+                         cudaStream_t st, cudaEvent_t after_cover);
 
 // kernels (sg_kernels.cu)
 sg_status run_heavy_index(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);

@@ -18,7 +18,7 @@ constexpr int WALK_BLOCKS = 2;                // closure-walk blocks per SM
 // gains), over the relevant ones (rounds, which leave more of the SM to L1
 // for the relevance bitmaps).
 constexpr int WALK_SMEM = 108 << 10;
-constexpr int ROUND_SMEM = 48 << 10;
+constexpr int ROUND_SMEM = 64 << 10;
 
 // Live arcs reserved per snapshot.  Their number is a sum of independent
 // coins: the mean plus 16 standard deviations (and a constant for small
@@ -63,6 +63,7 @@ size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base,
     v.tcap = (int32_t)std::min<int64_t>(g->n, 2 * (int64_t)v.cap);
     v.iw = (v.icap + 31) / 32;
     v.jw = (v.jcap + 127) / 128 * 4;  // copied 16 bytes at a time
+    v.aw = (v.cap + 31) / 32;
     v.n32 = (g->n + 255) / 256 * 8;
     v.m32 = (g->m + 255) / 256 * 8;
     v.wwarps = g->num_sms * WALK_BLOCKS * WK_W;
@@ -100,13 +101,15 @@ size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base,
     c.take(v.acc, ri);
     c.take(v.pj, ri);
     c.take(v.pn, ri);
+    c.take(v.up, ri);
+    c.take(v.rrange, ri);
     c.take(v.cv, ri);
     c.take(v.task, ri);
     c.take(v.fb, ri);
     c.take(v.ilist, ri);
     c.take(v.rec, rj);
     c.take(v.jnode, rj);
-    c.take(v.jint, rj);
+    c.take(v.jtn, rj);
     c.take(v.jlist, rj);
     c.take(v.inoff, R * ((size_t)v.jcap + 1));
     c.take(v.jarc, rc);
@@ -116,8 +119,13 @@ size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base,
     c.take(v.rel, R * v.jw);
     c.take(v.rel2, R * v.jw);
     c.take(v.lmr, R * v.jw);
+    c.take(v.lmc, R * v.jw);
     c.take(v.rrec, rj);
-    c.take(v.cstart, 2 * R + 3);
+    c.take(v.rarc, rc);
+    c.take(v.apos, rc);
+    c.take(v.abit, R * v.aw);
+    c.take(v.abit2, R * v.aw);
+    c.take(v.cstart, 2 * R + 4);
     c.take(v.wq, wb * WK_W * WK_QG);
     c.take(v.gbm, wb * v.jw);
     unsigned long long *masks = nullptr;
@@ -255,19 +263,24 @@ sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int mode
     return SG_OK;
 }
 
-// One selection round: argmax, cover, update.
-sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t round, cudaStream_t st,
-                         cudaEvent_t after_cover)
+// One selection round: argmax, cover, update; the edge counts only if `edges`.
+sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, int32_t round,
+                         cudaStream_t st, cudaEvent_t after_cover)
 {
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
     SG_TRY(run_argmax(g, ws, co, round, st));
-    const int T = snap_threads(v), lists = SW_CAP * T * 4;
-    SG_CUDA_TRY(cudaFuncSetAttribute(snap_cover_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lists));
-    snap_cover_kernel<<<v.R, T, lists, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    if (edges) snap_cover_kernel<true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    else snap_cover_kernel<false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
     SG_CUDA_TRY(cudaGetLastError());
     ++g_launches;
     if (after_cover) SG_CUDA_TRY(cudaEventRecord(after_cover, st));
+    const int blocks = g->num_sms * 6;
+    if (edges) snap_lose_kernel<true><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+    else snap_lose_kernel<false><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    ++g_launches;
+    if (edges) return launch_walk<2, true>(g, ws, v, st);
     return launch_walk<2, false>(g, ws, v, st);
 }
 

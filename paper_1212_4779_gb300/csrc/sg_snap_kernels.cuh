@@ -44,10 +44,13 @@ constexpr int WK_W = WK_T / 32;
 constexpr int WK_QS = 128;      // queue entries of a walk in shared memory
 constexpr int WK_QG = 8192;     // ... and in global memory
 constexpr int WK_TS = 128;      // visited joins remembered for a cheap undo
-constexpr int WK_CH = 16;       // most tasks a warp claims at a time
+constexpr int WK_CH = 16;       // most tasks a warp claims at a time (initial gains; rounds: one per lane)
 constexpr int SW_CAP = 16;      // joins a one-thread walk may visit
 constexpr int SW_ARCS = 96;     // ... and arcs it may scan
+constexpr int SW_U = 4;         // ... several at a time
 constexpr int WK_U = 4;         // arcs in flight per lane
+constexpr int ROUND_ONE = 2;    // tasks per chunk from which a round walks with single threads first
+constexpr int ROUND_LMK = 512;  // newly covered joins from which a round has a landmark
 constexpr uint32_t CV_CYCLE = 0x80000000u;
 constexpr uint32_t ARC_LEAF = 0x80000000u;  // jarc: the join has no live out-arc (weight 1, nothing below)
 
@@ -128,7 +131,8 @@ __device__ __forceinline__ int sn_warp_offset(int v, int *sh, int &total)
 // Ranges of queue entries [q0, q1), spread evenly over the block: range(q)
 // gives (first, length) of an entry, body(q, k) is called for each of its
 // elements k.  Few entries hold most elements (hubs), so one warp per entry
-// left most of the block idle.  Ends with a barrier.
+// left most of the block idle.  The body may push to the queue: every thread
+// has read its entries by then.  Ends with a barrier.
 struct ExpandShared {
     int sh[33];
     int ex[SN_T];
@@ -157,6 +161,63 @@ __device__ __forceinline__ void sn_expand(ExpandShared &S, int q0, int q1, Range
         }
         __syncthreads();
     }
+}
+
+// A level-synchronous search over a queue in global memory.  Whoever pushes
+// an entry also loads its range, beside the atomic that claims the entry, and
+// leaves it in shared memory: a level is then two dependent memory accesses
+// (element, claim) where reading queue and range first made it four.
+struct QueueShared {
+    int tail;
+    int2 range[SN_T];
+};
+__device__ __forceinline__ void sn_push(QueueShared &Q, int32_t *queue, int x, int2 range)
+{
+    const int p = atomicAdd(&Q.tail, 1);
+    queue[p] = x;
+    Q.range[p & (SN_T - 1)] = range;
+}
+// Upward searches over internal nodes: the arcs into a join root as its
+// range; a tree node has none, its marker goes on to the parent itself
+// (a tree path is then one level, not one per node).
+__device__ __forceinline__ int2 joins_above(int2 up) { return up.x < 0 ? make_int2(0, 0) : up; }
+__device__ __forceinline__ void mark_path(QueueShared &Q, const int2 *up, uint32_t *marks, int32_t *queue, int i)
+{
+    while (true) {
+        const uint32_t bit = 1u << (i & 31);
+        const int2 e = up[i];
+        if (atomicOr(&marks[i >> 5], bit) & bit) return;
+        sn_push(Q, queue, i, joins_above(e));
+        if (e.x >= 0) return;
+        i = ~e.x;
+    }
+}
+// Expands the queue from entry `from` until no level adds to it (entry(x)
+// gives an entry's range where a level is too long for shared memory,
+// body(k) takes the elements and may push); returns the queue's length.
+// Starts and ends with a barrier.
+template <class Entry, class Body>
+__device__ __forceinline__ int sn_search(ExpandShared &S, QueueShared &Q, const int32_t *queue, int from, Entry entry,
+                                         Body body)
+{
+    int h = from;
+    __syncthreads();
+    while (true) {
+        const int t = Q.tail;
+        if (h >= t) break;
+        const bool held = t - h <= (int)blockDim.x;  // then all are read before any push
+        sn_expand(
+            S, h, t,
+            [&](int q, int &first, int &len) {
+                const int2 e = held ? Q.range[q & (SN_T - 1)] : entry(queue[q]);
+                first = e.x;
+                len = e.y;
+            },
+            [&](int, int k) { body(k); });
+        h = t;
+    }
+    __syncthreads();
+    return h;
 }
 
 // ------------------------------------------------------- coins to bitmaps
@@ -422,7 +483,7 @@ __global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
     unsigned long long *acc = v.acc + io, *pj = v.pj + io, *pn = v.pn + io;
     uint32_t *deg = v.deg + io;
     uint32_t *joinb = v.joinb + (size_t)r * v.n32;
-    int32_t *cut = v.jin + (size_t)r * v.cap;  // scratch here
+    int32_t *cut = v.apos + (size_t)r * v.cap;  // scratch here
     // Pointer doubling: pj = (an ancestor, lowest index on the path up to
     // it).  A round without a change leaves exactly the nodes above which
     // lies a cycle unrooted, each with the cycle's lowest index.
@@ -518,7 +579,10 @@ __global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
             oj += __shfl_sync(SN_FULL, ia, 31);
             on += __shfl_sync(SN_FULL, ib, 31);
         }
-        if (tid == 0) info->JA = JA;
+        if (tid == 0) {
+            info->JA = JA;
+            info->N = N;
+        }
     }
     // absolute positions: (ancestor or ~root, offset below it)
     rounds = 0;
@@ -576,10 +640,10 @@ __global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
 
 // The chunks of tasks of every snapshot's two task segments, in order, and
 // the most bits a walk needs (one block; cnt(r, seg) gives the lengths,
-// ids(r) the bits).  A chunk is WK_CH tasks, fewer when there would not be
-// several chunks for each walking warp.
+// ids(r) the bits).  A chunk is `chunk` tasks, fewer (not below `least`) when
+// there would not be several chunks for each walking warp.
 template <class F, class G>
-__device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, F cnt, G ids)
+__device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, int least, int chunk, F cnt, G ids)
 {
     const int tid = threadIdx.x, T = blockDim.x;
     __shared__ int most;
@@ -597,7 +661,7 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, F cnt, G ids
         }
     }
     __syncthreads();
-    const int ch = (int)max(1ull, min((unsigned long long)WK_CH, all / (unsigned long long)(8 * v.wwarps)));
+    const int ch = (int)max((unsigned long long)least, min((unsigned long long)chunk, all / (unsigned long long)(8 * v.wwarps)));
     int carry = 0;
     for (int base = 0; base < 2 * v.R; base += T) {
         const int q = base + tid;
@@ -611,6 +675,7 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, F cnt, G ids
         v.cstart[2 * v.R] = carry;
         v.cstart[2 * v.R + 1] = most;
         v.cstart[2 * v.R + 2] = ch;
+        v.cstart[2 * v.R + 3] = 0;
         *v.cnext = 0;
     }
 }
@@ -622,7 +687,7 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, F cnt, G ids
 __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
 {
     __shared__ ExpandShared S;
-    __shared__ int tail;
+    __shared__ QueueShared Q;
     __shared__ unsigned long long best;
     __shared__ unsigned int lc, ld;
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
@@ -635,28 +700,29 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
     unsigned long long *fill = v.cv + io;
     int32_t *inoff = v.inoff + (size_t)r * (v.jcap + 1);
     uint32_t *jarc = v.jarc + ao;
-    int32_t *jin = v.jin + ao, *tn = v.tn + (size_t)r * v.tcap;
+    int2 *jin = v.jin + ao, *tn = v.tn + (size_t)r * v.tcap;
     int4 *rec = v.rec + jo;
     for (int c = tid; c <= C; c += T) inoff[c] = 0;
     if (tid == 0) {
         best = 0;
         lc = 0;
         ld = 0;
-        tail = 0;
+        Q.tail = 0;
     }
-    for (int i = tid; i < nI; i += T) tn[sn_lo(pn[i])] = v.inode[io + i];
+    for (int i = tid; i < nI; i += T) tn[sn_lo(pn[i])] = make_int2(v.inode[io + i], i);
     __syncthreads();
     for (int j = tid; j < L; j += T) {
         const int2 a = v.arc[ao + j];
         const bool out = sn_bit(outb, a.y);
         if (sn_bit(joinb, a.y)) {
             const int c = sn_rank(joinb, joinp, a.y);
-            const int k = sn_hi(atomicAdd(&fill[a.x], 1ull << 32));
-            jarc[sn_lo(pj[a.x]) + k] = (uint32_t)c | (out ? 0u : ARC_LEAF);
+            const int k = sn_hi(atomicAdd(&fill[a.x], 1ull << 32)) + (int)sn_lo(pj[a.x]);
+            jarc[k] = (uint32_t)c | (out ? 0u : ARC_LEAF);
+            v.apos[ao + j] = k;
             atomicAdd(&inoff[c + 1], 1);
         } else if (!out) {
             const int k = (int)sn_lo(atomicAdd(&fill[a.x], 1ull));
-            tn[sn_lo(pn[a.x]) + 1 + k] = a.y;
+            tn[sn_lo(pn[a.x]) + 1 + k] = make_int2(a.y, -1);
         }
     }
     __syncthreads();
@@ -678,31 +744,44 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
             off += __shfl_sync(SN_FULL, inc, 31);
         }
     }
+    // joins without out-arcs follow the trees in the node list
+    const int trees = info->N;
+    if (tid == 0) ld = 0;
+    __syncthreads();
     for (int c = tid; c < C; c += T) {
         const int y = v.jnode[jo + c];
         if (sn_bit(outb, y)) {
             const int i = sn_rank(outb, outp, y);
-            v.jint[jo + c] = i;
             v.jid[io + i] = c;
+            v.jtn[jo + c] = make_int2((int)sn_lo(pn[i]), (int)sn_lo(acc[i]));
             rec[c] = make_int4((int)sn_lo(acc[i]), (int)v.deg[io + i], (int)sn_lo(pj[i]), sn_hi(acc[i]));
         } else {
-            v.jint[jo + c] = -1;
+            const int p = trees + (int)atomicAdd(&ld, 1u);
+            tn[p] = make_int2(y, -1);
+            v.jtn[jo + c] = make_int2(p, 1);
             rec[c] = make_int4(1, __ldg(v.rp + y + 1) - __ldg(v.rp + y), 0, 0);
         }
     }
     __syncthreads();
     for (int j = tid; j < L; j += T) {
         const int2 a = v.arc[ao + j];
-        if (sn_bit(joinb, a.y)) jin[atomicAdd(&inoff[sn_rank(joinb, joinp, a.y) + 1], 1)] = a.x;
+        if (sn_bit(joinb, a.y))
+            jin[atomicAdd(&inoff[sn_rank(joinb, joinp, a.y) + 1], 1)] = make_int2(a.x, v.apos[ao + j]);
     }
     __syncthreads();
+    int2 *up = v.up + io;
+    for (int i = tid; i < nI; i += T) {
+        const int p = v.par[io + i], j = v.jid[io + i];
+        up[i] = p >= 0 ? make_int2(~p, 1) : (j >= 0 ? make_int2(inoff[j], inoff[j + 1] - inoff[j]) : make_int2(0, 0));
+    }
+    if (tid == 0) ld = 0;
     // landmark: join arcs below times in-arcs up to two steps above
     for (int c = tid; c < C; c += T) {
         const int w = rec[c].w;
         if (w < 2) continue;
         unsigned long long up = 0;
         for (int k = inoff[c]; k < inoff[c + 1]; ++k) {
-            const int j = v.jid[io + ~sn_hi(pj[jin[k]])];
+            const int j = v.jid[io + ~sn_hi(pj[jin[k].x])];
             up += 1ull + (j >= 0 ? (unsigned long long)(inoff[j + 1] - inoff[j]) : 0ull);
         }
         const unsigned long long sc = min(up * (unsigned long long)w, (1ull << 31) - 1ull);
@@ -717,61 +796,32 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
     for (int i = tid; i < iw; i += T) lu[i] = 0;
     __syncthreads();
     if (x >= 0) {
+        auto below = [&](int j) {
+            const int4 e = rec[j];
+            return make_int2(e.z, e.w);
+        };
         if (tid == 0) {
             lr[x >> 5] = 1u << (x & 31);
-            ql[0] = x;
-            tail = 1;
+            sn_push(Q, ql, x, below(x));
         }
-        __syncthreads();
-        for (int h = 0;;) {  // R(x): joins
-            const int t = tail;
-            __syncthreads();
-            if (h >= t) break;
-            sn_expand(
-                S, h, t,
-                [&](int q, int &first, int &len) {
-                    const int4 e = rec[ql[q]];
-                    atomicAdd(&lc, (unsigned)e.x);
-                    atomicAdd(&ld, (unsigned)e.y);
-                    first = e.z;
-                    len = e.w;
-                },
-                [&](int, int k) {
-                    const int j = (int)(jarc[k] & ~ARC_LEAF);
-                    const uint32_t bit = 1u << (j & 31);
-                    if (!(atomicOr(&lr[j >> 5], bit) & bit)) ql[atomicAdd(&tail, 1)] = j;
-                });
-            h = t;
+        const int nl = sn_search(S, Q, ql, 0, below, [&](int k) {  // R(x): joins
+            const uint32_t a = jarc[k];
+            const int j = (int)(a & ~ARC_LEAF);
+            const uint32_t bit = 1u << (j & 31);
+            const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
+            if (!(atomicOr(&lr[j >> 5], bit) & bit)) sn_push(Q, ql, j, e);
+        });
+        for (int q = tid; q < nl; q += T) {
+            const int4 e = rec[ql[q]];
+            atomicAdd(&lc, (unsigned)e.x);
+            atomicAdd(&ld, (unsigned)e.y);
         }
-        __syncthreads();
-        if (tid == 0) tail = 0;
+        if (tid == 0) Q.tail = 0;
         __syncthreads();
         // U(x): internal nodes that reach x
-        auto mark = [&](int i) {
-            const uint32_t bit = 1u << (i & 31);
-            if (!(atomicOr(&lu[i >> 5], bit) & bit)) qi[atomicAdd(&tail, 1)] = i;
-        };
-        for (int k = inoff[x] + tid; k < inoff[x + 1]; k += T) mark(jin[k]);
-        __syncthreads();
-        for (int h = 0;;) {
-            const int t = tail;
-            __syncthreads();
-            if (h >= t) break;
-            sn_expand(
-                S, h, t,
-                [&](int q, int &first, int &len) {
-                    const int i = qi[q];
-                    const int p = v.par[io + i], j = v.jid[io + i];
-                    if (p >= 0) {
-                        mark(p);
-                    } else if (j >= 0) {
-                        first = inoff[j];
-                        len = inoff[j + 1] - first;
-                    }
-                },
-                [&](int, int k) { mark(jin[k]); });
-            h = t;
-        }
+        auto mark = [&](int i) { mark_path(Q, up, lu, qi, i); };
+        for (int k = inoff[x] + tid; k < inoff[x + 1]; k += T) mark(jin[k].x);
+        sn_search(S, Q, qi, 0, [&](int i) { return joins_above(up[i]); }, [&](int k) { mark(jin[k].x); });
     }
     __syncthreads();
     if (tid == 0) {
@@ -785,13 +835,12 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
 // One thread's closure walk, for the many ranges that reach only a few
 // joins (on R-MAT 20 three in four): the visited joins are a short list,
 // looked through only when a 64-bit filter says that one may be there.
-// skip: joins left out (NULL: none).  REL: only joins in rel are entered, and
-// only covered ones (covj) count.  Returns false, with the totals
+// skip: joins left out (NULL: none).  Returns false, with the totals
 // meaningless, when the walk is too large; n: visited joins.
-template <bool REL, bool EDGES>
+template <bool EDGES>
 __device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uint32_t *jarc, const int4 *rec,
-                                           const uint32_t *skip, const uint32_t *rel, const uint32_t *covj, int pos,
-                                           int wd, unsigned int &cnt, unsigned int &deg, int &n)
+                                           const uint32_t *skip, int pos, int wd, unsigned int &cnt, unsigned int &deg,
+                                           int &n)
 {
     n = 0;
     int h = 0, p = pos, e = pos + wd, scanned = 0;
@@ -799,23 +848,37 @@ __device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uin
     if (wd > SW_ARCS) return false;
     while (true) {
         if (p < e) {
-            const uint32_t a = jarc[p++];
-            const int j = (int)(a & ~ARC_LEAF);
-            if (REL && !sn_bit(rel, j)) continue;
-            if (skip && sn_bit(skip, j)) continue;
-            const unsigned long long f = 1ull << (((uint32_t)j * 2654435761u) >> 26);
-            if (seen & f) {
-                bool found = false;
-                for (int k = 0; k < n; ++k) found |= list[k * stride] == a;
-                if (found) continue;
+            uint32_t a[SW_U];  // several loads in flight
+            bool in[SW_U];
+#pragma unroll
+            for (int u = 0; u < SW_U; ++u) {
+                in[u] = p + u < e;
+                a[u] = in[u] ? jarc[p + u] : 0u;
             }
-            if (n == SW_CAP) return false;
-            seen |= f;
-            list[n * stride] = a;
-            ++n;
-            if (a & ARC_LEAF) {
-                cnt += 1u;
-                if (EDGES) deg += (unsigned)rec[j].y;
+#pragma unroll
+            for (int u = 0; u < SW_U; ++u) {
+                const int j = (int)(a[u] & ~ARC_LEAF);
+                if (skip && in[u]) in[u] = !sn_bit(skip, j);
+            }
+            p += SW_U;
+#pragma unroll
+            for (int u = 0; u < SW_U; ++u) {
+                if (!in[u]) continue;
+                const int j = (int)(a[u] & ~ARC_LEAF);
+                const unsigned long long f = 1ull << (((uint32_t)j * 2654435761u) >> 26);
+                if (seen & f) {
+                    bool found = false;
+                    for (int k = 0; k < n; ++k) found |= list[k * stride] == a[u];
+                    if (found) continue;
+                }
+                if (n == SW_CAP) return false;
+                seen |= f;
+                list[n * stride] = a[u];
+                ++n;
+                if (a[u] & ARC_LEAF) {
+                    cnt += 1u;
+                    if (EDGES) deg += (unsigned)rec[j].y;
+                }
             }
         } else {
             while (h < n && (list[h * stride] & ARC_LEAF)) ++h;
@@ -823,7 +886,7 @@ __device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uin
             const int j = (int)list[h * stride];
             ++h;
             const int4 r = rec[j];
-            if (!REL || sn_bit(covj, j)) cnt += (unsigned)r.x;
+            cnt += (unsigned)r.x;
             if (EDGES) deg += (unsigned)r.y;
             scanned += r.w;
             if (scanned > SW_ARCS) return false;
@@ -856,8 +919,8 @@ __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
             const bool l = sn_bit(lu, i);
             unsigned int c = l ? (unsigned)info->lmk_cnt : 0u, d = l ? (unsigned)info->lmk_deg : 0u;
             int n;
-            if (small_walk<false, EDGES>(&list[0][tid], 256, v.jarc + (size_t)r * v.cap, v.rec + jo, l ? lmr : nullptr,
-                                         nullptr, nullptr, (int)sn_lo(pj), wd, c, d, n)) {
+            if (small_walk<EDGES>(&list[0][tid], 256, v.jarc + (size_t)r * v.cap, v.rec + jo, l ? lmr : nullptr,
+                                  (int)sn_lo(pj), wd, c, d, n)) {
                 const int rj = v.jid[io + ~sn_hi(pj)];
                 bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
                 for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
@@ -877,7 +940,7 @@ __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
     __syncthreads();
     if (!last) return;
     __threadfence();
-    sn_plan(v, sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); },
+    sn_plan(v, sh, 1, WK_CH, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); },
             [&](int q) { return sn_vol(&v.info[q].C); });
     if (tid == 0) *v.arrive = 0;
 }
@@ -889,27 +952,30 @@ __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
 // entries lie in shared memory; entries past its end are dropped and the
 // walk then re-expands every join it visited (which changes nothing for
 // those already expanded) until no entry was dropped.
-//   REL false  ids are join ids, vis one bit per join, rec their records
-//   REL true   a round: only the relevant joins (rel: bitmap word and set
-//              bits before it) are entered, under their rank among them; vis
-//              and rec (weight, first arc, arcs) are by that rank, so a late
-//              round's few relevant joins take a few words per warp
-template <bool REL>
+template <bool SH>
 struct Walk {
-    uint32_t *vis;
-    int32_t *qs, *ts;    // shared queue and undo list
+    int off;             // the warp's shared memory: queue, undo list, bits (SH)
+    uint32_t *gvis;      // bits in global memory (not SH)
     int32_t *qg;         // global queue
     const uint32_t *jarc;
     const int4 *rec;
-    const uint2 *rel;    // REL
-    int count;           // ids
+    int count;           // joins
     int qt, nt, na;      // queued, visited, arcs scanned
     bool lost;
     unsigned int cnt, deg;
 
-    __device__ __forceinline__ static int first_of(const int4 &e) { return REL ? e.y : e.z; }
-    __device__ __forceinline__ static int arcs_of(const int4 &e) { return REL ? e.z : e.w; }
-
+    // addressed from the shared array itself, so that the accesses compile to
+    // shared-memory instructions
+    __device__ __forceinline__ int32_t *qs() const
+    {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        return reinterpret_cast<int32_t *>(smem_raw + off);
+    }
+    __device__ __forceinline__ int32_t *ts() const { return qs() + WK_QS; }
+    __device__ __forceinline__ uint32_t *vis() const
+    {
+        return SH ? reinterpret_cast<uint32_t *>(qs() + WK_QS + WK_TS) : gvis;
+    }
     // arcs a[u] of this lane, valid where act[u]
     template <bool EDGES, int U>
     __device__ __forceinline__ void arcs(const uint32_t (&a)[U], const bool (&act)[U], int lane)
@@ -920,18 +986,9 @@ struct Walk {
         for (int u = 0; u < U; ++u) {
             id[u] = (int)(a[u] & ~ARC_LEAF);
             fresh[u] = act[u];
-            if (REL && fresh[u]) {
-                const uint2 w = rel[id[u] >> 5];
-                const uint32_t bit = 1u << (id[u] & 31);
-                fresh[u] = (w.x & bit) != 0;
-                id[u] = (int)w.y + __popc(w.x & (bit - 1u));
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
             if (fresh[u]) {
                 const uint32_t bit = 1u << (id[u] & 31);
-                fresh[u] = !(atomicOr(&vis[id[u] >> 5], bit) & bit);
+                fresh[u] = !(atomicOr(&vis()[id[u] >> 5], bit) & bit);
             }
         }
 #pragma unroll
@@ -944,7 +1001,7 @@ struct Walk {
                 const int4 e = rec[id[u]];
                 cnt += (unsigned)e.x;
                 if (EDGES) deg += (unsigned)e.y;
-                push[u] = arcs_of(e) > 0;
+                push[u] = e.w > 0;
             }
         }
         const unsigned lt = (1u << lane) - 1u;
@@ -954,13 +1011,13 @@ struct Walk {
             if (!bf) continue;
             if (fresh[u]) {
                 const int p = nt + __popc(bf & lt);
-                if (p < WK_TS) ts[p] = id[u];
+                if (p < WK_TS) ts()[p] = id[u];
             }
             nt += __popc(bf);
             const unsigned bp = __ballot_sync(SN_FULL, push[u]);
             if (push[u]) {
                 const int p = qt + __popc(bp & lt);
-                if (p < WK_QS) qs[p] = id[u];
+                if (p < WK_QS) qs()[p] = id[u];
                 else if (p < WK_QS + WK_QG) qg[p - WK_QS] = id[u];
             }
             qt += __popc(bp);
@@ -1017,9 +1074,9 @@ struct Walk {
             int pos = 0, wd = 0;
             if (lane < nb) {
                 const int p = qh + lane;
-                const int4 e = rec[p < WK_QS ? qs[p] : qg[p - WK_QS]];
-                pos = first_of(e);
-                wd = arcs_of(e);
+                const int4 e = rec[p < WK_QS ? qs()[p] : qg[p - WK_QS]];
+                pos = e.z;
+                wd = e.w;
             }
             qh += nb;
             const int inc = sn_warp_incl(wd, lane);
@@ -1069,12 +1126,12 @@ struct Walk {
             lost = false;
             const int words = (count + 31) >> 5;
             for (int i = 0; i < words; ++i) {
-                const uint32_t b = *(volatile uint32_t *)&vis[i] & ~(base ? base[i] : 0u);
+                const uint32_t b = *(volatile uint32_t *)&vis()[i] & ~(base ? base[i] : 0u);
                 const int j = i * 32 + lane;
-                const bool act = ((b >> lane) & 1u) && j < count && arcs_of(rec[j]) > 0;
+                const bool act = ((b >> lane) & 1u) && j < count && rec[j].w > 0;
                 const unsigned bp = __ballot_sync(SN_FULL, act);
                 if (!bp) continue;
-                if (act) qs[__popc(bp & ((1u << lane) - 1u))] = j;  // at most 32 <= WK_QS
+                if (act) qs()[__popc(bp & ((1u << lane) - 1u))] = j;  // at most 32 <= WK_QS
                 qt = __popc(bp);
                 queue<EDGES>(lane);
             }
@@ -1086,7 +1143,7 @@ struct Walk {
     {
         __syncwarp();
         if (nt <= WK_TS) {
-            for (int t = lane; t < nt; t += 32) atomicAnd(&vis[ts[t] >> 5], ~(1u << (ts[t] & 31)));
+            for (int t = lane; t < nt; t += 32) atomicAnd(&vis()[ts()[t] >> 5], ~(1u << (ts()[t] & 31)));
             __syncwarp();
         } else {
             load(base, lane);
@@ -1097,7 +1154,7 @@ struct Walk {
     {
         const int words = (count + 31) >> 5;
         // vis areas and bases are 16-byte aligned and padded to 16 bytes
-        int4 *d = reinterpret_cast<int4 *>(vis);
+        int4 *d = reinterpret_cast<int4 *>(vis());
         const int4 *b = reinterpret_cast<const int4 *>(base);
 #pragma unroll 4
         for (int i = lane; i < (words + 3) >> 2; i += 32) d[i] = base ? b[i] : make_int4(0, 0, 0, 0);
@@ -1107,6 +1164,7 @@ struct Walk {
 
 // Internal node i and the tree ancestors that share its range lose c;
 // returns the reverse edges.
+template <bool EDGES>
 __device__ __forceinline__ unsigned long long snap_lose(const SnapView &v, long long *s, size_t io, int i,
                                                         unsigned int c)
 {
@@ -1115,20 +1173,26 @@ __device__ __forceinline__ unsigned long long snap_lose(const SnapView &v, long 
         const int x = v.inode[io + u];
         v.cnt[io + u] -= c;
         atomicAdd((unsigned long long *)&s[x], (unsigned long long)(-(long long)c));
-        edges += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + x + 1) - __ldg(v.crp + x));
+        if (EDGES) edges += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + x + 1) - __ldg(v.crp + x));
         const int p = v.par[io + u];
         if (p < 0 || v.share[io + p] != u) return edges;
         u = p;
     }
 }
 
+// Largest q in [0, count) with start[q] <= t (non-decreasing, start[0] = 0);
+// the whole warp searches, 32 ways a step.
 __device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t)
 {
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (start[mid] <= t) lo = mid;
-        else hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = count;
+    while (n > 1) {
+        const int step = (n + 31) / 32, at = lo + lane * step;
+        const unsigned le = __ballot_sync(SN_FULL, at < lo + n && start[at] <= t);
+        const int k = 31 - __clz((int)le);
+        const int end = lo + n;
+        lo += k * step;
+        n = min(step, end - lo);
     }
     return lo;
 }
@@ -1137,27 +1201,23 @@ __device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t
 // MODE 1: initial gains, sources whose count needs their own walk.
 // MODE 2: a round's marked ranges: the newly covered nodes each reaches,
 //         subtracted from it and from the tree ancestors that share its range.
-// EDGES: also the out-degree sums (MODE 0 and 1).
+// EDGES: also the out-degree sums / reverse edges.
 // Warps claim chunks of tasks in snapshot order, so the graphs of the few
 // snapshots in flight stay in L2.  (Chunks claimed per block, with a barrier
 // after each, left warps waiting for the block's longest walk 40 % of the
 // time.)  Each warp keeps its bits in shared memory (in global memory, one
 // warp per block, when they are more than that holds) and undoes a small
 // walk's bits one by one instead of clearing all.
-template <int MODE, bool EDGES>
-__global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl, long long *s, int smem_bytes)
+template <int MODE, bool EDGES, bool SH>
+__device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long long *s, int area)
 {
-    constexpr bool REL = MODE == 2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int total = v.cstart[2 * v.R], most = v.cstart[2 * v.R + 1], per = v.cstart[2 * v.R + 2];
-    Walk<REL> w;
-    const int area = ((((most + 31) >> 5) * 4 + 15) & ~15) + (WK_QS + WK_TS) * 4;
-    const int nact = smem_bytes / area;
-    if (wid >= max(1, nact)) return;
-    w.qs = reinterpret_cast<int32_t *>(smem_raw + (size_t)wid * (nact ? area : 0));
-    w.ts = w.qs + WK_QS;
-    w.vis = nact ? reinterpret_cast<uint32_t *>(w.ts + WK_TS) : v.gbm + (size_t)blockIdx.x * v.jw;
+    constexpr bool ROUND = MODE == 2;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int total = v.cstart[2 * v.R], per = v.cstart[2 * v.R + 2];
+    const bool all = ROUND && v.cstart[2 * v.R + 3];  // no one-thread walks ran before
+    Walk<SH> w;
+    w.off = SH ? wid * area : 0;
+    w.gvis = v.gbm + (size_t)blockIdx.x * v.jw;
     w.qg = v.wq + ((size_t)blockIdx.x * WK_W + wid) * WK_QG;
     int q = -1, qbeg = 0, qend = 0;  // (snapshot, segment) at hand: its base is in vis
     int cnt = 0, lcnt = 0, ldeg = 0;
@@ -1176,30 +1236,35 @@ __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl
             qend = v.cstart[q + 1];
             const int r = q >> 1, seg = q & 1;
             const SnapInfo *in = v.info + r;
-            cnt = MODE == 1 ? (seg ? in->f1 : in->f0) : (seg ? in->t1 : in->t0);
+            cnt = MODE == 0 || all ? (seg ? in->t1 : in->t0) : (seg ? in->f1 : in->f0);
             lcnt = seg ? in->lmk_cnt : 0;
             ldeg = seg ? in->lmk_deg : 0;
             io = (size_t)r * v.icap;
-            w.count = REL ? in->nrel : in->C;
-            w.jarc = v.jarc + (size_t)r * v.cap;
-            w.rec = (REL ? v.rrec : v.rec) + (size_t)r * v.jcap;
-            w.rel = v.rel2 + (size_t)r * v.jw;
-            base = seg ? v.lmr + (size_t)r * v.jw : nullptr;
-            list = (MODE == 1 ? v.fb : v.task) + io;
+            w.count = ROUND ? in->nrel : in->C;
+            w.jarc = (ROUND ? v.rarc : v.jarc) + (size_t)r * v.cap;
+            w.rec = (ROUND ? v.rrec : v.rec) + (size_t)r * v.jcap;
+            base = seg ? (ROUND ? v.lmc : v.lmr) + (size_t)r * v.jw : nullptr;
+            list = (MODE == 0 || all ? v.task : (MODE == 1 ? v.fb : v.ilist)) + io;
             w.load(base, lane);
         }
         const int k0 = (ch - qbeg) * per, nk = min(cnt - k0, per);
         int ti = 0, tp = 0, tw = 0, tr = 0;  // the chunk's tasks, one per lane
         if (lane < nk) {
             ti = list[(q & 1) ? v.icap - 1 - (k0 + lane) : k0 + lane];
-            const unsigned long long pj = v.pj[io + ti];
-            tp = (int)sn_lo(pj);
-            tw = sn_hi(v.acc[io + ti]);
-            if (!REL) tr = v.jid[io + ~sn_hi(pj)];
+            if (ROUND) {
+                const int2 a = v.rrange[io + ti];
+                tp = a.x;
+                tw = a.y;
+            } else {
+                const unsigned long long pj = v.pj[io + ti];
+                tp = (int)sn_lo(pj);
+                tw = sn_hi(v.acc[io + ti]);
+                tr = v.jid[io + ~sn_hi(pj)];
+            }
         }
         for (int k = 0; k < nk; ++k) {
             const int i = __shfl_sync(SN_FULL, ti, k), rj = __shfl_sync(SN_FULL, tr, k);
-            w.template range<EDGES>(__shfl_sync(SN_FULL, tp, k), __shfl_sync(SN_FULL, tw, k), base, lane);
+            w.template range<EDGES && !ROUND>(__shfl_sync(SN_FULL, tp, k), __shfl_sync(SN_FULL, tw, k), base, lane);
             unsigned int c = w.cnt, d = w.deg;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -1210,7 +1275,7 @@ __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl
                 c += (unsigned)lcnt;
                 d += (unsigned)ldeg;
                 if (MODE != 2) {
-                    const bool cyc = rj >= 0 && (*(volatile uint32_t *)&w.vis[rj >> 5] >> (rj & 31) & 1u);
+                    const bool cyc = rj >= 0 && (*(volatile uint32_t *)&w.vis()[rj >> 5] >> (rj & 31) & 1u);
                     if (MODE == 0) {
                         v.cv[io + i] = sn_pack((int)(c | (cyc ? CV_CYCLE : 0u)), d);
                     } else {
@@ -1223,7 +1288,7 @@ __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl
                         edges += d;
                     }
                 } else {
-                    edges += snap_lose(v, s, io, i, c);
+                    edges += snap_lose<EDGES>(v, s, io, i, c);
                 }
             }
             arcs += (unsigned long long)w.na;
@@ -1231,11 +1296,21 @@ __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl
             w.undo(base, lane);
         }
     }
-    if (lane == 0 && edges) atomicAdd(MODE == 2 ? &ctl->rev_edges : &ctl->init_edges, edges);
+    if (EDGES && lane == 0 && edges) atomicAdd(MODE == 2 ? &ctl->rev_edges : &ctl->init_edges, edges);
     if (lane == 0 && arcs) {
         atomicAdd(&ctl->work_elems[MODE == 2 ? 1 : 0][MODE == 0 ? 0 : 2], arcs);
         atomicAdd(&ctl->work_keys[MODE == 2 ? 1 : 0][MODE == 0 ? 0 : 2], joins);
     }
+}
+
+template <int MODE, bool EDGES>
+__global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl, long long *s, int smem_bytes)
+{
+    const int wid = threadIdx.x >> 5;
+    const int area = ((((v.cstart[2 * v.R + 1] + 31) >> 5) * 4 + 15) & ~15) + (WK_QS + WK_TS) * 4;
+    const int nact = smem_bytes / area;
+    if (wid < nact) walk_tasks<MODE, EDGES, true>(v, ctl, s, area);
+    else if (nact == 0 && wid == 0) walk_tasks<MODE, EDGES, false>(v, ctl, s, area);
 }
 
 // Counts of all internal nodes from the walked ranges.  A node's closure is
@@ -1260,6 +1335,8 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
         const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
         const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
         const uint32_t *lu = v.marki + (size_t)r * v.iw, *lmr = v.lmr + (size_t)r * v.jw;
+        const uint32_t *outb = v.outb + (size_t)r * v.n32;
+        const int32_t *outp = v.outp + (size_t)r * v.n32;
         for (int i = part * 256 + tid; i < nI; i += per * 256) {
             const unsigned long long a = v.acc[io + i];
             unsigned int c = sn_lo(a), d = v.deg[io + i];
@@ -1293,7 +1370,7 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
                         break;
                     }
                     before = j;
-                    o = v.jint[jo + j];
+                    o = sn_rank(outb, outp, v.jnode[jo + j]);
                     while (v.share[io + o] >= 0) o = v.share[io + o];
                     wd = e.w;
                     pos = e.z;
@@ -1305,8 +1382,8 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
                 c = l ? (unsigned)info->lmk_cnt : 0u;
                 d = l ? (unsigned)info->lmk_deg : 0u;
                 int n;
-                if (small_walk<false, EDGES>(&list[0][tid], 256, jarc, v.rec + jo, l ? lmr : nullptr, nullptr, nullptr,
-                                             (int)sn_lo(pj), sn_hi(a), c, d, n)) {
+                if (small_walk<EDGES>(&list[0][tid], 256, jarc, v.rec + jo, l ? lmr : nullptr, (int)sn_lo(pj),
+                                      sn_hi(a), c, d, n)) {
                     const int rj = v.jid[io + ~sn_hi(pj)];
                     bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
                     for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
@@ -1338,7 +1415,7 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
     __syncthreads();
     if (!last) return;
     __threadfence();
-    sn_plan(v, sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].f1 : &v.info[q].f0); },
+    sn_plan(v, sh, 1, WK_CH, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].f1 : &v.info[q].f0); },
             [&](int q) { return sn_vol(&v.info[q].C); });
     if (tid == 0) *v.arrive = 0;
 }
@@ -1350,11 +1427,12 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
 // joins such a walk may enter: the newly covered ones and the marked ones
 // above them.  With many newly covered joins one of them serves as the
 // round's landmark, as in the initial gains.
+template <bool EDGES>
 __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, long long *s, unsigned long long *cov)
 {
-    extern __shared__ uint32_t smem_list[];  // [SW_CAP][T]
     __shared__ ExpandShared S;
-    __shared__ int tail, itail, nnew, tnew, nt0, nt1, last, pleaf;
+    __shared__ QueueShared Q;
+    __shared__ int nnew, tnew, nt0, nt1, last, pleaf;
     __shared__ unsigned int lw;
     __shared__ unsigned long long best;
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
@@ -1368,21 +1446,24 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
     unsigned long long *covw = cov + (size_t)(r >> 6) * (size_t)v.n;
     const unsigned long long cbit = 1ull << (r & 63);
     const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
-    const int32_t *jin = v.jin + (size_t)r * v.cap;
+    const int2 *jin = v.jin + (size_t)r * v.cap;
     const int32_t *inoff = v.inoff + (size_t)r * (v.jcap + 1);
-    const int32_t *tn = v.tn + (size_t)r * v.tcap, *par = v.par + io, *jid = v.jid + io;
+    const int2 *tn = v.tn + (size_t)r * v.tcap, *up = v.up + io;
+    const int32_t *par = v.par + io, *jid = v.jid + io;
     const int4 *rec = v.rec + jo;
     uint32_t *covj = v.covj + (size_t)r * v.jw, *rel = v.rel + (size_t)r * v.jw, *lmr = v.lmr + (size_t)r * v.jw;
     uint2 *rel2 = v.rel2 + (size_t)r * v.jw;
+    // mk: covered or marked in this round; covi: covered
     uint32_t *covi = v.covi + (size_t)r * v.iw, *mk = v.marki + (size_t)r * v.iw;
-    int32_t *ql = v.jlist + jo, *qi = v.ilist + io;
-    const int cw = (C + 31) >> 5;
+    int32_t *ql = v.jlist + jo, *qi = v.ilist + io, *qr = v.fb + io;  // fb is free after the initial gains
+    uint32_t *abit = v.abit + (size_t)r * v.aw;  // arcs to relevant joins, by position in jarc
+    uint2 *abit2 = v.abit2 + (size_t)r * v.aw;
+    const int cw = (C + 31) >> 5, aw = (info->JA + 31) >> 5;
     unsigned long long fwd = 0, rev = 0;
     const bool run = x >= 0 && !info->bad && !(covw[x] & cbit);
     int nrel = 0;
     if (tid == 0) {
-        tail = 0;
-        itail = 0;
+        Q.tail = 0;
         nnew = 0;
         tnew = 0;
         nt0 = 0;
@@ -1391,79 +1472,50 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
         lw = 0;
         best = 0;
     }
-    __syncthreads();
     if (run) {
         const bool internal = sn_bit(outb, x), isj = sn_bit(joinb, x);
         const int xi = internal ? sn_rank(outb, outp, x) : -1;
         const int xj = isj ? sn_rank(joinb, joinp, x) : -1;
         for (int i = tid; i < cw; i += T) rel[i] = 0;
+        for (int i = tid; i < aw; i += T) abit[i] = 0;
         __syncthreads();
         // newly covered joins: closure from v* over uncovered joins
-        auto cover = [&](int j) {
+        auto below = [&](int j) {
+            const int4 e = rec[j];
+            return make_int2(e.z, e.w);
+        };
+        auto cover = [&](uint32_t a) {
+            const int j = (int)(a & ~ARC_LEAF);
             const uint32_t bit = 1u << (j & 31);
+            const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
             if (!(atomicOr(&covj[j >> 5], bit) & bit)) {
-                ql[atomicAdd(&tail, 1)] = j;
                 atomicOr(&rel[j >> 5], bit);
+                sn_push(Q, ql, j, e);
             }
         };
         if (isj) {
-            if (tid == 0) cover(xj);
+            if (tid == 0) cover((uint32_t)xj);
         } else if (internal) {
             const int p0 = (int)sn_lo(v.pj[io + xi]), wd = sn_hi(v.acc[io + xi]);
-            for (int k = tid; k < wd; k += T) cover((int)(jarc[p0 + k] & ~ARC_LEAF));
+            for (int k = tid; k < wd; k += T) cover(jarc[p0 + k]);
         }
+        const int nd = sn_search(S, Q, ql, 0, below, [&](int k) { cover(jarc[k]); });
+        // Ancestors of v*: uncovered internal nodes above it, through newly
+        // covered nodes too (v* may lie in a component with them).  A leaf
+        // keeps no parent: its live in-arc is looked up among its canonical
+        // ones.
+        auto mark = [&](int i) { mark_path(Q, up, mk, qi, i); };
+        auto mark_up = [&](int k) { mark(jin[k].x); };
+        auto mark_arc = [&](int k) {
+            const int2 a = jin[k];
+            atomicOr(&abit[a.y >> 5], 1u << (a.y & 31));
+            mark(a.x);
+        };
+        auto above = [&](int i) { return joins_above(up[i]); };
+        if (tid == 0) Q.tail = 0;
         __syncthreads();
-        for (int h = 0;;) {
-            const int t = tail;
-            __syncthreads();
-            if (h >= t) break;
-            sn_expand(
-                S, h, t,
-                [&](int q, int &first, int &len) {
-                    const int4 e = rec[ql[q]];
-                    first = e.z;
-                    len = e.w;
-                },
-                [&](int, int k) { cover((int)(jarc[k] & ~ARC_LEAF)); });
-            h = t;
-        }
-        const int nd = tail;
-        // Uncovered internal nodes above something: marks, and all above
-        // qi[from ..).  Covered (covi) means before this round until the
-        // newly covered nodes are entered below.
-        auto mark = [&](int i) {
-            const uint32_t bit = 1u << (i & 31);
-            if (covi[i >> 5] & bit) return;
-            if (!(atomicOr(&mk[i >> 5], bit) & bit)) qi[atomicAdd(&itail, 1)] = i;
-        };
-        auto up = [&](int from) -> int {
-            int h = from;
-            while (true) {
-                __syncthreads();
-                const int t = itail;
-                __syncthreads();
-                if (h >= t) return t;
-                sn_expand(
-                    S, h, t,
-                    [&](int q, int &first, int &len) {
-                        const int i = qi[q];
-                        const int p = par[i], j = jid[i];
-                        if (p >= 0) {
-                            mark(p);
-                        } else if (j >= 0) {
-                            first = inoff[j];
-                            len = inoff[j + 1] - first;
-                        }
-                    },
-                    [&](int, int k) { mark(jin[k]); });
-                h = t;
-            }
-        };
-        // Ancestors of v*, through newly covered nodes too (v* may lie in a
-        // component with them).  A leaf keeps no parent: its live in-arc is
-        // looked up among its canonical ones.
         if (isj) {
-            for (int k = inoff[xj] + tid; k < inoff[xj + 1]; k += T) mark(jin[k]);
+            for (int k = inoff[xj] + tid; k < inoff[xj + 1]; k += T) mark(jin[k].x);
         } else if (internal) {
             if (tid == 0 && par[xi] >= 0) {
                 pleaf = par[xi];
@@ -1479,113 +1531,112 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
                 }
             }
         }
-        const int na = up(0);
+        const int na = sn_search(S, Q, qi, 0, above, mark_up);
         // newly covered nodes: the trees of those joins and T(v*)
-        auto node = [&](int y) -> int {
+        auto node = [&](int y, int i) -> int {
             if (atomicOr(&covw[y], cbit) & cbit) return 0;
             unsigned int c = 1;
-            if (sn_bit(outb, y)) {
-                const int i = sn_rank(outb, outp, y);
+            if (i >= 0) {
                 atomicOr(&covi[i >> 5], 1u << (i & 31));
+                atomicOr(&mk[i >> 5], 1u << (i & 31));
                 c = v.cnt[io + i];
                 v.cnt[io + i] = 0;
             }
             atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)c));
-            fwd += (unsigned long long)(__ldg(v.rp + y + 1) - __ldg(v.rp + y));
-            rev += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
+            if (EDGES) {
+                fwd += (unsigned long long)(__ldg(v.rp + y + 1) - __ldg(v.rp + y));
+                rev += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
+            }
             return 1;
         };
         int got = 0, gott = 0;
         if (!isj) {
             if (internal) {
                 const int p0 = (int)sn_lo(v.pn[io + xi]), len = (int)sn_lo(v.acc[io + xi]);
-                for (int k = tid; k < len; k += T) gott += node(tn[p0 + k]);
+                for (int k = tid; k < len; k += T) gott += node(tn[p0 + k].x, tn[p0 + k].y);
             } else if (tid == 0) {
-                gott += node(x);
+                gott += node(x, -1);
             }
         }
         sn_expand(
             S, 0, nd,
             [&](int q, int &first, int &len) {
-                const int j = ql[q], i = v.jint[jo + j];
-                if (i < 0) {
-                    got += node(v.jnode[jo + j]);
-                } else {
-                    first = (int)sn_lo(v.pn[io + i]);
-                    len = (int)sn_lo(v.acc[io + i]);
-                }
+                const int2 e = v.jtn[jo + ql[q]];
+                first = e.x;
+                len = e.y;
             },
-            [&](int, int k) { got += node(tn[k]); });
+            [&](int, int k) {
+                const int2 a = tn[k];
+                got += node(a.x, a.y);
+            });
         if (gott) atomicAdd(&tnew, gott);
         if (got + gott) atomicAdd(&nnew, got + gott);
         __syncthreads();
         const int N = nnew;
         for (int q = tid; q < na; q += T) {
             const int i = qi[q];
-            if (covi[i >> 5] >> (i & 31) & 1u) continue;
+            if (sn_bit(covi, i)) continue;
             const int y = v.inode[io + i];
             v.cnt[io + i] -= (unsigned)N;
             atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)N));
-            rev += (unsigned long long)N * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
+            if (EDGES) rev += (unsigned long long)N * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
         }
         if (tid == 0 && pleaf >= 0 && tnew) {
             // the tree v* hangs in lost T(v*)
             const int j = jid[~sn_hi(v.pj[io + pleaf])];
-            if (j >= 0 && !(covj[j >> 5] >> (j & 31) & 1u)) v.rec[jo + j].x -= tnew;
+            if (j >= 0 && !sn_bit(covj, j)) v.rec[jo + j].x -= tnew;
         }
         // The round's landmark: the newly covered join with the most arcs
         // below times in-arcs from uncovered non-ancestors, two steps up.
-        int nu = na;
-        const bool lmk = nd >= 64;
-        if (lmk) {
+        int nu = na, nl = 0;
+        if (nd >= ROUND_LMK) {
             for (int i = tid; i < cw; i += T) lmr[i] = 0;
-            for (int q = tid; q < nd; q += T) {
-                const int j = ql[q], w = rec[j].w;
-                if (w < 2) continue;
-                unsigned long long a = 0;
-                for (int k = inoff[j]; k < inoff[j + 1]; ++k) {
-                    const int i = jin[k];
-                    if ((covi[i >> 5] | mk[i >> 5]) >> (i & 31) & 1u) continue;
+            for (int q = tid; q < nd; q += T) qr[q] = 0;
+            __syncthreads();
+            sn_expand(
+                S, 0, nd,
+                [&](int q, int &first, int &len) {
+                    const int j = ql[q];
+                    if (rec[j].w < 2) return;
+                    first = inoff[j];
+                    len = inoff[j + 1] - first;
+                },
+                [&](int q, int k) {
+                    const int i = jin[k].x;
+                    if (sn_bit(mk, i)) return;
                     const int rj = jid[~sn_hi(v.pj[io + i])];
-                    a += 1ull + (rj >= 0 ? (unsigned long long)(inoff[rj + 1] - inoff[rj]) : 0ull);
-                }
-                if (a) atomicMax(&best, (min(a * (unsigned long long)w, (1ull << 31) - 1ull) << 32) | (uint32_t)j);
+                    atomicAdd(&qr[q], 1 + (rj >= 0 ? inoff[rj + 1] - inoff[rj] : 0));
+                });
+            for (int q = tid; q < nd; q += T) {
+                const unsigned long long a = (unsigned long long)(uint32_t)qr[q];
+                if (a)
+                    atomicMax(&best, (min(a * (unsigned long long)rec[ql[q]].w, (1ull << 31) - 1ull) << 32) |
+                                         (uint32_t)ql[q]);
             }
             __syncthreads();
             const int lj = best ? (int)(uint32_t)best : -1;
             if (lj >= 0) {
-                int32_t *qr = v.fb + io;  // free between the initial gains' last walk and the next query
                 if (tid == 0) {
+                    Q.tail = 0;
                     lmr[lj >> 5] = 1u << (lj & 31);
-                    qr[0] = lj;
-                    tail = 1;
+                    sn_push(Q, qr, lj, below(lj));
                 }
+                nl = sn_search(S, Q, qr, 0, below, [&](int k) {
+                    const uint32_t a = jarc[k];
+                    const int j = (int)(a & ~ARC_LEAF);
+                    const uint32_t bit = 1u << (j & 31);
+                    const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
+                    if (!(rel[j >> 5] & bit)) return;  // covered before
+                    if (!(atomicOr(&lmr[j >> 5], bit) & bit)) sn_push(Q, qr, j, e);
+                });
+                for (int q = tid; q < nl; q += T) atomicAdd(&lw, (unsigned)rec[qr[q]].x);
+                if (tid == 0) Q.tail = na;
                 __syncthreads();
-                for (int h = 0;;) {
-                    const int t = tail;
-                    __syncthreads();
-                    if (h >= t) break;
-                    sn_expand(
-                        S, h, t,
-                        [&](int q, int &first, int &len) {
-                            const int4 e = rec[qr[q]];
-                            atomicAdd(&lw, (unsigned)e.x);
-                            first = e.z;
-                            len = e.w;
-                        },
-                        [&](int, int k) {
-                            const int j = (int)(jarc[k] & ~ARC_LEAF);
-                            const uint32_t bit = 1u << (j & 31);
-                            if (!(rel[j >> 5] & bit)) return;  // covered before
-                            if (!(atomicOr(&lmr[j >> 5], bit) & bit)) qr[atomicAdd(&tail, 1)] = j;
-                        });
-                    h = t;
-                }
-                for (int k = inoff[lj] + tid; k < inoff[lj + 1]; k += T) mark(jin[k]);
-                nu = up(na);
+                for (int k = inoff[lj] + tid; k < inoff[lj + 1]; k += T) mark(jin[k].x);
+                nu = sn_search(S, Q, qi, na, above, mark_arc);
             }
         }
-        __syncthreads();
+        if (tid == 0) Q.tail = nu;
         // the other nodes that reach a newly covered join
         sn_expand(
             S, 0, nd,
@@ -1594,33 +1645,26 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
                 first = inoff[j];
                 len = inoff[j + 1] - first;
             },
-            [&](int, int k) { mark(jin[k]); });
-        const int ni = up(nu);
-        // marked joins are relevant too
-        for (int q = na + tid; q < ni; q += T) {
-            const int j = jid[qi[q]];
-            if (j >= 0) atomicOr(&rel[j >> 5], 1u << (j & 31));
-        }
-        for (int q = tid; q < ni; q += T) atomicAnd(&mk[qi[q] >> 5], ~(1u << (qi[q] & 31)));
-        __syncthreads();
-        // what each marked node loses: small walks here, the others as tasks
+            [&](int, int k) { mark_arc(k); });
+        const int ni = sn_search(S, Q, qi, nu, above, mark_arc);
+        // their ranges are tasks, the joins among them relevant too
         int32_t *task = v.task + io;
         for (int q = na + tid; q < ni; q += T) {
             const int i = qi[q];
+            const int j = jid[i];
+            if (j >= 0) atomicOr(&rel[j >> 5], 1u << (j & 31));
             if (v.share[io + i] >= 0) continue;  // with the child that has its range
-            unsigned int c = q < nu ? lw : 0u, d = 0;
-            int n;
-            if (!small_walk<true, false>(smem_list + tid, T, jarc, rec, q < nu ? lmr : nullptr, rel, covj,
-                                         (int)sn_lo(v.pj[io + i]), sn_hi(v.acc[io + i]), c, d, n)) {
-                if (q < nu) task[v.icap - 1 - atomicAdd(&nt1, 1)] = i;
-                else task[atomicAdd(&nt0, 1)] = i;
-                continue;
-            }
-            rev += snap_lose(v, s, io, i, c);
+            if (q < nu) task[v.icap - 1 - atomicAdd(&nt1, 1)] = i;
+            else task[atomicAdd(&nt0, 1)] = i;
+        }
+        for (int q = tid; q < ni; q += T) {
+            const int i = qi[q];
+            if (!sn_bit(covi, i)) atomicAnd(&mk[i >> 5], ~(1u << (i & 31)));
         }
         __syncthreads();
         if (nt0 + nt1) {
-            // ranks and records of the relevant joins
+            // The round's own closure graph: relevant joins by rank, the arcs
+            // to them in order; a range of join arcs is again a range.
             for (int b = 0; b < cw; b += T) {
                 const int i = b + tid;
                 int tot;
@@ -1628,48 +1672,80 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
                 const int ex = sn_block_excl(__popc(w), S.sh, tot);
                 if (i < cw) rel2[i] = make_uint2(w, (unsigned)(nrel + ex));
                 nrel += tot;
-                __syncthreads();
             }
+            int na2 = 0;
+            for (int b = 0; b < aw; b += T) {
+                const int i = b + tid;
+                int tot;
+                const uint32_t w = i < aw ? abit[i] : 0u;
+                const int ex = sn_block_excl(__popc(w), S.sh, tot);
+                if (i < aw) abit2[i] = make_uint2(w, (unsigned)(na2 + ex));
+                na2 += tot;
+            }
+            __syncthreads();
             int4 *rrec = v.rrec + jo;
-            auto rank = [&](int j) {
-                const uint2 w = rel2[j >> 5];
+            int2 *rrange = v.rrange + io;
+            uint32_t *rarc = v.rarc + (size_t)r * v.cap;
+            auto rank2 = [](const uint2 *b, int j) {
+                const uint2 w = b[j >> 5];
                 return (int)w.y + __popc(w.x & ((1u << (j & 31)) - 1u));
             };
-            for (int q = tid; q < nd; q += T) {
-                const int j = ql[q];
+            auto range2 = [&](int pos, int wd) {
+                if (wd == 0) return make_int2(0, 0);
+                const int a = rank2(abit2, pos);
+                const int l = pos + wd - 1;  // the last position: its own bit counts too
+                return make_int2(a, rank2(abit2, l) + (int)((abit2[l >> 5].x >> (l & 31)) & 1u) - a);
+            };
+            auto record = [&](int j, bool covered) {
                 const int4 e = rec[j];
-                rrec[rank(j)] = make_int4(e.x, e.z, e.w, 0);
-            }
+                const int2 a = range2(e.z, e.w);
+                rrec[rank2(rel2, j)] = make_int4(covered ? e.x : 0, 0, a.x, a.y);
+            };
             for (int q = na + tid; q < ni; q += T) {
-                const int j = jid[qi[q]];
-                if (j < 0) continue;
-                const int4 e = rec[j];
-                rrec[rank(j)] = make_int4(0, e.z, e.w, 0);
+                const int i = qi[q], j = jid[i];
+                if (j >= 0) record(j, false);
+                if (v.share[io + i] < 0) rrange[i] = range2((int)sn_lo(v.pj[io + i]), sn_hi(v.acc[io + i]));
             }
+            sn_expand(
+                S, 0, nd + ni - na,
+                [&](int q, int &first, int &len) {
+                    const int j = q < nd ? ql[q] : jid[qi[na + q - nd]];
+                    if (j < 0) return;
+                    if (q < nd) record(j, true);
+                    first = inoff[j];
+                    len = inoff[j + 1] - first;
+                },
+                [&](int q, int k) {
+                    const int j = q < nd ? ql[q] : jid[qi[na + q - nd]];
+                    rarc[rank2(abit2, jin[k].y)] = (uint32_t)rank2(rel2, j) | (jarc[jin[k].y] & ARC_LEAF);
+                });
             if (nt1) {
-                // the landmark's reach by rank, in place of the join bitmap
-                int32_t *qr = v.fb + io;
-                const int nl = tail;
-                for (int i = tid; i < cw; i += T) lmr[i] = 0;
+                // the landmark's reach by rank
+                uint32_t *lmc = v.lmc + (size_t)r * v.jw;
+                for (int i = tid; i < v.jw && i * 32 < nrel + 128; i += T) lmc[i] = 0;
                 __syncthreads();
                 for (int q = tid; q < nl; q += T) {
-                    const int k = rank(qr[q]);
-                    atomicOr(&lmr[k >> 5], 1u << (k & 31));
+                    const int k = rank2(rel2, qr[q]);
+                    atomicOr(&lmc[k >> 5], 1u << (k & 31));
                 }
             }
         }
     }
+    if (EDGES) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        fwd += __shfl_xor_sync(SN_FULL, fwd, o);
-        rev += __shfl_xor_sync(SN_FULL, rev, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            fwd += __shfl_xor_sync(SN_FULL, fwd, o);
+            rev += __shfl_xor_sync(SN_FULL, rev, o);
+        }
+        if (lane == 0 && fwd) atomicAdd(&ctl->fwd_edges, fwd);
+        if (lane == 0 && rev) atomicAdd(&ctl->rev_edges, rev);
     }
-    if (lane == 0 && fwd) atomicAdd(&ctl->fwd_edges, fwd);
-    if (lane == 0 && rev) atomicAdd(&ctl->rev_edges, rev);
     __syncthreads();
     if (tid == 0) {
         info->t0 = nt0;
         info->t1 = nt1;
+        info->f0 = 0;
+        info->f1 = 0;
         info->nrel = nrel;
         info->lmk_cnt = (int)lw;
         if (nt0 + nt1) atomicAdd(&ctl->rev_tasks, (unsigned long long)(nt0 + nt1));
@@ -1680,7 +1756,70 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    sn_plan(v, S.sh, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); },
+    // few tasks: one warp each at once, without the one-thread walks
+    auto tasks = [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); };
+    auto ids = [&](int q) { return sn_vol(&v.info[q].nrel); };
+    sn_plan(v, S.sh, 1, WK_CH, tasks, ids);
+    __syncthreads();
+    if (v.cstart[2 * v.R + 2] >= ROUND_ONE) {
+        __syncthreads();
+        sn_plan(v, S.sh, 32, 32, tasks, ids);
+    } else if (tid == 0) {
+        v.cstart[2 * v.R + 3] = 1;
+    }
+    if (tid == 0) *v.arrive = 0;
+}
+
+// What the nodes marked in a round lose, one thread each (a warp claims 32
+// tasks of a snapshot); ranges that are too large go to the warp walks.
+template <bool EDGES>
+__global__ void __launch_bounds__(256) snap_lose_kernel(SnapView v, Ctl *ctl, long long *s)
+{
+    __shared__ uint32_t list[SW_CAP][256];
+    __shared__ int sh[33];
+    __shared__ int last;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int total = v.cstart[2 * v.R];
+    if (v.cstart[2 * v.R + 3] || total == 0) return;
+    unsigned long long edges = 0;
+    while (true) {
+        int ch = 0;
+        if (lane == 0) ch = atomicAdd(v.cnext, 1);
+        ch = __shfl_sync(SN_FULL, ch, 0);
+        if (ch >= total) break;
+        const int q = find_chunk(v.cstart, 2 * v.R, ch);
+        const int r = q >> 1, seg = q & 1;
+        SnapInfo *info = v.info + r;
+        const int k = (ch - v.cstart[q]) * 32 + lane;
+        if (k >= (seg ? info->t1 : info->t0)) continue;
+        const size_t io = (size_t)r * v.icap, jw = (size_t)r * v.jw;
+        const int i = v.task[io + (seg ? v.icap - 1 - k : k)];
+        unsigned int c = seg ? (unsigned)info->lmk_cnt : 0u, d = 0;
+        int n;
+        const int2 a = v.rrange[io + i];
+        if (small_walk<false>(&list[0][tid], 256, v.rarc + (size_t)r * v.cap, v.rrec + (size_t)r * v.jcap,
+                              seg ? v.lmc + jw : nullptr, a.x, a.y, c, d, n))
+            edges += snap_lose<EDGES>(v, s, io, i, c);
+        else if (seg)
+            v.ilist[io + v.icap - 1 - atomicAdd(&info->f1, 1)] = i;
+        else
+            v.ilist[io + atomicAdd(&info->f0, 1)] = i;
+    }
+    if (EDGES) {
+        __syncwarp();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) edges += __shfl_xor_sync(SN_FULL, edges, o);
+        if (lane == 0 && edges) atomicAdd(&ctl->rev_edges, edges);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(v.arrive, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sn_plan(v, sh, 1, WK_CH, [&](int q, int seg) { return sn_vol(seg ? &v.info[q].f1 : &v.info[q].f0); },
             [&](int q) { return sn_vol(&v.info[q].nrel); });
     if (tid == 0) *v.arrive = 0;
 }
