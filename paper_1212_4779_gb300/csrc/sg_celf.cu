@@ -7,14 +7,20 @@
 // this round makes it the seed (every other candidate's gain is at most its
 // bound, and an equal bound comes with a larger id, so this is the lowest-id
 // argmax), otherwise its marginal gain sum_r |R(G'_r, v) \ Cov_r| is
-// computed on the GPU -- a walk from v over a copy of the coverage bits --
-// and it goes back with that bound.  The seed's walk over the coverage
-// itself then marks what it newly covers.
+// computed on the GPU -- a walk from v that leaves out what is covered -- and
+// it goes back with that bound.  The seed's walk over the coverage itself
+// then marks what it newly covers.
+// On the compact snapshot graphs (sg_snap.cu) one launch evaluates the next
+// few stale heads at once: the coverage stands still within a round, so a
+// value computed ahead is the value computed in turn, and only values the
+// queue takes are counted as evaluations.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <queue>
+#include <unordered_map>
 #include <vector>
 
 #include "sg_internal.cuh"
@@ -61,15 +67,22 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     const int launches0 = g_launches;
     sg_workspace &ws = g->ws;
     const size_t n = (size_t)g->n, nw = n * (size_t)co.W;
-    SG_TRY(ensure_workspace(g, ws, co.W, k, st));
+    SG_TRY(check_lt_masks(g, co));
+    const bool snap = snap_route(g, co, model);
     // the linear threshold model reads every coin from the live-mask cache
     const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
-    if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
-    ws.slists_on = 0;
-    // every per-query cache is rebuilt for this query's coins
-    ws.fl_on = 0;
-    if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
-    SG_TRY(ensure_mask_cache(g, ws, co, st));
+    if (snap) {
+        SG_TRY(ensure_core(g, ws, co.W, k, st));
+        SG_TRY(ensure_snap(g, ws, co, model, st));
+    } else {
+        SG_TRY(ensure_workspace(g, ws, co.W, k, st));
+        if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
+        ws.slists_on = 0;
+        // every per-query cache is rebuilt for this query's coins
+        ws.fl_on = 0;
+        if (heavy_on) SG_TRY(ensure_fwd_lists(g, ws, co, c.p, model, st));
+        SG_TRY(ensure_mask_cache(g, ws, co, st));
+    }
 
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     struct EvGuard {
@@ -83,17 +96,22 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     if (stats)
         for (auto &e : ev) SG_CUDA_TRY(cudaEventCreate(&e));
     if (stats) SG_CUDA_TRY(cudaEventRecord(ev[0], st));
-    SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, n * sizeof(long long), st));
     SG_CUDA_TRY(cudaMemsetAsync(ws.cov.p, 0, nw * 8, st));
     SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
-    if (heavy_on) {
-        SG_TRY(run_heavy_index(g, ws, co, model, st));
-        if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
-        SG_TRY(run_row_desc(g, ws, co, st));
-        ws.rd_on = 1;
+    if (snap) {
+        SG_TRY(run_snap_build(g, ws, co, model, st));
+        SG_TRY(run_snap_init(g, ws, co, model, stats != nullptr, st, nullptr));
+    } else {
+        SG_CUDA_TRY(cudaMemsetAsync(ws.s.p, 0, n * sizeof(long long), st));
+        if (heavy_on) {
+            SG_TRY(run_heavy_index(g, ws, co, model, st));
+            if (ws.fl_on) SG_TRY(run_fwd_lists(g, ws, co, st));
+            SG_TRY(run_row_desc(g, ws, co, st));
+            ws.rd_on = 1;
+        }
+        if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
+        SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st, nullptr));
     }
-    if (ws.lm_on) SG_TRY(run_mask_cache(g, ws, co, model, st));
-    SG_TRY(run_init_gains(g, ws, co, model, heavy_on, st, nullptr));
     SG_TRY(plant_injected_flags(ws, st));
     if (stats) SG_CUDA_TRY(cudaEventRecord(ev[1], st));
     std::vector<long long> s0(n);
@@ -119,8 +137,9 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
             dbuf_free(c, st);
         }
     } bufs{scratch, cnt, dv, st};
-    SG_TRY(dbuf_alloc(scratch, nw, st));
-    SG_TRY(dbuf_alloc(cnt, 2, st));
+    const int32_t ahead = snap ? snap_eval_count(g, co, model) : 1;  // candidates per evaluation launch
+    SG_TRY(dbuf_alloc(scratch, snap ? (snap_eval_words(g, co, model) + 1) / 2 : nw, st));
+    SG_TRY(dbuf_alloc(cnt, (size_t)std::max(2, ahead), st));
     SG_TRY(dbuf_alloc(dv, 1, st));
 
     std::vector<CelfEntry> heap;
@@ -132,12 +151,40 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     long long evals = 0;
     unsigned long long fwd_edges = 0;
     long long hc[2];
+    std::vector<CelfEntry> next;
+    std::vector<int32_t> cand;
+    std::vector<long long> vals((size_t)ahead);
+    std::unordered_map<int32_t, long long> known;  // this round's values
     for (int32_t i = 0; i < k; ++i) {
         CelfEntry top;
+        known.clear();
         while (true) {
             top = pq.top();
             pq.pop();
             if (top.stamp == i) break;
+            if (snap) {
+                auto it = known.find(top.v);
+                if (it == known.end()) {
+                    cand.assign(1, top.v);
+                    next.clear();
+                    while ((int32_t)cand.size() < ahead && !pq.empty() && pq.top().stamp != i) {
+                        next.push_back(pq.top());
+                        pq.pop();
+                        if (!known.count(next.back().v)) cand.push_back(next.back().v);
+                    }
+                    for (const CelfEntry &e : next) pq.push(e);
+                    SG_TRY(run_snap_eval(g, ws, co, model, cand.data(), (int32_t)cand.size(),
+                                         reinterpret_cast<uint32_t *>(scratch.p),
+                                         reinterpret_cast<unsigned long long *>(cnt.p), st));
+                    SG_CUDA_TRY(cudaMemcpyAsync(vals.data(), cnt.p, cand.size() * 8, cudaMemcpyDeviceToHost, st));
+                    SG_CUDA_TRY(cudaStreamSynchronize(st));
+                    for (size_t b = 0; b < cand.size(); ++b) known[cand[b]] = vals[b];
+                    it = known.find(top.v);
+                }
+                ++evals;
+                pq.push(CelfEntry{it->second, top.v, i});
+                continue;
+            }
             SG_CUDA_TRY(cudaMemcpyAsync(scratch.p, ws.cov.p, nw * 8, cudaMemcpyDeviceToDevice, st));
             SG_TRY(walk_from(g, ws, co, model, heavy_on, top.v, scratch.p, cnt.p, dv.p, hc, st));
             ++evals;
@@ -145,6 +192,10 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
         }
         seeds[(size_t)i] = top.v;
         gains[(size_t)i] = top.bound;
+        if (snap) {
+            SG_TRY(run_snap_cover(g, ws, co, model, top.v, st));
+            continue;
+        }
         SG_TRY(walk_from(g, ws, co, model, heavy_on, top.v, ws.cov.p, cnt.p, dv.p, hc, st));
         if (hc[0] != top.bound) {
             set_error("sg_select_celf: seed %d newly covers %lld, its gain was %lld", top.v, hc[0], top.bound);
@@ -155,6 +206,20 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     if (stats) {
         SG_CUDA_TRY(cudaEventRecord(ev[2], st));
         SG_CUDA_TRY(cudaEventSynchronize(ev[2]));
+    }
+    if (snap) {
+        Ctl hf;
+        SG_CUDA_TRY(cudaMemcpyAsync(&hf, ws.ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+        SG_CUDA_TRY(cudaStreamSynchronize(st));
+        SG_TRY(flags_status(hf.flags));
+        long long covered = 0;
+        for (int64_t v : gains) covered += v;
+        if ((long long)hf.du_entries != covered) {
+            set_error("sg_select_celf: the seeds cover %lld pairs, their gains add to %lld", (long long)hf.du_entries,
+                      covered);
+            return SG_EINTERNAL;
+        }
+        fwd_edges = hf.fwd_edges;
     }
     SG_CUDA_TRY(cudaMemcpy(out_seeds, seeds.data(), (size_t)k * 4, cudaMemcpyDefault));
     SG_CUDA_TRY(cudaMemcpy(out_gains, gains.data(), (size_t)k * 8, cudaMemcpyDefault));
@@ -167,7 +232,7 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
         stats->init_tier3_tasks = h.init_t3;
         stats->kernel_launches = g_launches - launches0;
         stats->heavy_index = heavy_on;
-        stats->mask_cache = ws.lm_on;
+        stats->mask_cache = snap ? (co.lt ? 1 : 0) : ws.lm_on;
         memcpy(stats->work_keys, h.work_keys, sizeof(h.work_keys));
         memcpy(stats->work_elems, h.work_elems, sizeof(h.work_elems));
         cudaEventElapsedTime(&stats->ms_init, ev[0], ev[1]);

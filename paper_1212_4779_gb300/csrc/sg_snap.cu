@@ -263,6 +263,52 @@ sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int mode
     return SG_OK;
 }
 
+// Candidates one evaluation launch takes: their scratch within 8 GiB.
+int32_t snap_eval_count(const sg_graph *g, const Coins &co, int model)
+{
+    SnapView v;
+    carve(g, co, model, nullptr, v, nullptr, nullptr);
+    const size_t each = (size_t)v.R * ((size_t)v.jcap + v.jw) * 4;
+    return (int32_t)std::max<size_t>(1, std::min<size_t>(EV_MAX, ((size_t)8 << 30) / each));
+}
+
+size_t snap_eval_words(const sg_graph *g, const Coins &co, int model)
+{
+    SnapView v;
+    carve(g, co, model, nullptr, v, nullptr, nullptr);
+    return (size_t)snap_eval_count(g, co, model) * v.R * ((size_t)v.jcap + v.jw);
+}
+
+// out[b] = marginal gain of cand[b], b < count (scratch: snap_eval_words).
+sg_status run_snap_eval(sg_graph *g, sg_workspace &ws, const Coins &co, int model, const int32_t *cand, int32_t count,
+                        uint32_t *scratch, unsigned long long *out, cudaStream_t st)
+{
+    SnapView v;
+    carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
+    EvalArgs ev{};
+    for (int32_t b = 0; b < count; ++b) ev.v[b] = cand[b];
+    ev.bits = scratch;
+    ev.queue = reinterpret_cast<int32_t *>(scratch + (size_t)snap_eval_count(g, co, model) * v.R * v.jw);
+    ev.out = out;
+    SG_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)count * 8, st));
+    snap_eval_kernel<<<dim3((unsigned)v.R, (unsigned)count), 256, 0, st>>>(v, ev, ws.cov.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    ++g_launches;
+    return SG_OK;
+}
+
+// Covers what x reaches (forward edges and newly covered pairs into ctl).
+sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t x, cudaStream_t st)
+{
+    SnapView v;
+    carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
+    snap_choose_kernel<<<1, 1, 0, st>>>(ws.ctl.p, x);
+    snap_cover_kernel<true, false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    SG_CUDA_TRY(cudaGetLastError());
+    g_launches += 2;
+    return SG_OK;
+}
+
 // One selection round: argmax, cover, update; the edge counts only if `edges`.
 sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, int32_t round,
                          cudaStream_t st, cudaEvent_t after_cover)
@@ -270,8 +316,8 @@ sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int mod
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
     SG_TRY(run_argmax(g, ws, co, round, st));
-    if (edges) snap_cover_kernel<true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
-    else snap_cover_kernel<false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    if (edges) snap_cover_kernel<true, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    else snap_cover_kernel<false, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
     SG_CUDA_TRY(cudaGetLastError());
     ++g_launches;
     if (after_cover) SG_CUDA_TRY(cudaEventRecord(after_cover, st));

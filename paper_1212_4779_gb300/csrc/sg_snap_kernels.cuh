@@ -1427,7 +1427,8 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
 // joins such a walk may enter: the newly covered ones and the marked ones
 // above them.  With many newly covered joins one of them serves as the
 // round's landmark, as in the initial gains.
-template <bool EDGES>
+// DU false: cover only (no gain is kept current).
+template <bool EDGES, bool DU>
 __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, long long *s, unsigned long long *cov)
 {
     __shared__ ExpandShared S;
@@ -1515,11 +1516,12 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
         if (tid == 0) Q.tail = 0;
         __syncthreads();
         if (isj) {
-            for (int k = inoff[xj] + tid; k < inoff[xj + 1]; k += T) mark(jin[k].x);
+            if (DU)
+                for (int k = inoff[xj] + tid; k < inoff[xj + 1]; k += T) mark(jin[k].x);
         } else if (internal) {
             if (tid == 0 && par[xi] >= 0) {
                 pleaf = par[xi];
-                mark(par[xi]);
+                if (DU) mark(par[xi]);
             }
         } else {
             for (int k = __ldg(v.crp + x) + tid; k < __ldg(v.crp + x + 1); k += T) {
@@ -1527,22 +1529,22 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
                 if ((lb[(uint32_t)a.y >> 5] >> (a.y & 31)) & 1u) {
                     const int i = sn_rank(outb, outp, a.x);
                     pleaf = i;
-                    mark(i);
+                    if (DU) mark(i);
                 }
             }
         }
-        const int na = sn_search(S, Q, qi, 0, above, mark_up);
+        const int na = DU ? sn_search(S, Q, qi, 0, above, mark_up) : 0;
         // newly covered nodes: the trees of those joins and T(v*)
         auto node = [&](int y, int i) -> int {
             if (atomicOr(&covw[y], cbit) & cbit) return 0;
             unsigned int c = 1;
-            if (i >= 0) {
+            if (DU && i >= 0) {
                 atomicOr(&covi[i >> 5], 1u << (i & 31));
                 atomicOr(&mk[i >> 5], 1u << (i & 31));
                 c = v.cnt[io + i];
                 v.cnt[io + i] = 0;
             }
-            atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)c));
+            if (DU) atomicAdd((unsigned long long *)&s[y], (unsigned long long)(-(long long)c));
             if (EDGES) {
                 fwd += (unsigned long long)(__ldg(v.rp + y + 1) - __ldg(v.rp + y));
                 rev += (unsigned long long)c * (unsigned long long)(__ldg(v.crp + y + 1) - __ldg(v.crp + y));
@@ -1589,7 +1591,7 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
         // The round's landmark: the newly covered join with the most arcs
         // below times in-arcs from uncovered non-ancestors, two steps up.
         int nu = na, nl = 0;
-        if (nd >= ROUND_LMK) {
+        if (DU && nd >= ROUND_LMK) {
             for (int i = tid; i < cw; i += T) lmr[i] = 0;
             for (int q = tid; q < nd; q += T) qr[q] = 0;
             __syncthreads();
@@ -1636,17 +1638,20 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
                 nu = sn_search(S, Q, qi, na, above, mark_arc);
             }
         }
-        if (tid == 0) Q.tail = nu;
-        // the other nodes that reach a newly covered join
-        sn_expand(
-            S, 0, nd,
-            [&](int q, int &first, int &len) {
-                const int j = ql[q];
-                first = inoff[j];
-                len = inoff[j + 1] - first;
-            },
-            [&](int, int k) { mark_arc(k); });
-        const int ni = sn_search(S, Q, qi, nu, above, mark_arc);
+        int ni = 0;
+        if (DU) {
+            if (tid == 0) Q.tail = nu;
+            // the other nodes that reach a newly covered join
+            sn_expand(
+                S, 0, nd,
+                [&](int q, int &first, int &len) {
+                    const int j = ql[q];
+                    first = inoff[j];
+                    len = inoff[j + 1] - first;
+                },
+                [&](int, int k) { mark_arc(k); });
+            ni = sn_search(S, Q, qi, nu, above, mark_arc);
+        }
         // their ranges are tasks, the joins among them relevant too
         int32_t *task = v.task + io;
         for (int q = na + tid; q < ni; q += T) {
@@ -1755,6 +1760,10 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
     }
     __syncthreads();
     if (!last) return;
+    if (!DU) {
+        if (tid == 0) *v.arrive = 0;
+        return;
+    }
     __threadfence();
     // few tasks: one warp each at once, without the one-thread walks
     auto tasks = [&](int q, int seg) { return sn_vol(seg ? &v.info[q].t1 : &v.info[q].t0); };
@@ -1769,6 +1778,87 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
     }
     if (tid == 0) *v.arrive = 0;
 }
+
+// Marginal gains of up to EV_MAX candidates (lazy evaluation): block (r, b)
+// adds to out[b] the nodes candidate b would newly cover in snapshot r, a
+// closure over uncovered joins like the cover's, with nothing written back.
+// bits [EV_MAX][R][jw], queues [EV_MAX][R][jcap]: scratch.
+constexpr int EV_MAX = 16;
+struct EvalArgs {
+    int32_t v[EV_MAX];
+    uint32_t *bits;
+    int32_t *queue;
+    unsigned long long *out;
+};
+__global__ void __launch_bounds__(256) snap_eval_kernel(SnapView v, EvalArgs ev, const unsigned long long *cov)
+{
+    __shared__ ExpandShared S;
+    __shared__ QueueShared Q;
+    __shared__ unsigned int sum;
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+    const int x = ev.v[blockIdx.y];
+    const unsigned long long *covw = cov + (size_t)(r >> 6) * (size_t)v.n;
+    const unsigned long long cbit = 1ull << (r & 63);
+    const SnapInfo *info = v.info + r;
+    if (info->bad || (covw[x] & cbit)) return;
+    const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
+    const uint32_t *outb = v.outb + (size_t)r * v.n32, *joinb = v.joinb + (size_t)r * v.n32;
+    const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
+    const int4 *rec = v.rec + jo;
+    const size_t slot = (size_t)blockIdx.y * v.R + r;
+    uint32_t *bits = ev.bits + slot * v.jw;
+    int32_t *ql = ev.queue + slot * v.jcap;
+    const bool internal = sn_bit(outb, x), isj = sn_bit(joinb, x);
+    unsigned int c = 0;
+    if (tid == 0) {
+        sum = 0;
+        Q.tail = 0;
+    }
+    if (internal || isj) {
+        const uint32_t *covj = v.covj + (size_t)r * v.jw;
+        const int cw = (info->C + 31) >> 5;
+        for (int i = tid; i < cw; i += T) bits[i] = covj[i];
+        __syncthreads();
+        auto below = [&](int j) {
+            const int4 e = rec[j];
+            return make_int2(e.z, e.w);
+        };
+        auto found = [&](uint32_t a) {
+            const int j = (int)(a & ~ARC_LEAF);
+            const uint32_t bit = 1u << (j & 31);
+            const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
+            if (!(atomicOr(&bits[j >> 5], bit) & bit)) sn_push(Q, ql, j, e);
+        };
+        const int xi = internal ? sn_rank(outb, v.outp + (size_t)r * v.n32, x) : -1;
+        if (isj) {
+            if (tid == 0) found((uint32_t)sn_rank(joinb, v.joinp + (size_t)r * v.n32, x));
+        } else {
+            const int p0 = (int)sn_lo(v.pj[io + xi]), wd = sn_hi(v.acc[io + xi]);
+            for (int k = tid; k < wd; k += T) found(jarc[p0 + k]);
+        }
+        const int nd = sn_search(S, Q, ql, 0, below, [&](int k) { found(jarc[k]); });
+        for (int q = tid; q < nd; q += T) c += (unsigned)rec[ql[q]].x;
+        if (!isj) {
+            // T(x), unless its tree is among those found
+            const int rj = v.jid[io + ~sn_hi(v.pj[io + xi])];
+            if (rj < 0 || !sn_bit(bits, rj)) {
+                const int2 *tn = v.tn + (size_t)r * v.tcap + (int)sn_lo(v.pn[io + xi]);
+                const int len = (int)sn_lo(v.acc[io + xi]);
+                for (int k = tid; k < len; k += T) c += !(covw[tn[k].x] & cbit);
+            }
+        }
+    } else {
+        __syncthreads();
+        c = tid == 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(SN_FULL, c, o);
+    if (lane == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (tid == 0) atomicAdd(&ev.out[blockIdx.y], (unsigned long long)sum);
+}
+
+__global__ void snap_choose_kernel(Ctl *ctl, int32_t x) { ctl->vstar = x; }
 
 // What the nodes marked in a round lose, one thread each (a warp claims 32
 // tasks of a snapshot); ranges that are too large go to the warp walks.
