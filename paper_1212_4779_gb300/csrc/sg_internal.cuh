@@ -504,6 +504,10 @@ sg_status run_fwd_lists(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStre
 sg_status ensure_fwd_lists(sg_graph *g, sg_workspace &ws, const Coins &co, double p_uic, int model, cudaStream_t st);
 sg_status run_spread(sg_graph *g, const Coins &co, int model, const int32_t *d_S, int32_t ns, long long *d_total,
                      unsigned long long *d_edges, cudaStream_t st);
+// The same, one snapshot per block at a time (sg_spread.cu).
+bool spread_by_snapshot(const sg_graph *g, const Coins &co);
+sg_status run_spread_snapshots(sg_graph *g, const Coins &co, int model, const int32_t *d_S, int32_t ns,
+                               long long *d_total, unsigned long long *d_edges, cudaStream_t st);
 // Walk from d_S over all W words (FWD_GROUPS blocks per word) on the query's
 // coins (heavy-row index and caches of ws when heavy_on): vis [W][n] holds
 // the nodes to leave out and gains the reached bits; pend [W][n] zero;

@@ -2802,6 +2802,8 @@ sg_status run_spread(sg_graph *g, const Coins &co, int model, const int32_t *d_S
                      unsigned long long *d_edges, cudaStream_t st)
 {
     const size_t n = (size_t)g->n;
+    if (spread_by_snapshot(g, co))
+        return run_spread_snapshots(g, co, model, d_S, ns, d_total, d_edges, st);
     // words per launch: dense vis/pend (8 B each) and two level queues (4 B
     // each) per node and word (LT: both orders of the chunk's live-mask
     // cache as well), within 8 GiB, split into launches of equal size (one
