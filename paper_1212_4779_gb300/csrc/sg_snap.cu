@@ -303,7 +303,7 @@ sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int mod
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
     snap_choose_kernel<<<1, 1, 0, st>>>(ws.ctl.p, x);
-    snap_cover_kernel<true, false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    snap_cover_kernel<true, false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, 1);
     SG_CUDA_TRY(cudaGetLastError());
     g_launches += 2;
     return SG_OK;
@@ -316,16 +316,21 @@ sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int mod
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
     SG_TRY(run_argmax(g, ws, co, round, st));
-    if (edges) snap_cover_kernel<true, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
-    else snap_cover_kernel<false, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p);
+    // Small queries (at most 2^18 internal nodes over all snapshots) mark a
+    // few hundred nodes a round; walking those by warps at once saves a launch.
+    const int direct = (long long)v.R * v.icap <= (1 << 18);
+    if (edges) snap_cover_kernel<true, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, direct);
+    else snap_cover_kernel<false, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, direct);
     SG_CUDA_TRY(cudaGetLastError());
     ++g_launches;
     if (after_cover) SG_CUDA_TRY(cudaEventRecord(after_cover, st));
-    const int blocks = g->num_sms * 6;
-    if (edges) snap_lose_kernel<true><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-    else snap_lose_kernel<false><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-    SG_CUDA_TRY(cudaGetLastError());
-    ++g_launches;
+    if (!direct) {
+        const int blocks = g->num_sms * 6;
+        if (edges) snap_lose_kernel<true><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+        else snap_lose_kernel<false><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
+        SG_CUDA_TRY(cudaGetLastError());
+        ++g_launches;
+    }
     if (edges) return launch_walk<2, true>(g, ws, v, st);
     return launch_walk<2, false>(g, ws, v, st);
 }

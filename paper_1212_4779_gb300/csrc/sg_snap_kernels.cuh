@@ -1028,25 +1028,24 @@ struct Walk {
         }
     }
 
-    // arcs a0 + 32u + lane of the batch of ranges (pos, ex) the lanes hold
+    // arcs a0 + 32u + lane of the batch of ranges the lanes hold (none is
+    // empty; ex: a range's offset in the batch): arc t belongs to the last
+    // range starting at or before t; the starts within 32 arcs are a bit
+    // mask, so that is a population count.  rows: ranges starting before a0.
     template <bool EDGES, int U>
-    __device__ __forceinline__ void spread(int a0, int total, int pos, int ex, int lane)
+    __device__ __forceinline__ void spread(int a0, int total, int base, int ex, bool has, int &rows, int lane)
     {
         uint32_t a[U];
         bool act[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int t = a0 + 32 * u + lane;
-            int k = 0;
-            if (U == 1 || a0 + 32 * u < total) {  // the same for the whole warp
-#pragma unroll
-                for (int step = 16; step >= 1; step >>= 1)
-                    if (__shfl_sync(SN_FULL, ex, k + step) <= t) k += step;
-                const int kp = __shfl_sync(SN_FULL, pos, k), kx = __shfl_sync(SN_FULL, ex, k);
-                k = kp + t - kx;
-            }
+            const int t = a0 + 32 * u + lane, at = ex - a0 - 32 * u;
+            const unsigned starts = __reduce_or_sync(SN_FULL, has && (unsigned)at < 32u ? 1u << at : 0u);
+            const int k = rows + __popc(starts & (SN_FULL >> (31 - lane))) - 1;
+            rows += __popc(starts);
+            const int b = __shfl_sync(SN_FULL, base, k);
             act[u] = t < total;
-            a[u] = act[u] ? jarc[k] : 0u;
+            a[u] = act[u] ? jarc[b + t] : 0u;
         }
         arcs<EDGES, U>(a, act, lane);
     }
@@ -1087,12 +1086,13 @@ struct Walk {
                 qh = 0;
                 qt = 0;
             }
+            int rows = 0;
             for (int a0 = 0; a0 < total;) {
                 if (total - a0 > 32) {
-                    spread<EDGES, WK_U>(a0, total, pos, ex, lane);
+                    spread<EDGES, WK_U>(a0, total, pos - ex, ex, lane < nb, rows, lane);
                     a0 += 32 * WK_U;
                 } else {
-                    spread<EDGES, 1>(a0, total, pos, ex, lane);
+                    spread<EDGES, 1>(a0, total, pos - ex, ex, lane < nb, rows, lane);
                     a0 += 32;
                 }
             }
@@ -1427,9 +1427,11 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
 // joins such a walk may enter: the newly covered ones and the marked ones
 // above them.  With many newly covered joins one of them serves as the
 // round's landmark, as in the initial gains.
-// DU false: cover only (no gain is kept current).
+// DU false: cover only (no gain is kept current).  direct: every task goes
+// to the warp walks (the caller launches no one-thread walks).
 template <bool EDGES, bool DU>
-__global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, long long *s, unsigned long long *cov)
+__global__ void __launch_bounds__(SN_T)
+    snap_cover_kernel(SnapView v, Ctl *ctl, long long *s, unsigned long long *cov, int direct)
 {
     __shared__ ExpandShared S;
     __shared__ QueueShared Q;
@@ -1770,7 +1772,7 @@ __global__ void __launch_bounds__(SN_T) snap_cover_kernel(SnapView v, Ctl *ctl, 
     auto ids = [&](int q) { return sn_vol(&v.info[q].nrel); };
     sn_plan(v, S.sh, 1, WK_CH, tasks, ids);
     __syncthreads();
-    if (v.cstart[2 * v.R + 2] >= ROUND_ONE) {
+    if (!direct && v.cstart[2 * v.R + 2] >= ROUND_ONE) {
         __syncthreads();
         sn_plan(v, S.sh, 32, 32, tasks, ids);
     } else if (tid == 0) {
