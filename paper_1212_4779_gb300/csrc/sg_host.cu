@@ -1096,10 +1096,7 @@ sg_status cc_select_impl(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t
     SG_TRY(cc_clear_cover(g, ws, co, st));
     SG_TRY(cc_init_gains(g, ws, co, st));
     if (stats) SG_CUDA_TRY(cudaEventRecord(ev[1], st));
-    for (int32_t i = 0; i < k; ++i) {
-        SG_TRY(run_argmax(g, ws, co, i, st));
-        SG_TRY(cc_round(g, ws, co, st));
-    }
+    SG_TRY(cc_rounds(g, ws, co, k, st));
     SG_TRY(plant_injected_flags(ws, st));
     SG_TRY(run_poison(g, ws, ws.out_seeds.p, ws.out_gains.p, k, st));
     SG_CUDA_TRY(cudaMemcpyAsync(out_seeds, ws.out_seeds.p, (size_t)k * 4, cudaMemcpyDefault, st));

@@ -349,7 +349,7 @@ struct sg_workspace {
     sgi::DBuf<unsigned long long> lm_out, lm_in;
     int32_t lm_cap = 0;       // words the cache was sized for
     // undirected variant: per-snapshot component labels, sizes, degree sums,
-    // covered flags [R][n]; the round's roots and new sizes [2R]
+    // covered flags [R][n]; the roots covered in the last two rounds [2R]
     sgi::DBuf<int32_t> cc_lab, cc_size, cc_root;
     sgi::DBuf<long long> cc_deg;
     sgi::DBuf<uint8_t> cc_cov;
@@ -495,7 +495,7 @@ sg_status cc_prepare_graph(sg_graph *g, cudaStream_t st);
 size_t cc_workspace_bytes(const sg_graph *g, int32_t R);
 sg_status cc_ensure(sg_graph *g, sg_workspace &ws, int32_t R, cudaStream_t st);
 sg_status cc_init_gains(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st);
-sg_status cc_round(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st);
+sg_status cc_rounds(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t k, cudaStream_t st);
 sg_status cc_clear_cover(sg_graph *g, sg_workspace &ws, const Coins &co, cudaStream_t st);
 sg_status cc_spread(sg_graph *g, sg_workspace &ws, const Coins &co, const int32_t *d_S, int32_t ns, long long *d_total,
                     unsigned long long *d_edges, cudaStream_t st);
