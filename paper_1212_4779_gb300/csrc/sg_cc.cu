@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(CC_T) cc_round_kernel(int n, int R, int round,
     __shared__ long long sg[CC_T / 32];
     __shared__ int si[CC_T / 32];
     __shared__ int sh_last;
+    chain_start();
     const int vs = *(volatile int32_t *)&ctl->vstar;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     unsigned long long fwd = 0, rev = 0;
@@ -313,6 +314,7 @@ __global__ void __launch_bounds__(CC_T) cc_round_kernel(int n, int R, int round,
     if (tid == 0) {
         pg[blockIdx.x] = bg;
         pi[blockIdx.x] = bi;
+        chain_next();
         __threadfence();
         sh_last = atomicAdd(&ctl->argmax_arrivals, 1u) == gridDim.x - 1;
     }
@@ -491,11 +493,10 @@ sg_status cc_rounds(sg_graph *g, sg_workspace &ws, const Coins &co, int32_t k, c
     // one partial maximum per block
     const int blocks = std::min(ws.am_blocks, grid_for(g, g->n));
     for (int32_t i = 0; i < k; ++i) {
-        cc_round_kernel<<<blocks, CC_T, 0, st>>>((int)g->n, co.R, i, i + 1 == k, ws.cc_lab.p, ws.cc_size.p,
-                                                 reinterpret_cast<const unsigned long long *>(ws.cc_deg.p),
-                                                 ws.cc_cov.p, ws.cc_root.p, ws.ctl.p, ws.s.p, ws.am_gain.p,
-                                                 ws.am_id.p, ws.out_seeds.p, ws.out_gains.p);
-        SG_CUDA_TRY(cudaGetLastError());
+        SG_CUDA_TRY(launch_chained(cc_round_kernel, blocks, CC_T, 0, st, (int)g->n, co.R, i, i + 1 == k, ws.cc_lab.p,
+                                   ws.cc_size.p, reinterpret_cast<const unsigned long long *>(ws.cc_deg.p),
+                                   ws.cc_cov.p, ws.cc_root.p, ws.ctl.p, ws.s.p, ws.am_gain.p, ws.am_id.p,
+                                   ws.out_seeds.p, ws.out_gains.p));
         ++g_launches;
     }
     return SG_OK;

@@ -91,6 +91,34 @@ void clear_error();
         }                                                                                  \
     } while (0)
 
+// Kernels of a round follow one another within microseconds.  Launched with
+// launch_chained, a kernel's blocks are set up while the last one still runs,
+// and chain_start, their first statement, holds them until it is complete and
+// its writes are seen.  The next kernel is set up once every block of this one
+// has passed chain_next or is done: late, so that waiting blocks do not hold
+// the places of another stream's kernels.  15k nodes, R = 100, k = 50, UIC:
+// 2.20 -> 1.93 ms; with chain_next as the second statement 1.98 ms, but
+// requests on four streams took 129 ms in place of 113.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                  A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 #define SG_TRY(expr)                      \
     do {                                  \
         sg_status s_ = (expr);            \

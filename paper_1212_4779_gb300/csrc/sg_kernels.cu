@@ -2100,6 +2100,7 @@ __global__ void __launch_bounds__(AM_T) argmax_kernel(long long *s, int n, Ctl *
     __shared__ long long sg[AM_T / 32];
     __shared__ int si[AM_T / 32];
     __shared__ int sh_last;
+    chain_start();
     long long bg = -1;
     int bi = -1;
     // 64-bit index: n may lie within one grid stride of 2^31
@@ -2133,6 +2134,7 @@ __global__ void __launch_bounds__(AM_T) argmax_kernel(long long *s, int n, Ctl *
             }
         pg[blockIdx.x] = bg;
         pi[blockIdx.x] = bi;
+        chain_next();
         __threadfence();
         const unsigned prev = atomicAdd(&ctl->argmax_arrivals, 1u);
         sh_last = (prev == gridDim.x - 1);
@@ -2681,9 +2683,8 @@ sg_status init_gains_t(sg_graph *g, sg_workspace &ws, const Coins &co, int heavy
 // For the routes that keep no per-word counts of newly covered nodes.
 sg_status launch_argmax(sg_graph *g, sg_workspace &ws, int32_t round, cudaStream_t st)
 {
-    argmax_kernel<<<ws.am_blocks, AM_T, 0, st>>>(ws.s.p, (int)g->n, ws.ctl.p, ws.am_gain.p, ws.am_id.p,
-                                                 ws.out_seeds.p, ws.out_gains.p, round, nullptr, 0);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(argmax_kernel, ws.am_blocks, AM_T, 0, st, ws.s.p, (int)g->n, ws.ctl.p, ws.am_gain.p,
+                               ws.am_id.p, ws.out_seeds.p, ws.out_gains.p, round, nullptr, 0));
     ++g_launches;
     return SG_OK;
 }

@@ -195,8 +195,7 @@ sg_status launch_walk(sg_graph *g, sg_workspace &ws, const SnapView &v, cudaStre
     auto kern = snap_walk_kernel<MODE, EDGES>;
     constexpr int smem = MODE == 2 ? ROUND_SMEM : WALK_SMEM;
     SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<g->num_sms * WALK_BLOCKS, WK_T, smem, st>>>(v, ws.ctl.p, ws.s.p, smem);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(kern, g->num_sms * WALK_BLOCKS, WK_T, smem, st, v, ws.ctl.p, ws.s.p, smem));
     ++g_launches;
     return SG_OK;
 }
@@ -226,11 +225,10 @@ sg_status run_snap_build(sg_graph *g, sg_workspace &ws, const Coins &co, int mod
     }
     SG_CUDA_TRY(cudaGetLastError());
     const int ntiles = (int)std::min<long long>(((long long)v.n + SN_TILE - 1) / SN_TILE, (long long)g->num_sms * 8);
-    snap_nodes_kernel<<<ntiles, SN_TILE, 0, st>>>(v, ws.ctl.p, ws.s.p);
-    snap_compact_kernel<<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p);
-    snap_trees_kernel<<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p);
-    snap_place_kernel<<<v.R, snap_threads(v), 0, st>>>(v);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(snap_nodes_kernel, ntiles, SN_TILE, 0, st, v, ws.ctl.p, ws.s.p));
+    SG_CUDA_TRY(launch_chained(snap_compact_kernel, v.R, snap_threads(v), 0, st, v, ws.ctl.p));
+    SG_CUDA_TRY(launch_chained(snap_trees_kernel, v.R, snap_threads(v), 0, st, v, ws.ctl.p));
+    SG_CUDA_TRY(launch_chained(snap_place_kernel, v.R, snap_threads(v), 0, st, v));
     g_launches += 5;
     return SG_OK;
 }
@@ -244,15 +242,12 @@ sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int mode
     if (ev && ev->start) SG_CUDA_TRY(cudaEventRecord(ev->start, st));
     // blocks per snapshot of the kernels that give each internal node a thread
     const int per = (int)std::max<long long>(1, std::min<long long>((v.icap + 1023) / 1024, (8LL * g->num_sms + v.R - 1) / v.R));
-    if (edges) snap_small_kernel<true><<<v.R * per, 256, 0, st>>>(v);
-    else snap_small_kernel<false><<<v.R * per, 256, 0, st>>>(v);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(edges ? snap_small_kernel<true> : snap_small_kernel<false>, v.R * per, 256, 0, st, v));
     if (edges) SG_TRY((launch_walk<0, true>(g, ws, v, st)));
     else SG_TRY((launch_walk<0, false>(g, ws, v, st)));
     if (ev && ev->t1) SG_CUDA_TRY(cudaEventRecord(ev->t1, st));
-    if (edges) snap_resolve_kernel<true><<<v.R * per, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-    else snap_resolve_kernel<false><<<v.R * per, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(edges ? snap_resolve_kernel<true> : snap_resolve_kernel<false>, v.R * per, 256, 0, st, v,
+                               ws.ctl.p, ws.s.p));
     g_launches += 2;
     if (ev && ev->t2) SG_CUDA_TRY(cudaEventRecord(ev->t2, st));
     if (edges) SG_TRY((launch_walk<1, true>(g, ws, v, st)));
@@ -319,16 +314,14 @@ sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int mod
     // Small queries (at most 2^18 internal nodes over all snapshots) mark a
     // few hundred nodes a round; walking those by warps at once saves a launch.
     const int direct = (long long)v.R * v.icap <= (1 << 18);
-    if (edges) snap_cover_kernel<true, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, direct);
-    else snap_cover_kernel<false, true><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, direct);
-    SG_CUDA_TRY(cudaGetLastError());
+    SG_CUDA_TRY(launch_chained(edges ? snap_cover_kernel<true, true> : snap_cover_kernel<false, true>, v.R,
+                               snap_threads(v), 0, st, v, ws.ctl.p, ws.s.p, ws.cov.p, direct));
     ++g_launches;
     if (after_cover) SG_CUDA_TRY(cudaEventRecord(after_cover, st));
     if (!direct) {
         const int blocks = g->num_sms * 6;
-        if (edges) snap_lose_kernel<true><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-        else snap_lose_kernel<false><<<blocks, 256, 0, st>>>(v, ws.ctl.p, ws.s.p);
-        SG_CUDA_TRY(cudaGetLastError());
+        SG_CUDA_TRY(launch_chained(edges ? snap_lose_kernel<true> : snap_lose_kernel<false>, blocks, 256, 0, st, v,
+                                   ws.ctl.p, ws.s.p));
         ++g_launches;
     }
     if (edges) return launch_walk<2, true>(g, ws, v, st);

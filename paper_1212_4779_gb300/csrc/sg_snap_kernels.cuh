@@ -304,6 +304,7 @@ __global__ void __launch_bounds__(SN_TILE) snap_coins_kernel(SnapView v, Coins c
 __global__ void __launch_bounds__(SN_TILE) snap_nodes_kernel(SnapView v, Ctl *ctl, long long *s)
 {
     __shared__ uint32_t to[64][SN_TILE / 32], tj[64][SN_TILE / 32];
+    chain_start();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int tiles = (v.n + SN_TILE - 1) / SN_TILE;
     unsigned long long ed = 0;
@@ -385,6 +386,7 @@ __device__ __forceinline__ int sn_chunk_count(const uint32_t *b, long long lo, l
 __global__ void __launch_bounds__(SN_T) snap_compact_kernel(SnapView v, Ctl *ctl)
 {
     __shared__ int sh[33];
+    chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const uint32_t *outb = v.outb + (size_t)r * v.n32, *joinb = v.joinb + (size_t)r * v.n32;
     const uint32_t *lb = v.lb + (size_t)r * v.m32;
@@ -473,6 +475,7 @@ __global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
 {
     __shared__ int sh[33];
     __shared__ int changed, ncut;
+    chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
     SnapInfo *info = v.info + r;
     if (info->bad) return;
@@ -690,6 +693,7 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
     __shared__ QueueShared Q;
     __shared__ unsigned long long best;
     __shared__ unsigned int lc, ld;
+    chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
     SnapInfo *info = v.info + r;
     const int nI = info->nI, L = info->L, C = info->C;
@@ -904,6 +908,7 @@ __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
     __shared__ uint32_t list[SW_CAP][256];
     __shared__ int sh[33];
     __shared__ int last;
+    chain_start();
     const int tid = threadIdx.x;
     const int per = gridDim.x / v.R > 0 ? gridDim.x / v.R : 1;  // blocks per snapshot
     for (int b = blockIdx.x; b < per * v.R; b += gridDim.x) {
@@ -1306,6 +1311,7 @@ __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long lon
 template <int MODE, bool EDGES>
 __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl, long long *s, int smem_bytes)
 {
+    chain_start();
     const int wid = threadIdx.x >> 5;
     const int area = ((((v.cstart[2 * v.R + 1] + 31) >> 5) * 4 + 15) & ~15) + (WK_QS + WK_TS) * 4;
     const int nact = smem_bytes / area;
@@ -1325,6 +1331,7 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
     __shared__ uint32_t list[SW_CAP][256];
     __shared__ int sh[33];
     __shared__ int last;
+    chain_start();
     const int tid = threadIdx.x, lane = tid & 31;
     unsigned long long edges = 0;
     const int per = gridDim.x / v.R > 0 ? gridDim.x / v.R : 1;  // blocks per snapshot
@@ -1438,6 +1445,7 @@ __global__ void __launch_bounds__(SN_T)
     __shared__ int nnew, tnew, nt0, nt1, last, pleaf;
     __shared__ unsigned int lw;
     __shared__ unsigned long long best;
+    chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
     SnapInfo *info = v.info + r;
     const int x = sn_vol(&ctl->vstar);
@@ -1757,6 +1765,7 @@ __global__ void __launch_bounds__(SN_T)
         info->lmk_cnt = (int)lw;
         if (nt0 + nt1) atomicAdd(&ctl->rev_tasks, (unsigned long long)(nt0 + nt1));
         if (nnew) atomicAdd(&ctl->du_entries, (unsigned long long)nnew);
+        chain_next();
         __threadfence();
         last = atomicAdd(v.arrive, 1) == (int)gridDim.x - 1;
     }
@@ -1870,6 +1879,7 @@ __global__ void __launch_bounds__(256) snap_lose_kernel(SnapView v, Ctl *ctl, lo
     __shared__ uint32_t list[SW_CAP][256];
     __shared__ int sh[33];
     __shared__ int last;
+    chain_start();
     const int tid = threadIdx.x, lane = tid & 31;
     const int total = v.cstart[2 * v.R];
     if (v.cstart[2 * v.R + 3] || total == 0) return;
