@@ -68,13 +68,11 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     sg_workspace &ws = g->ws;
     const size_t n = (size_t)g->n, nw = n * (size_t)co.W;
     SG_TRY(check_lt_masks(g, co));
-    const bool snap = snap_route(g, co, model);
+    bool snap = false;
+    SG_TRY(ensure_snap(g, ws, co, model, k, st, &snap));
     // the linear threshold model reads every coin from the live-mask cache
     const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
-    if (snap) {
-        SG_TRY(ensure_core(g, ws, co.W, k, st));
-        SG_TRY(ensure_snap(g, ws, co, model, st));
-    } else {
+    if (!snap) {
         SG_TRY(ensure_workspace(g, ws, co.W, k, st));
         if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
         ws.slists_on = 0;

@@ -419,6 +419,7 @@ void free_workspace(sg_workspace &ws, cudaStream_t st)
     free_core(ws, st);
     free_tiers(ws, st);
     dbuf_free(ws.snap, st);
+    ws.snap_limit = SIZE_MAX;
     dbuf_free(ws.out_seeds, st);
     dbuf_free(ws.out_gains, st);
     ws.kcap = 0;
@@ -1147,11 +1148,9 @@ sg_status select_impl(sg_graph *g, sg_workspace &ws, int32_t R, int32_t k, sg_ca
     // the linear threshold model reads every coin from the live-mask cache
     const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
     SG_TRY(check_lt_masks(g, co));
-    const bool snap = snap_route(g, co, model);
-    if (snap) {
-        SG_TRY(ensure_core(g, ws, co.W, k, st));
-        SG_TRY(ensure_snap(g, ws, co, model, st));
-    } else {
+    bool snap = false;
+    SG_TRY(ensure_snap(g, ws, co, model, k, st, &snap));
+    if (!snap) {
         SG_TRY(ensure_workspace(g, ws, co.W, k, st));
         if (heavy_on) SG_TRY(ensure_heavy_index(g, ws, co.W, st));
         ws.slists_on = 0;
@@ -1360,10 +1359,9 @@ sg_status sg_workspace_create(const sg_graph *g, int32_t R_max, int32_t k_max, v
     // cascade or route adds what it needs when it first runs
     Coins co;
     sg_status rc = make_coins(sg_cascade{SG_WIC, 0.0}, 0, R_max, &co);
-    if (rc == SG_OK && snap_route(g, co, MODEL_WIC)) {
-        rc = ensure_core(gm, *ws, W, k_max, st);
-        if (rc == SG_OK) rc = ensure_snap(gm, *ws, co, MODEL_WIC, st);
-    } else if (rc == SG_OK) {
+    bool snap = false;
+    if (rc == SG_OK) rc = ensure_snap(gm, *ws, co, MODEL_WIC, k_max, st, &snap);
+    if (rc == SG_OK && !snap) {
         rc = ensure_workspace(gm, *ws, W, k_max, st);
         if (rc == SG_OK && heavy_index_enabled(g, W)) rc = ensure_heavy_index(gm, *ws, W, st);
     }
@@ -1517,9 +1515,9 @@ sg_status sg_init_gains(sg_graph *g, int32_t R, sg_cascade c, uint64_t seed, voi
         return flags_status(h.flags);
     }
     SG_TRY(check_lt_masks(g, co));
-    if (snap_route(g, co, model)) {
-        SG_TRY(ensure_core(g, ws, co.W, 1, st));
-        SG_TRY(ensure_snap(g, ws, co, model, st));
+    bool snap = false;
+    SG_TRY(ensure_snap(g, ws, co, model, 1, st, &snap));
+    if (snap) {
         SG_CUDA_TRY(cudaMemsetAsync(ws.ctl.p, 0, sizeof(Ctl), st));
         SG_TRY(run_snap_build(g, ws, co, model, st));
         SG_TRY(run_snap_init(g, ws, co, model, init_edges != nullptr, st, nullptr));

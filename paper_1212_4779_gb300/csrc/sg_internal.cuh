@@ -329,6 +329,7 @@ struct sg_workspace {
     int32_t wcap = 0;     // words of capacity of the [W][n] arrays
     int32_t core_w = 0;   // words of capacity of cov
     sgi::DBuf<unsigned char> snap;  // compact snapshot graphs, laid out per query
+    size_t snap_limit = SIZE_MAX;   // queries that need this much or more run on the tiered engines
     int32_t nslots = 0;   // tier-3 (CTA engine) slots
     int32_t fq_groups = 0;    // forward-walk blocks per word the queues fq_a/fq_b were sized for
     int32_t walk_groups = 8;  // forward/landmark walk blocks per word for the current query
@@ -501,7 +502,8 @@ struct TierEvents {
 bool snap_route(const sg_graph *g, const Coins &co, int model);
 size_t snap_bytes(const sg_graph *g, const Coins &co, int model);
 sg_status build_arc_sources(sg_graph *g, cudaStream_t st);
-sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
+sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t k, cudaStream_t st,
+                      bool *snap);
 sg_status run_snap_build(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st);
 sg_status run_snap_init(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, cudaStream_t st,
                         const TierEvents *ev);

@@ -248,12 +248,17 @@ int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fr
     // the compact graphs' size depends on the cascade, the tiered engines'
     // arrays only on the graph and W
     const bool cc = rq->c.model == SG_UIC_UNDIRECTED;
-    const bool snap = !cc && snap_route(g, co, model);
+    bool snap = !cc && snap_route(g, co, model);
     const size_t core = core_bytes(g, W, s->cfg.k_cap);
+    // a dense cascade whose compact graphs pass the budget runs on the engines
+    const bool dense = snap && core + snap_bytes(g, co, model) > s->budget;
+    if (dense) snap = false;
     const size_t need = cc ? core + cc_workspace_bytes(g, rq->R)
                            : (snap ? core + snap_bytes(g, co, model) : workspace_bytes(g, W, s->cfg.k_cap));
     for (size_t i = 0; i < s->pool.size(); ++i)
-        if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W && s->pool[i].bytes >= need) return (int)i;
+        if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W && s->pool[i].bytes >= need &&
+            (cc || dense == (s->pool[i].ws->snap_limit == 0)))
+            return (int)i;
     while (s->used + need > s->budget) {
         int lru = -1;
         for (size_t i = 0; i < s->pool.size(); ++i)
@@ -278,7 +283,10 @@ int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fr
     sg_workspace *w = new (std::nothrow) sg_workspace();
     if (!w) return -1;
     cudaStream_t st = s->setup_st;
-    if (ensure_core(g, *w, W, s->cfg.k_cap, st) != SG_OK || (snap && ensure_snap(g, *w, co, model, st) != SG_OK) ||
+    if (dense) w->snap_limit = 0;
+    bool fits = true;
+    if (ensure_core(g, *w, W, s->cfg.k_cap, st) != SG_OK ||
+        (snap && (ensure_snap(g, *w, co, model, s->cfg.k_cap, st, &fits) != SG_OK || !fits)) ||
         (!snap && !cc && ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK) ||
         (!snap && !cc && heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
         cudaEventRecord(s->setup_ev, st) != cudaSuccess) {

@@ -177,12 +177,25 @@ sg_status build_arc_sources(sg_graph *g, cudaStream_t st)
     return SG_OK;
 }
 
-sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, cudaStream_t st)
+// Sizes ws for a query on the compact graphs; *snap false, with nothing more
+// done, where it goes to the tiered engines: by snap_route, or because the
+// graphs do not fit into the device's memory (dense cascades: the engines'
+// arrays do not grow with the live arcs).  A workspace remembers the size that
+// did not fit, so that sizing ahead of a capture and recording take one route.
+sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t k, cudaStream_t st,
+                      bool *snap)
 {
     const size_t need = snap_bytes(g, co, model);
+    *snap = snap_route(g, co, model) && need < ws.snap_limit;
+    if (!*snap) return SG_OK;
+    SG_TRY(ensure_core(g, ws, co.W, k, st));
     if (ws.snap.bytes < need) {
         dbuf_free(ws.snap, st);
-        SG_TRY(dbuf_alloc(ws.snap, need, st));
+        if (dbuf_alloc(ws.snap, need, st) != SG_OK) {
+            clear_error();
+            ws.snap_limit = need;
+            *snap = false;
+        }
     }
     return SG_OK;
 }

@@ -150,3 +150,66 @@ def test_undirected_rounds(sg, n, R, k, p):
         assert np.array_equal(res.seeds, ref["seeds"]) and np.array_equal(res.gains, ref["gains"])
         assert [res.stats["init_edges"], res.stats["fwd_edges"]] == [int(x) for x in ref["counters"][:2]]
         assert np.array_equal(g.init_gains(R, "uic_undirected", p, 4)[0], ref["s_init"])
+
+
+@pytest.mark.parametrize("p,R", [(1.0, 256), (0.5, 200)])
+def test_dense_cascades_that_do_not_fit(sg, p, R):
+    """Compact graphs that the allocator, or a server's budget, has no room for
+    leave the query to the tiered engines, whose arrays do not grow with the
+    live arcs: in a selection, in a captured batch and in a server."""
+    import time
+
+    import torch
+
+    n, s, d = inputs.er_directed(2000, 20000, 6)
+    ref = oracle.Graph(n, s, d, "uic", p).select(R, 4, 9, mode=oracle.COVER)
+    held, refused = {}, []
+
+    def alloc(nbytes, stream):
+        if nbytes > 128 << 20:
+            refused.append(nbytes)
+            return None
+        t = torch.empty(max(1, nbytes), dtype=torch.uint8, device="cuda")
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    def release(ptr, nbytes, stream):
+        torch.cuda.synchronize()
+        held.pop(ptr, None)
+
+    sg.sg_set_allocator(alloc, release)
+    try:
+        g = sg.Graph.from_coo(n, s, d)
+        got = [g.select(R, 4, "uic", p, 9), g.select(R, 4, "uic", p, 9), g.select_celf(R, 4, "uic", p, 9)[0]]
+        ws = sg.sg_workspace_create(g.handle, 64, 4)
+        so = torch.zeros(4, dtype=torch.int32, device="cuda")
+        go = torch.zeros(4, dtype=torch.int64, device="cuda")
+        stream = torch.cuda.Stream()
+        b = sg.sg_batch_capture([(g.handle, ws, R, 4, "uic", p, 9, so, go)], 1, stream)
+        sg.sg_batch_launch(b, stream)
+        stream.synchronize()
+        got.append(sg.Selection(so.cpu().numpy(), go.cpu().numpy(), None))
+        sg.sg_batch_free(b)
+        sg.sg_workspace_free(ws)
+        assert len(refused) == 2  # asked for once by each workspace
+        g.close()
+    finally:
+        sg.sg_set_allocator(None, None)
+    g = sg.Graph.from_coo(n, s, d)
+    sv = sg.sg_server_create(2, sg.sg_workspace_bytes(g.handle, R, 128), 128)
+    try:
+        ids = [sg.sg_server_submit(sv, g.handle, R, 4, "uic", p, 9) for _ in range(3)]
+        end = time.time() + 60
+        while ids and time.time() < end:
+            done, seeds, gains, _ = sg.sg_server_poll(sv, ids[0], 4)
+            if not done:
+                time.sleep(0.01)
+                continue
+            got.append(sg.Selection(seeds, gains, None))
+            ids.pop(0)
+        assert not ids
+    finally:
+        sg.sg_server_destroy(sv)
+    g.close()
+    for res in got:
+        assert np.array_equal(res.seeds, ref["seeds"]) and np.array_equal(res.gains, ref["gains"])
