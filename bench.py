@@ -44,19 +44,16 @@ from paper_1212_4779_gb300 import inputs  # noqa: E402
 METRIC = "GTEPS (snapshot-edges/s) of StaticGreedyDU k-seed selection"
 UNIT = "GTEPS"
 
-# Algorithmic bytes per expanded element (one arc, or one live-index entry,
-# for one 64-bit task word, or one per-snapshot list entry) plus the
-# neighbour's 8-byte state word: an arc record is 8 bytes (destination and
-# threshold); a live-index entry (heavy rows) or a cached arc is a 4-byte
-# destination and an 8-byte live mask; a list entry is a 4-byte destination.
-# algorithmic bytes of one expanded element of the dominant kernel
-BYTES_PER_ELEMENT = 16  # hashed arc: 8-byte arc record (destination, threshold) + 8-byte state word
-BYTES_PER_ELEMENT_INDEXED = 20  # index entry: 4-byte neighbour + 8-byte live mask + 8-byte state word
-BYTES_PER_LIST_ELEMENT = 12  # per-snapshot list entry: 4-byte neighbour + 8-byte state word
-# and per expanded (node, 64-snapshot word) of a task: its 8-byte row
-# offsets and its 8-byte state word (the per-node term of the same model)
-BYTES_PER_EXPANDED_NODE = 16
-LANES_PER_SM = 128  # INT32 lanes per SM per clock (4 SMSP x 32)
+# Bytes that the cover kernel of a round cannot do without.  Per newly covered
+# (node, snapshot): its node-list entry (8), its coverage word read and written
+# (16) and its gain read and written (16).  Per range that loses gains: the
+# in-arc that led to it (8), its way up (8), its join's record for the round (16),
+# its range (8) and its task (4).
+BYTES_PER_COVERED = 40
+BYTES_PER_RANGE = 44
+# ... and a closure walk: 16 bytes per visited join, 4 per scanned join arc
+BYTES_PER_JOIN = 16
+BYTES_PER_JOIN_ARC = 4
 
 
 def _peaks():
@@ -124,11 +121,11 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def _recorded_traffic(kernel_src="paper_1212_4779_gb300/csrc/sg_kernels.cu",
-                      summary="profiles/coop_engine_tier3_init_rmat20_traffic.md"):
-    """DRAM bytes per launch of the tier-3 initial-gain kernel from the
-    committed ncu summary, or None when the kernel source has changed since
-    that capture (its sha256 prefix is recorded in the summary)."""
+def _recorded_traffic(kernel_src="paper_1212_4779_gb300/csrc/sg_snap_kernels.cuh",
+                      summary="profiles/snap_cover_rmat20_traffic.md"):
+    """DRAM bytes per launch (mean over the rounds) of the cover kernel from
+    the committed ncu summary, or None when the kernel source has changed
+    since that capture (its sha256 prefix is recorded in the summary)."""
     import hashlib
 
     here = os.path.dirname(os.path.abspath(__file__))
@@ -663,7 +660,7 @@ def main():
     if ws > 1:
         torch.distributed.barrier()
     torch.cuda.synchronize()
-    t_steps, t_t1, t_t3, edges, launches, st_last = [], [], [], [], 0, None
+    t_steps, t_walk, t_fwd, t_lose, edges, launches, st_last = [], [], [], [], [], 0, None
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     for _ in range(args.steps):
@@ -673,8 +670,9 @@ def main():
         ev1.record(stream)
         ev1.synchronize()
         t_steps.append(ev0.elapsed_time(ev1))
-        t_t1.append(st["ms_init_tier1"])
-        t_t3.append(st["ms_init_tier3"])
+        t_walk.append(st["ms_init_tier1"])
+        t_fwd.append(st["ms_fwd"])
+        t_lose.append(st["ms_rounds"] - st["ms_fwd"])
         edges.append(st["init_edges"] + st["fwd_edges"] + st["rev_edges"])
         launches += st["kernel_launches"]
         st_last = st
@@ -685,35 +683,10 @@ def main():
     value /= 1e9
 
     peaks, src = _peaks()
-    sm_mhz = clocks.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
-    n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    # dominant kernel: the initial-gain tier-3 launch (cooperative engine over
-    # dense per-block arrays).  Algorithmic bytes: per expanded (node, word)
-    # its row offsets and state word (16 B); per element an index entry
-    # (4-byte neighbour + 8-byte live mask) or arc record, plus the
-    # neighbour's 8-byte state word; a per-snapshot list entry is a 4-byte
-    # neighbour plus the state word.
-    t3_ms = float(np.mean(t_t3))
-    bpe = BYTES_PER_ELEMENT_INDEXED if (st_last["mask_cache"] or st_last["heavy_index"]) else BYTES_PER_ELEMENT
-    t3_list = st_last["list_elems"][2]
-    t3_keys = st_last["work_keys"][0][2]
-    t3_bytes = (t3_keys * BYTES_PER_EXPANDED_NODE + (st_last["work_elems"][0][2] - t3_list) * bpe +
-                t3_list * BYTES_PER_LIST_ELEMENT)
-    hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
-    achieved = t3_bytes / (t3_ms / 1e3) / 1e9 if t3_ms > 0 else 0.0
-    roofline = {"bound": "hbm", "kernel": "coop_engine_kernel<dense> (initial gains, tier 3)",
-                "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
-                "traffic": _recorded_traffic() if wl.name == "rmat20" else None,
-                "traffic_source": "profiles/coop_engine_tier3_init_rmat20_traffic.md (full-size ncu capture)",
-                "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({src})",
-                "kernel_ms": t3_ms, "elements_per_launch": st_last["work_elems"][0][2],
-                "list_elements_per_launch": t3_list, "expanded_nodes_per_launch": t3_keys,
-                "bytes_per_element": bpe, "bytes_per_list_element": BYTES_PER_LIST_ELEMENT,
-                "bytes_per_expanded_node": BYTES_PER_EXPANDED_NODE, "algorithmic_bytes_per_launch": t3_bytes}
-    t1_ms = float(np.mean(t_t1))
-    alu_view = {"kernel": "warp_engine_kernel (initial gains, tier 1)", "kernel_ms": t1_ms,
-                "elements_per_launch": st_last["work_elems"][0][0],
-                "int_peak_tops": n_sm * LANES_PER_SM * sm_mhz * 1e6 / 1e12}
+    roofline, walks = cover_roofline(wl, st_last, float(np.mean(t_fwd)), peaks, src), None
+    if roofline:
+        walks = {"initial gains": walk_view(st_last, 0, 0, float(np.mean(t_walk))),
+                 "rounds": walk_view(st_last, 1, 2, float(np.mean(t_lose)))}
 
     e2e = None
     if not args.no_e2e:
@@ -749,7 +722,7 @@ def main():
         "work": {"keys": st_last["work_keys"], "elems": st_last["work_elems"]},
         "gpu_launches": launches,
         "roofline": roofline,
-        "tier1_alu_view": alu_view,
+        "closure_walks": walks,
         "cpu_baseline": cpu,
         "e2e": e2e,
         "clocks": clocks,
@@ -763,6 +736,34 @@ def main():
     if ws > 1:
         torch.distributed.destroy_process_group()
     return 0
+
+
+def cover_roofline(wl, st, fwd_ms, peaks, src):
+    """The dominant kernel, snap_cover_kernel: its bytes over the rounds against
+    the copy bandwidth.  Its time includes the rounds' argmax (a few
+    microseconds each).  None where a knob on the command line sent the query to
+    the tiered engines."""
+    if st["init_tier2_tasks"] or st["init_tier3_tasks"] or fwd_ms <= 0:
+        return None
+    need = st["du_entries"] * BYTES_PER_COVERED + st["rev_tasks"] * BYTES_PER_RANGE
+    peak = float(peaks.get("hbm_gbs", 6800.0))
+    achieved = need / (fwd_ms / 1e3) / 1e9
+    return {"bound": "hbm", "kernel": "snap_cover_kernel (one launch a round, with the argmax)",
+            "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            "traffic": _recorded_traffic() if wl.name == "rmat20" else None,
+            "traffic_source": "profiles/snap_cover_rmat20_traffic.md (full-size ncu capture)",
+            "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({src})",
+            "kernel_ms": fwd_ms / wl.k, "launches": wl.k, "algorithmic_bytes_per_launch": need / wl.k,
+            "bytes_per_covered_pair": BYTES_PER_COVERED, "bytes_per_range": BYTES_PER_RANGE}
+
+
+def walk_view(st, phase, col, ms):
+    """Joins visited and join arcs scanned by one phase's closure walks; most
+    of their bytes come from L2, their visited bits from shared memory."""
+    joins, arcs = st["work_keys"][phase][col], st["work_elems"][phase][col]
+    need = joins * BYTES_PER_JOIN + arcs * BYTES_PER_JOIN_ARC
+    return {"ms": ms, "joins": joins, "arcs": arcs, "algorithmic_bytes": need,
+            "gb_per_s": need / (ms / 1e3) / 1e9 if ms > 0 else None}
 
 
 def apply_knobs(sg, args):
@@ -779,10 +780,10 @@ def phase_rates(st):
     expanded per second.  The reverse counter is the implementation-
     independent sum over every (w, r) the dynamic update removes and every u
     reaching w of indeg(u) (the paper's per-node reverse BFS); the library
-    settles most of it without walking (the ancestor pass credits |N_r| to
-    every ancestor of v* at once, target-sliced tasks share walks), so the
-    reverse and total rates are nominal, while `elements_per_s` counts the
-    index entries, arcs and list entries the engines really expanded."""
+    settles most of it without walking (|N_r| comes off every ancestor of v*
+    at once, the others lose a closure's sizes), so the reverse and total
+    rates are nominal, while `elements_per_s` counts the join arcs that the
+    walks really scanned."""
     ms_init = st["ms_init"]
     ms_fwd = st["ms_fwd"]
     ms_rev = max(1e-6, st["ms_rounds"] - ms_fwd)

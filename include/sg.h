@@ -73,9 +73,9 @@ typedef enum {
  *   own the intervals [j w, (j+1) w), w = floor(2^32 / indeg(v)), and the
  *   arc whose interval holds the draw is live (none when the draw is past
  *   indeg(v) w).  p is ignored.  Every entry point accepts it; the coins are
- *   materialised once per query into the live-mask cache (2 x W x m x 8
- *   bytes, at most 16 GiB, else SG_ENOMEM) and the heavy-row index is not
- *   used. */
+ *   materialised once per query: live masks of W x m x 8 bytes on the default
+ *   route, 2 x W x m x 8 in the live-mask cache of the tiered engines (more
+ *   than 16 GiB of the latter gives SG_ENOMEM on either). */
 typedef enum { SG_UIC = 0, SG_WIC = 1, SG_UIC_UNDIRECTED = 2, SG_LT = 3 } sg_model;
 
 /* Cascade model: UIC uses p in [0, 1] for every arc; WIC ignores p and uses
@@ -91,32 +91,46 @@ typedef struct {
  *   fwd_edges  = sum over newly covered (u, r) of outdeg(u)
  *   rev_edges  = sum over newly covered (w, r) and u in U(G'_r, w) of indeg(u)
  * (outdeg / indeg of the canonical graph, live or not).  The other fields
- * describe how this implementation ran (tiers, task counts, device times). */
+ * describe how this implementation ran (task counts, device times).
+ *
+ * Two routes give the same results.  The default builds each snapshot's live
+ * graph in compact form once per query and counts by walks over its joins
+ * (nodes with two or more live in-arcs).  The tiered engines traverse 64
+ * snapshots at a time; they take a query whose knobs (sg_set_walk_groups,
+ * sg_set_direction, sg_set_engine_limits, sg_set_landmarks,
+ * sg_set_scc_condensation, sg_set_forward_lists, sg_set_snapshot_lists,
+ * sg_set_mask_cache, sg_set_heavy_threshold, sg_tuning) are not all at their
+ * defaults, graphs without arcs, and cascades whose compact graphs pass 64 GiB
+ * or the memory there is.  Where a field means something else on the default
+ * route, its comment names that after "default:". */
 typedef struct {
     uint64_t init_edges;
     uint64_t fwd_edges;
     uint64_t rev_edges;
-    uint64_t init_tier2_tasks;  /* initial-gain tasks that outgrew the shared-memory table */
+    uint64_t init_tier2_tasks;  /* initial-gain tasks that outgrew the shared-memory table (default: 0, as the next three) */
     uint64_t init_tier3_tasks;  /* ... and the global-memory table */
     uint64_t rev_tier2_tasks;   /* same for reverse (dynamic-update) tasks */
     uint64_t rev_tier3_tasks;
-    uint64_t rev_tasks;         /* reverse tasks (one snapshot, <= 64 targets), all rounds */
-    uint64_t du_entries;        /* (node, 64-snapshot word) pairs newly covered, all rounds */
-    float ms_index;             /* device time building the heavy-row live index and lists */
+    uint64_t rev_tasks;         /* reverse tasks (one snapshot, <= 64 targets), all rounds; default: ranges walked */
+    uint64_t du_entries;        /* (node, 64-snapshot word) pairs newly covered, all rounds; default: (node, snapshot) */
+    float ms_index;             /* device time building the heavy-row live index and lists; default: the compact graphs */
     float ms_init;              /* device time of the initial gains (index included) */
-    float ms_init_tier1;        /* device time of the initial-gain tier-1 launch */
+    float ms_init_tier1;        /* device time of the initial-gain tier-1 launch; default: all ranges' walks */
     float ms_rounds;            /* device time of the k selection rounds */
     float ms_fwd;               /* ... of which argmax + forward update, summed */
     float ms_total;             /* device time of the whole call */
-    int32_t status_flags;       /* device flags: 1 no argmax candidate, 2 a bounded wait gave up, 8 union-find out of retries */
+    int32_t status_flags;       /* device flags: 1 no argmax candidate, 2 a bounded wait gave up, 8 union-find out of retries,
+                                   16 a snapshot has more live arcs than sized for (16 standard deviations) */
     int32_t kernel_launches;    /* kernels this call launched */
-    int32_t heavy_index;        /* 1 if the heavy-row live index was used */
-    int32_t mask_cache;         /* 1 if the live-mask cache was used */
-    uint64_t work_keys[2][3];   /* [initial, reverse][tier 1..3]: nodes held in task tables */
-    uint64_t work_elems[2][3];  /* [initial, reverse][tier 1..3]: arcs / index entries expanded */
-    float ms_landmarks;         /* device time of the landmark reach sets */
-    float ms_init_tier2;        /* device time of the initial-gain tier-2 launch */
-    float ms_init_tier3;        /* device time of the initial-gain tier-3 launch */
+    int32_t heavy_index;        /* 1 if the heavy-row live index was used (default: as the engines would) */
+    int32_t mask_cache;         /* 1 if the live-mask cache was used (default: LT masks) */
+    uint64_t work_keys[2][3];   /* [initial, reverse][tier 1..3]: nodes held in task tables;
+                                   default: joins visited by walks, [0][0] and [0][2] initial, [1][2] rounds */
+    uint64_t work_elems[2][3];  /* [initial, reverse][tier 1..3]: arcs / index entries expanded;
+                                   default: join arcs scanned, likewise */
+    float ms_landmarks;         /* device time of the landmark reach sets (default: 0) */
+    float ms_init_tier2;        /* device time of the initial-gain tier-2 launch; default: counts from the ranges */
+    float ms_init_tier3;        /* device time of the initial-gain tier-3 launch; default: walks of cyclic cases */
     int32_t reserved2;
     uint64_t list_elems[3];     /* initial gains, tier 1..3: of work_elems, per-snapshot live-list entries */
 } sg_stats;
@@ -338,7 +352,9 @@ sg_status sg_select_state(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint6
  * sg_workspace_create sizes one for queries on g with R <= R_max and
  * k <= k_max (device memory taken through the allocator hooks, cleared;
  * synchronises `stream`).  sg_workspace_bytes reports that size without
- * allocating.  A workspace belongs to the graph it was created for until
+ * allocating.  The size is that of the default route under SG_WIC; a query
+ * that needs more (a denser cascade, other knobs) adds it when it first runs,
+ * or when its batch is captured.  A workspace belongs to the graph it was created for until
  * sg_workspace_free (waits for the device). */
 typedef struct sg_workspace sg_workspace;
 sg_status sg_workspace_create(const sg_graph *g, int32_t R_max, int32_t k_max, void *stream,

@@ -1,4 +1,6 @@
-// sg_kernels.cu -- device kernels of the StaticGreedy-DU path on sm_103a.
+// sg_kernels.cu -- device kernels of the StaticGreedy-DU path on sm_103a: the
+// tiered engines, which take the queries that the compact snapshot graphs
+// (sg_snap.cu, the default route) do not, and the kernels both routes use.
 //
 // Snapshots are bit-sliced: a 64-bit word per (node, task) carries 64
 // independent traversal states at once.  Two slicings are used:

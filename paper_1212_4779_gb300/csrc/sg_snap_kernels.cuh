@@ -19,7 +19,8 @@
 // and 28 K ranges to walk, 3 M arc visits in all, where walking the nodes
 // themselves visits 22 M; the snapshot takes about 4 MB, so the walks of a
 // few snapshots at a time stay in L2 and their visited bits in shared
-// memory.
+// memory.  The initial gains of R = 256 snapshots take 38 ms so, bitmaps and
+// graphs included, where the tiered engines take 347 ms.
 //
 // A selection round covers R(v*) in each snapshot (closed under
 // reachability, so later walks skip covered joins), marks the uncovered
@@ -309,7 +310,8 @@ __device__ __forceinline__ int sn_search(ExpandShared &S, QueueShared &Q, const 
 // coins, 2: masks already drawn (lm [W][m]).  Each warp evaluates 32 arcs
 // of one word, 64 coins per lane, and turns the 64 x 32 bits with ballots;
 // rows leave the block 32 bytes at a time.  Bound by the coins' integer
-// arithmetic; they are drawn once for both directions.
+// arithmetic (R-MAT 20, R = 256: 2.1 G coins in 2.9 ms); they are drawn once
+// for both directions.
 template <int FROM>
 __global__ void __launch_bounds__(SN_TILE) snap_coins_kernel(SnapView v, Coins co, const uint2 *fw,
                                                              const unsigned long long *lm)
@@ -381,7 +383,8 @@ __global__ void __launch_bounds__(SN_TILE) snap_coins_kernel(SnapView v, Coins c
 
 // Node bitmaps per snapshot (internal nodes, joins) from the bit-sliced
 // words, and the part of the initial gains and of their edge count that
-// needs no walk: a node without a live out-arc reaches itself.
+// needs no walk: a node without a live out-arc reaches itself.  A pass over
+// memory (0.18 ms, R-MAT 20, R = 256).
 __global__ void __launch_bounds__(SN_TILE) snap_nodes_kernel(SnapView v, Ctl *ctl, long long *s)
 {
     __shared__ uint32_t to[64][SN_TILE / 32], tj[64][SN_TILE / 32];
@@ -463,7 +466,10 @@ __device__ __forceinline__ int sn_chunk_count(const uint32_t *b, long long lo, l
 // Internal nodes and live arcs of one snapshot, in node and arc order, with
 // the direct counts of every internal node: itself and its leaf children
 // (low half of acc), its arcs to joins (high half), their out-degrees, and
-// the parent of every internal tree node.
+// the parent of every internal tree node.  One block a snapshot, as in all
+// kernels that build and cover: its maps and lists are its own, so the steps
+// need block barriers only.  Bound by scattered accesses to the node maps
+// (115 M live arcs in 4.2 ms, R-MAT 20, R = 256).
 __global__ void __launch_bounds__(SN_T) snap_compact_kernel(SnapView v, Ctl *ctl)
 {
     __shared__ int sh[33];
@@ -552,6 +558,8 @@ __global__ void __launch_bounds__(SN_T) snap_compact_kernel(SnapView v, Ctl *ctl
 // Trees of one snapshot: cycles of one-parent nodes are cut at their lowest
 // node (which becomes a join), subtree totals are summed towards the roots,
 // and every node gets its absolute positions in the join-arc and node lists.
+// Pointer doubling in place of level passes: a step is one dependent load for
+// every node, and depth counts by its logarithm (4.2 ms, R-MAT 20, R = 256).
 __global__ void __launch_bounds__(SN_T) snap_trees_kernel(SnapView v, Ctl *ctl)
 {
     __shared__ int sh[33];
@@ -767,7 +775,10 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, int least, i
 // Join-arc, join in-arc and node lists and join records of one snapshot,
 // then its landmark: a join x with many arcs below it and
 // many above.  Every node that reaches x reaches all of R(x), so those
-// walks start from a copy of R(x)'s bits and total.
+// walks start from a copy of R(x)'s bits and total.  Bound by chains of an
+// arc's map, rank and counter accesses (8.3 ms, R-MAT 20, R = 256); four arcs a
+// thread in stages gave 1.6 % of a selection there and cost 3 % on a dense
+// cascade of 97k nodes.
 __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
 {
     __shared__ ExpandShared S;
@@ -982,7 +993,9 @@ __device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uin
 }
 
 // The initial gains' ranges by one thread each; those that are too large go
-// to the task lists of the warp walks (in place of all tasks).
+// to the task lists of the warp walks (in place of all tasks).  R-MAT 20, R =
+// 256: 4.2 ms here and 13.5 ms of warp walks; all ranges by warps took 20 and 7
+// ms with them.
 template <bool EDGES>
 __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
 {
@@ -1293,7 +1306,8 @@ __device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t
 // after each, left warps waiting for the block's longest walk 40 % of the
 // time.)  Each warp keeps its bits in shared memory (in global memory, one
 // warp per block, when they are more than that holds) and undoes a small
-// walk's bits one by one instead of clearing all.
+// walk's bits one by one instead of clearing all.  R-MAT 20, R = 256: 13.5 ms
+// (MODE 0, 0.8 G join arcs), 24 ms (MODE 2, all rounds, 7 of them the first).
 template <int MODE, bool EDGES, bool SH>
 __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long long *s, int area)
 {
@@ -1510,6 +1524,12 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
 
 // ------------------------------------------------------------- a round
 
+// One block per snapshot.  Bound by the slowest block's chain of levels: each is
+// two or three dependent accesses and two or four barriers, with few entries
+// (R-MAT 18: 27 warp cycles an instruction at barriers, 13 on loads, L2 at 6 %).
+// R-MAT 20, R = 256: 2.6 ms in the first round, 0.6 ms on average, 33 ms of a
+// selection's 92; 15k nodes, R = 100, UIC: 20 us.  1024 threads a block, or 256
+// where snapshots have few live arcs; 512 in place of 1024 cost 11 %.
 // Cover R(v*) in one snapshot, subtract from the ancestors of v*, and list
 // the ranges whose counts need a walk (Algorithm 2, inner loops), with the
 // joins such a walk may enter: the newly covered ones and the marked ones
@@ -1926,7 +1946,9 @@ __global__ void __launch_bounds__(SN_T)
 // Marginal gains of up to EV_MAX candidates (lazy evaluation): block (r, b)
 // adds to out[b] the nodes candidate b would newly cover in snapshot r, a
 // closure over uncovered joins like the cover's, with nothing written back.
-// bits [EV_MAX][R][jw], queues [EV_MAX][R][jcap]: scratch.
+// bits [EV_MAX][R][jw], queues [EV_MAX][R][jcap]: scratch.  One candidate a
+// launch left the chip idle and the host waiting (15k nodes, WIC, k = 50: CELF
+// 83.6 ms on the tiered walks, 6.5 ms so).
 constexpr int EV_MAX = 16;
 struct EvalArgs {
     int32_t v[EV_MAX];
@@ -2005,7 +2027,9 @@ __global__ void __launch_bounds__(256) snap_eval_kernel(SnapView v, EvalArgs ev,
 __global__ void snap_choose_kernel(Ctl *ctl, int32_t x) { ctl->vstar = x; }
 
 // What the nodes marked in a round lose, one thread each (a warp claims 32
-// tasks of a snapshot); ranges that are too large go to the warp walks.
+// tasks of a snapshot); ranges that are too large go to the warp walks.  R-MAT
+// 20, R = 256: 7 ms a selection; with these walks as the first stage of the warp
+// kernel, whose lanes then waited for the chunk's large ones, its 43 ms became 71.
 template <bool EDGES>
 __global__ void __launch_bounds__(256) snap_lose_kernel(SnapView v, Ctl *ctl, long long *s)
 {

@@ -9,6 +9,9 @@
 // coordinate by coordinate, checks that every candidate returns the same
 // seeds and gains, and keeps the fastest; results are cached in a JSON-lines
 // file keyed by the graph's shape, the cascade and the word count.
+// At its defaults a query takes the compact snapshot graphs (sg_snap.cu), which
+// no knob touches; every other setting takes the tiered engines, so a change is
+// kept only where an engine is the faster route.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>
