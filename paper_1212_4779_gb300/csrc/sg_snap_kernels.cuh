@@ -776,7 +776,7 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, int least, i
 // then its landmark: a join x with many arcs below it and
 // many above.  Every node that reaches x reaches all of R(x), so those
 // walks start from a copy of R(x)'s bits and total.  Bound by chains of an
-// arc's map, rank and counter accesses (8.3 ms, R-MAT 20, R = 256); four arcs a
+// arc's map, rank and counter accesses (9 ms, R-MAT 20, R = 256); four arcs a
 // thread in stages gave 1.6 % of a selection there and cost 3 % on a dense
 // cascade of 97k nodes.
 __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
@@ -1307,7 +1307,7 @@ __device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t
 // time.)  Each warp keeps its bits in shared memory (in global memory, one
 // warp per block, when they are more than that holds) and undoes a small
 // walk's bits one by one instead of clearing all.  R-MAT 20, R = 256: 13.5 ms
-// (MODE 0, 0.8 G join arcs), 24 ms (MODE 2, all rounds, 7 of them the first).
+// (MODE 0, 0.8 G join arcs), 19 ms (MODE 2, all rounds, 7 of them the first).
 template <int MODE, bool EDGES, bool SH>
 __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long long *s, int area)
 {
@@ -1527,7 +1527,7 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
 // One block per snapshot.  Bound by the slowest block's chain of levels: each is
 // two or three dependent accesses and two or four barriers, with few entries
 // (R-MAT 18: 27 warp cycles an instruction at barriers, 13 on loads, L2 at 6 %).
-// R-MAT 20, R = 256: 2.6 ms in the first round, 0.6 ms on average, 33 ms of a
+// R-MAT 20, R = 256: 2.6 ms in the first round, 0.57 ms on average, 28 ms of a
 // selection's 92; 15k nodes, R = 100, UIC: 20 us.  1024 threads a block, or 256
 // where snapshots have few live arcs; 512 in place of 1024 cost 11 %.
 // Cover R(v*) in one snapshot, subtract from the ancestors of v*, and list
@@ -2028,7 +2028,7 @@ __global__ void snap_choose_kernel(Ctl *ctl, int32_t x) { ctl->vstar = x; }
 
 // What the nodes marked in a round lose, one thread each (a warp claims 32
 // tasks of a snapshot); ranges that are too large go to the warp walks.  R-MAT
-// 20, R = 256: 7 ms a selection; with these walks as the first stage of the warp
+// 20, R = 256: 6 ms a selection; with these walks as the first stage of the warp
 // kernel, whose lanes then waited for the chunk's large ones, its 43 ms became 71.
 template <bool EDGES>
 __global__ void __launch_bounds__(256) snap_lose_kernel(SnapView v, Ctl *ctl, long long *s)
