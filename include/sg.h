@@ -10,7 +10,7 @@
  *       hi32(splitmix64(seed ^ (r << 40) ^ e)) < thr(e),
  *     thr = floor(p * 2^32) (uniform cascade, UIC) or
  *     thr(u->v) = floor(2^32 / indeg(v)) (weighted cascade, WIC,
- *     p(u,v) = 1/d_v of Section 3.4.1); snapshots are never stored;
+ *     p(u,v) = 1/d_v of Section 3.4.1); no snapshot outlives its query;
  *   - initial gains s_v = sum_r |R(G'_r, v)| (Algorithm 2, first loop),
  *     where R(G'_r, v) includes v itself;
  *   - k rounds of: v* = argmax over non-seeds of s_v, lowest id on ties;

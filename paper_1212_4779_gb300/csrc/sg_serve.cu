@@ -284,11 +284,14 @@ int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fr
     if (!w) return -1;
     cudaStream_t st = s->setup_st;
     if (dense) w->snap_limit = 0;
-    bool fits = true;
+    // compact graphs that the device has no room for: wait for those running to
+    // end, then run on the engines
+    bool fits = snap;
     if (ensure_core(g, *w, W, s->cfg.k_cap, st) != SG_OK ||
-        (snap && (ensure_snap(g, *w, co, model, s->cfg.k_cap, st, &fits) != SG_OK || !fits)) ||
-        (!snap && !cc && ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK) ||
-        (!snap && !cc && heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
+        (snap && ensure_snap(g, *w, co, model, s->cfg.k_cap, st, &fits) != SG_OK) ||
+        (snap && !fits && s->running > 0) ||
+        (!fits && !cc && ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK) ||
+        (!fits && !cc && heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
         cudaEventRecord(s->setup_ev, st) != cudaSuccess) {
         free_workspace(*w, st);
         delete w;
