@@ -18,6 +18,7 @@ constexpr int SPREAD_HUB = 512;                     // ... and from which the wh
 constexpr int SPREAD_HUBS = 128;                    // such rows remembered per level
 constexpr size_t SPREAD_SMEM = (size_t)216 << 10;   // shared memory of one SM for visited bits ...
 constexpr size_t SPREAD_FIXED = 3200;               // ... and what a block takes beside them
+constexpr size_t SPREAD_DYNAMIC = SPREAD_SMEM - SPREAD_FIXED + 1024 * 4;  // most a launch asks for
 
 struct SpreadView {
     int32_t n, R, ns, words, none_live;
@@ -73,9 +74,10 @@ __device__ __forceinline__ void spread_arcs(const SpreadView &a, uint64_t s, con
 // snapshots draw 40 G coins (53 ms at the rate snap_coins_kernel draws them),
 // in 136 ms here against 319 ms bit-sliced, where most of the time went into
 // scattered records (R = 100: 1.2 against 155 ms, one block per word).  Bound
-// by issue (65 %), a third of it the coins.  A snapshot at a time keeps the whole visited set on the SM (128 KB for a million nodes)
-// and the arcs in L2; the bit-sliced walks it replaces kept 16 bytes a node
-// and word for all words in flight, 5 GB of scattered records.  A warp takes
+// by issue (65 %), a third of it the coins.  A snapshot at a time keeps the
+// whole visited set on the SM (128 KB for a million nodes) and the arcs in L2;
+// the bit-sliced walks it replaces kept 16 bytes a node and word for all words
+// in flight, 5 GB of scattered records.  A warp takes
 // 32 nodes of the level: their short rows spread over the lanes, a longer
 // one by the whole warp; hub rows wait for the next level, where all warps
 // share them (left to the warp that met them, the others waited two thirds
@@ -242,9 +244,11 @@ sg_status run_spread_snapshots(sg_graph *g, const Coins &co, int model, const in
     }
     a.queue = queue.p;
     a.next = next.p;
+    // The limit belongs to the kernel, not to the call: every call sets the same,
+    // so that none lowers it between another thread's set-up and launch.
     auto kern = model == MODEL_WIC ? spread_snapshots_kernel<MODEL_WIC> : spread_snapshots_kernel<MODEL_UIC>;
     if (cudaMemsetAsync(next.p, 0, 8, st) != cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SPREAD_DYNAMIC) != cudaSuccess) {
         set_error("sg_spread: launch set-up failed");
         rc = SG_ECUDA;
     } else {
