@@ -101,8 +101,10 @@ typedef struct {
  * sg_set_scc_condensation, sg_set_forward_lists, sg_set_snapshot_lists,
  * sg_set_mask_cache, sg_set_heavy_threshold, sg_tuning) are not all at their
  * defaults, graphs without arcs, and cascades whose compact graphs pass 64 GiB
- * or the memory there is.  Where a field means something else on the default
- * route, its comment names that after "default:". */
+ * or the memory there is.  A workspace whose compact graphs were refused memory
+ * asks again once the device has more of it free, and after 4 queries, then 8,
+ * 16, ... 64.  Where a field means something else on the default route, its
+ * comment names that after "default:". */
 typedef struct {
     uint64_t init_edges;
     uint64_t fwd_edges;

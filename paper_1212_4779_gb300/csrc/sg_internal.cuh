@@ -329,7 +329,12 @@ struct sg_workspace {
     int32_t wcap = 0;     // words of capacity of the [W][n] arrays
     int32_t core_w = 0;   // words of capacity of cov
     sgi::DBuf<unsigned char> snap;  // compact snapshot graphs, laid out per query
-    size_t snap_limit = SIZE_MAX;   // queries that need this much or more run on the tiered engines
+    // a size of them that the device had no room for (SIZE_MAX: none): queries
+    // that need as much run on the tiered engines until snap_ask has it asked
+    // for again; free device memory then, queries until and between askings
+    size_t snap_limit = SIZE_MAX, snap_free = 0;
+    int32_t snap_wait = 0, snap_gap = 0;
+    bool engines_only = false;      // never take the compact graphs
     int32_t nslots = 0;   // tier-3 (CTA engine) slots
     int32_t fq_groups = 0;    // forward-walk blocks per word the queues fq_a/fq_b were sized for
     int32_t walk_groups = 8;  // forward/landmark walk blocks per word for the current query

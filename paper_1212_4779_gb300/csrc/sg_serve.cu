@@ -257,7 +257,7 @@ int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fr
                            : (snap ? core + snap_bytes(g, co, model) : workspace_bytes(g, W, s->cfg.k_cap));
     for (size_t i = 0; i < s->pool.size(); ++i)
         if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W && s->pool[i].bytes >= need &&
-            (cc || dense == (s->pool[i].ws->snap_limit == 0)))
+            (cc || dense == s->pool[i].ws->engines_only))
             return (int)i;
     while (s->used + need > s->budget) {
         int lru = -1;
@@ -283,7 +283,7 @@ int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fr
     sg_workspace *w = new (std::nothrow) sg_workspace();
     if (!w) return -1;
     cudaStream_t st = s->setup_st;
-    if (dense) w->snap_limit = 0;
+    w->engines_only = dense;
     // compact graphs that the device has no room for: wait for those running to
     // end, then run on the engines
     bool fits = snap;

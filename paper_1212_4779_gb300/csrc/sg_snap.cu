@@ -177,25 +177,51 @@ sg_status build_arc_sources(sg_graph *g, cudaStream_t st)
     return SG_OK;
 }
 
+static size_t free_device_memory()
+{
+    size_t fr = 0, all = 0;
+    if (cudaMemGetInfo(&fr, &all) != cudaSuccess) cudaGetLastError();
+    return fr;
+}
+
+// Whether a size that was refused is asked for again: when the device has
+// clearly more room than it had then, else (memory behind the allocator hooks
+// does not show there) after 4 more queries, then 8, 16, ... 64, since a
+// refused request can be dear to whoever refuses it (a caching allocator gives
+// up its cache first).  A stream that is being captured takes the route its
+// query was sized for.
+static bool snap_ask(sg_workspace &ws, size_t need, cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs != cudaStreamCaptureStatusNone) return false;
+    if (free_device_memory() > ws.snap_free + need / 8) return true;
+    if (--ws.snap_wait > 0) return false;
+    return true;
+}
+
 // Sizes ws for a query on the compact graphs; *snap false, with nothing more
 // done, where it goes to the tiered engines: by snap_route, or because the
 // graphs do not fit into the device's memory (dense cascades: the engines'
-// arrays do not grow with the live arcs).  A workspace remembers the size that
-// did not fit, so that sizing ahead of a capture and recording take one route.
+// arrays do not grow with the live arcs).
 sg_status ensure_snap(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t k, cudaStream_t st,
                       bool *snap)
 {
     const size_t need = snap_bytes(g, co, model);
-    *snap = snap_route(g, co, model) && need < ws.snap_limit;
+    *snap = !ws.engines_only && snap_route(g, co, model) && (need < ws.snap_limit || snap_ask(ws, need, st));
     if (!*snap) return SG_OK;
     SG_TRY(ensure_core(g, ws, co.W, k, st));
-    if (ws.snap.bytes < need) {
-        dbuf_free(ws.snap, st);
-        if (dbuf_alloc(ws.snap, need, st) != SG_OK) {
-            clear_error();
-            ws.snap_limit = need;
-            *snap = false;
-        }
+    if (ws.snap.bytes >= need) return SG_OK;
+    dbuf_free(ws.snap, st);
+    if (dbuf_alloc(ws.snap, need, st) != SG_OK) {
+        clear_error();
+        ws.snap_gap = ws.snap_limit == SIZE_MAX ? 4 : std::min(64, 2 * ws.snap_gap);
+        ws.snap_wait = ws.snap_gap;
+        ws.snap_limit = need;
+        ws.snap_free = free_device_memory();
+        *snap = false;
+    } else if (need >= ws.snap_limit) {
+        ws.snap_limit = SIZE_MAX;
     }
     return SG_OK;
 }

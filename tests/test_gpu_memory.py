@@ -1,0 +1,87 @@
+"""Device memory that runs short or is shared: allocations refused for a while,
+scratch that does not fit, and a server whose requests take different routes.
+Results stay the oracle's; integers, so the tolerance is zero."""
+
+import time
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1212_4779_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sg():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1212_4779_gb300 import sg as _sg
+
+    return _sg
+
+
+class _Hooks:
+    """Allocator hooks that ask `refuse(bytes)` before every allocation."""
+
+    def __init__(self, sg, refuse):
+        self.sg, self.refuse, self.held, self.refused = sg, refuse, {}, []
+
+    def __enter__(self):
+        import torch
+
+        def alloc(nbytes, stream):
+            if self.refuse(nbytes):
+                self.refused.append(nbytes)
+                return None
+            t = torch.empty(max(1, nbytes), dtype=torch.uint8, device="cuda")
+            self.held[t.data_ptr()] = t
+            return t.data_ptr()
+
+        def release(ptr, nbytes, stream):
+            torch.cuda.synchronize()
+            self.held.pop(ptr, None)
+
+        self.sg.sg_set_allocator(alloc, release)
+        return self
+
+    def __exit__(self, *exc):
+        self.sg.sg_set_allocator(None, None)
+
+    def largest(self):
+        return max((t.numel() for t in self.held.values()), default=0)
+
+
+BIG = 128 << 20  # the compact graphs below take more, every array of the engines less
+
+
+def _same(res, ref):
+    assert np.array_equal(res.seeds, ref["seeds"]) and np.array_equal(res.gains, ref["gains"])
+
+
+def test_a_refused_allocation_is_asked_for_again(sg):
+    """One refusal sends a query to the engines; once there is room again, one
+    of the next few takes the compact graphs.  While there is none, they are
+    asked for now and then only."""
+    n, s, d = inputs.er_directed(2000, 20000, 6)
+    ref = oracle.Graph(n, s, d, "uic", 0.5).select(200, 4, 9, mode=oracle.COVER)
+    short = [True]
+    with _Hooks(sg, lambda b: short[0] and b > BIG) as h:
+        with sg.Graph.from_coo(n, s, d) as g:
+            _same(g.select(200, 4, "uic", 0.5, 9), ref)
+            assert len(h.refused) == 1 and h.largest() < BIG
+            short[0] = False
+            for _ in range(5):
+                _same(g.select(200, 4, "uic", 0.5, 9), ref)
+            assert h.largest() > BIG
+        short[0] = True
+        with sg.Graph.from_coo(n, s, d) as g:
+            del h.refused[:]
+            for _ in range(40):
+                _same(g.select(200, 4, "uic", 0.5, 9), ref)
+            assert 2 <= len(h.refused) <= 6
