@@ -70,6 +70,38 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     SG_TRY(check_lt_masks(g, co));
     bool snap = false;
     SG_TRY(ensure_snap(g, ws, co, model, k, st, &snap));
+
+    // scratch: an evaluation's own coverage (and queues), its counters, the source
+    DBuf<unsigned long long> scratch;
+    DBuf<long long> cnt;
+    DBuf<int32_t> dv;
+    struct BufGuard {
+        DBuf<unsigned long long> &a;
+        DBuf<long long> &b;
+        DBuf<int32_t> &c;
+        cudaStream_t st;
+        ~BufGuard()
+        {
+            dbuf_free(a, st);
+            dbuf_free(b, st);
+            dbuf_free(c, st);
+        }
+    } bufs{scratch, cnt, dv, st};
+    // candidates per evaluation launch: fewer where their scratch does not fit
+    // beside the graphs; without room for one the engines take the query
+    int32_t ahead = 1;
+    if (snap) {
+        ahead = snap_eval_count(g, co, model);
+        while (dbuf_alloc(scratch, (snap_eval_words(g, co, model, ahead) + 1) / 2, st) != SG_OK) {
+            clear_error();
+            if (ahead == 1) {
+                snap = false;
+                dbuf_free(ws.snap, st);
+                break;
+            }
+            ahead /= 2;
+        }
+    }
     // the linear threshold model reads every coin from the live-mask cache
     const int heavy_on = (!co.lt && heavy_index_enabled(g, co.W)) ? 1 : 0;
     if (!snap) {
@@ -119,24 +151,7 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     SG_CUDA_TRY(cudaStreamSynchronize(st));
     SG_TRY(flags_status(h.flags));
 
-    // scratch: the coverage copy of an evaluation, two counters, the source
-    DBuf<unsigned long long> scratch;
-    DBuf<long long> cnt;
-    DBuf<int32_t> dv;
-    struct BufGuard {
-        DBuf<unsigned long long> &a;
-        DBuf<long long> &b;
-        DBuf<int32_t> &c;
-        cudaStream_t st;
-        ~BufGuard()
-        {
-            dbuf_free(a, st);
-            dbuf_free(b, st);
-            dbuf_free(c, st);
-        }
-    } bufs{scratch, cnt, dv, st};
-    const int32_t ahead = snap ? snap_eval_count(g, co, model) : 1;  // candidates per evaluation launch
-    SG_TRY(dbuf_alloc(scratch, snap ? (snap_eval_words(g, co, model) + 1) / 2 : nw, st));
+    if (!snap) SG_TRY(dbuf_alloc(scratch, nw, st));
     SG_TRY(dbuf_alloc(cnt, (size_t)std::max(2, ahead), st));
     SG_TRY(dbuf_alloc(dv, 1, st));
 
@@ -171,7 +186,7 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
                         if (!known.count(next.back().v)) cand.push_back(next.back().v);
                     }
                     for (const CelfEntry &e : next) pq.push(e);
-                    SG_TRY(run_snap_eval(g, ws, co, model, cand.data(), (int32_t)cand.size(),
+                    SG_TRY(run_snap_eval(g, ws, co, model, cand.data(), (int32_t)cand.size(), ahead,
                                          reinterpret_cast<uint32_t *>(scratch.p),
                                          reinterpret_cast<unsigned long long *>(cnt.p), st));
                     SG_CUDA_TRY(cudaMemcpyAsync(vals.data(), cnt.p, cand.size() * 8, cudaMemcpyDeviceToHost, st));

@@ -306,23 +306,24 @@ int32_t snap_eval_count(const sg_graph *g, const Coins &co, int model)
     return (int32_t)std::max<size_t>(1, std::min<size_t>(EV_MAX, ((size_t)8 << 30) / each));
 }
 
-size_t snap_eval_words(const sg_graph *g, const Coins &co, int model)
+size_t snap_eval_words(const sg_graph *g, const Coins &co, int model, int32_t count)
 {
     SnapView v;
     carve(g, co, model, nullptr, v, nullptr, nullptr);
-    return (size_t)snap_eval_count(g, co, model) * v.R * ((size_t)v.jcap + v.jw);
+    return (size_t)count * v.R * ((size_t)v.jcap + v.jw);
 }
 
-// out[b] = marginal gain of cand[b], b < count (scratch: snap_eval_words).
+// out[b] = marginal gain of cand[b], b < count <= room (scratch: snap_eval_words
+// of room).
 sg_status run_snap_eval(sg_graph *g, sg_workspace &ws, const Coins &co, int model, const int32_t *cand, int32_t count,
-                        uint32_t *scratch, unsigned long long *out, cudaStream_t st)
+                        int32_t room, uint32_t *scratch, unsigned long long *out, cudaStream_t st)
 {
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
     EvalArgs ev{};
     for (int32_t b = 0; b < count; ++b) ev.v[b] = cand[b];
     ev.bits = scratch;
-    ev.queue = reinterpret_cast<int32_t *>(scratch + (size_t)snap_eval_count(g, co, model) * v.R * v.jw);
+    ev.queue = reinterpret_cast<int32_t *>(scratch + (size_t)room * v.R * v.jw);
     ev.out = out;
     SG_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)count * 8, st));
     snap_eval_kernel<<<dim3((unsigned)v.R, (unsigned)count), 256, 0, st>>>(v, ev, ws.cov.p);

@@ -85,3 +85,30 @@ def test_a_refused_allocation_is_asked_for_again(sg):
             for _ in range(40):
                 _same(g.select(200, 4, "uic", 0.5, 9), ref)
             assert 2 <= len(h.refused) <= 6
+
+
+@pytest.mark.parametrize("times", [1, 3, 5])
+def test_lazy_evaluation_with_little_scratch(sg, times):
+    """Scratch of the evaluations refused: fewer candidates a launch, and with
+    none left the engines."""
+    n, s, d = inputs.chung_lu_undirected(2000, 8000, 2.5, 8.0, 2)
+    ref = oracle.Graph(n, s, d, "wic").select(100, 12, 5, mode=oracle.CELF)
+    left = [0]
+
+    def refuse(nbytes):
+        if nbytes > BIG:
+            left[0] = times  # the arena was given; the next requests are the scratch
+            return False
+        if left[0] and nbytes > 1 << 19:
+            left[0] -= 1
+            return True
+        return False
+
+    with _Hooks(sg, refuse) as h:
+        with sg.Graph.from_coo(n, s, d) as g:
+            res, evals = g.select_celf(100, 12, "wic", 0.0, 5)
+            _same(res, ref)
+            assert evals == ref["evals"]
+            assert len(h.refused) == times and left[0] == 0
+            assert (h.largest() > BIG) == (times < 5)
+            _same(g.select(100, 12, "wic", 0.0, 5), ref)
