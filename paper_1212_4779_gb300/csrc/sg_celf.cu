@@ -23,6 +23,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "sg_celf_check.h"
 #include "sg_internal.cuh"
 
 using namespace sgi;
@@ -152,7 +153,9 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
     SG_TRY(flags_status(h.flags));
 
     if (!snap) SG_TRY(dbuf_alloc(scratch, nw, st));
-    SG_TRY(dbuf_alloc(cnt, (size_t)std::max(2, ahead), st));
+    // counters, then the pairs covered when each seed was chosen
+    const size_t counters = (size_t)std::max(2, ahead);
+    SG_TRY(dbuf_alloc(cnt, counters + (size_t)k, st));
     SG_TRY(dbuf_alloc(dv, 1, st));
 
     std::vector<CelfEntry> heap;
@@ -206,7 +209,7 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
         seeds[(size_t)i] = top.v;
         gains[(size_t)i] = top.bound;
         if (snap) {
-            SG_TRY(run_snap_cover(g, ws, co, model, top.v, st));
+            SG_TRY(run_snap_cover(g, ws, co, model, top.v, cnt.p + counters + i, st));
             continue;
         }
         SG_TRY(walk_from(g, ws, co, model, heavy_on, top.v, ws.cov.p, cnt.p, dv.p, hc, st));
@@ -225,11 +228,14 @@ sg_status celf_impl(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t se
         SG_CUDA_TRY(cudaMemcpyAsync(&hf, ws.ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         SG_CUDA_TRY(cudaStreamSynchronize(st));
         SG_TRY(flags_status(hf.flags));
-        long long covered = 0;
-        for (int64_t v : gains) covered += v;
-        if ((long long)hf.du_entries != covered) {
-            set_error("sg_select_celf: the seeds cover %lld pairs, their gains add to %lld", (long long)hf.du_entries,
-                      covered);
+        std::vector<long long> before((size_t)k);
+        SG_CUDA_TRY(cudaMemcpyAsync(before.data(), cnt.p + counters, (size_t)k * 8, cudaMemcpyDeviceToHost, st));
+        SG_CUDA_TRY(cudaStreamSynchronize(st));
+        const int32_t bad = celf_first_mismatch(before.data(), (long long)hf.du_entries, gains.data(), k);
+        if (bad >= 0) {
+            set_error("sg_select_celf: seed %d newly covers %lld, its gain was %lld", seeds[(size_t)bad],
+                      (bad + 1 < k ? before[(size_t)bad + 1] : (long long)hf.du_entries) - before[(size_t)bad],
+                      (long long)gains[(size_t)bad]);
             return SG_EINTERNAL;
         }
         fwd_edges = hf.fwd_edges;

@@ -516,7 +516,8 @@ int32_t snap_eval_count(const sg_graph *g, const Coins &co, int model);
 size_t snap_eval_words(const sg_graph *g, const Coins &co, int model, int32_t count);
 sg_status run_snap_eval(sg_graph *g, sg_workspace &ws, const Coins &co, int model, const int32_t *cand, int32_t count,
                         int32_t room, uint32_t *scratch, unsigned long long *out, cudaStream_t st);
-sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t x, cudaStream_t st);
+sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t x, long long *before,
+                         cudaStream_t st);
 sg_status run_snap_round(sg_graph *g, sg_workspace &ws, const Coins &co, int model, bool edges, int32_t round,
                          cudaStream_t st, cudaEvent_t after_cover);
 

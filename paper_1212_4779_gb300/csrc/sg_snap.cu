@@ -332,12 +332,14 @@ sg_status run_snap_eval(sg_graph *g, sg_workspace &ws, const Coins &co, int mode
     return SG_OK;
 }
 
-// Covers what x reaches (forward edges and newly covered pairs into ctl).
-sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t x, cudaStream_t st)
+// Covers what x reaches (forward edges and newly covered pairs into ctl);
+// *before: the pairs covered until then.
+sg_status run_snap_cover(sg_graph *g, sg_workspace &ws, const Coins &co, int model, int32_t x, long long *before,
+                         cudaStream_t st)
 {
     SnapView v;
     carve(g, co, model, ws.snap.p, v, nullptr, nullptr);
-    snap_choose_kernel<<<1, 1, 0, st>>>(ws.ctl.p, x);
+    snap_choose_kernel<<<1, 1, 0, st>>>(ws.ctl.p, x, before);
     snap_cover_kernel<true, false><<<v.R, snap_threads(v), 0, st>>>(v, ws.ctl.p, ws.s.p, ws.cov.p, 1);
     SG_CUDA_TRY(cudaGetLastError());
     g_launches += 2;

@@ -2024,7 +2024,11 @@ __global__ void __launch_bounds__(256) snap_eval_kernel(SnapView v, EvalArgs ev,
     if (tid == 0) atomicAdd(&ev.out[blockIdx.y], (unsigned long long)sum);
 }
 
-__global__ void snap_choose_kernel(Ctl *ctl, int32_t x) { ctl->vstar = x; }
+__global__ void snap_choose_kernel(Ctl *ctl, int32_t x, long long *before)
+{
+    ctl->vstar = x;
+    *before = (long long)ctl->du_entries;
+}
 
 // What the nodes marked in a round lose, one thread each (a warp claims 32
 // tasks of a snapshot); ranges that are too large go to the warp walks.  R-MAT
