@@ -150,13 +150,20 @@ struct SrvRequest {
     double t_submit = 0, t_done = 0;
     sg_status status = SG_OK;
     int state = 0;  // 0 queued, 1 running, 2 finished
+    bool engines = false;  // the device has no room for its compact graphs
     std::vector<int32_t> seeds;
     std::vector<int64_t> gains;
 };
 
+// What a workspace holds beside the arrays every query needs.  Each kind serves
+// requests of its own kind only: another's arrays would come on top, unseen by
+// the budget.
+enum SrvRoute { SRV_COMPACT, SRV_ENGINES, SRV_COMPONENTS };
+
 struct SrvWs {
     sg_graph *g;
     sg_workspace *ws;
+    SrvRoute route;
     int32_t W;
     size_t bytes;
     bool busy;
@@ -195,6 +202,7 @@ struct sg_server {
     int64_t next_id = 1;
     uint64_t tick = 0;
     int64_t running = 0, finished = 0;
+    bool starved = false;  // the device refused memory; no request has ended since
 };
 
 namespace {
@@ -225,7 +233,29 @@ void srv_retire(sg_server *s)
         sl.ws_index = -1;
         --s->running;
         ++s->finished;
+        s->starved = false;
     }
+}
+
+// Releases the least recently used idle workspace; false: none is idle.
+bool srv_evict(sg_server *s)
+{
+    int lru = -1;
+    for (size_t i = 0; i < s->pool.size(); ++i)
+        if (!s->pool[i].busy && (lru < 0 || s->pool[i].last_use < s->pool[(size_t)lru].last_use)) lru = (int)i;
+    if (lru < 0) return false;
+    // idle: its last request has finished (its slot event completed), so the
+    // release is queued in stream order without waiting
+    sg_workspace *w = s->pool[(size_t)lru].ws;
+    free_workspace(*w, s->setup_st);
+    delete w;
+    s->used -= s->pool[(size_t)lru].bytes;
+    s->pool.erase(s->pool.begin() + lru);
+    // running slots index the pool: entries after the erased one moved down
+    // (the erased entry was idle, so no slot held it)
+    for (auto &sl : s->slots)
+        if (sl.req && sl.ws_index > lru) --sl.ws_index;
+    return true;
 }
 
 // An idle workspace for a request, creating one within the memory budget
@@ -233,77 +263,79 @@ void srv_retire(sg_server *s)
 // *fresh: the workspace was created now; its set-up (allocations and
 // clears) is queued on the setup stream and marked by setup_ev.  Nothing
 // here waits on the host.
-int srv_workspace(sg_server *s, const SrvRequest *rq, bool *impossible, bool *fresh)
+int srv_workspace(sg_server *s, SrvRequest *rq, bool *impossible, bool *fresh)
 {
     *impossible = false;
     *fresh = false;
     sg_graph *g = rq->g;
-    const int32_t W = (rq->R + 63) / 64;
+    const int32_t W = (rq->R + 63) / 64, k = s->cfg.k_cap;
     const int model = rq->c.model == SG_WIC ? MODEL_WIC : MODEL_UIC;
     Coins co;
     if (make_coins(rq->c, rq->seed, rq->R, &co) != SG_OK) {
         *impossible = true;
         return -1;
     }
-    // the compact graphs' size depends on the cascade, the tiered engines'
-    // arrays only on the graph and W
-    const bool cc = rq->c.model == SG_UIC_UNDIRECTED;
-    bool snap = !cc && snap_route(g, co, model);
-    const size_t core = core_bytes(g, W, s->cfg.k_cap);
-    // a dense cascade whose compact graphs pass the budget runs on the engines
-    const bool dense = snap && core + snap_bytes(g, co, model) > s->budget;
-    if (dense) snap = false;
-    const size_t need = cc ? core + cc_workspace_bytes(g, rq->R)
-                           : (snap ? core + snap_bytes(g, co, model) : workspace_bytes(g, W, s->cfg.k_cap));
-    for (size_t i = 0; i < s->pool.size(); ++i)
-        if (!s->pool[i].busy && s->pool[i].g == g && s->pool[i].W >= W && s->pool[i].bytes >= need &&
-            (cc || dense == s->pool[i].ws->engines_only))
-            return (int)i;
-    while (s->used + need > s->budget) {
-        int lru = -1;
-        for (size_t i = 0; i < s->pool.size(); ++i)
-            if (!s->pool[i].busy && (lru < 0 || s->pool[i].last_use < s->pool[(size_t)lru].last_use)) lru = (int)i;
-        if (lru < 0) break;
-        // idle: its last request has finished (its slot event completed), so
-        // the release is queued in stream order without waiting
-        sg_workspace *w = s->pool[(size_t)lru].ws;
-        free_workspace(*w, s->setup_st);
-        delete w;
-        s->used -= s->pool[(size_t)lru].bytes;
-        s->pool.erase(s->pool.begin() + lru);
-        // running slots index the pool: entries after the erased one moved
-        // down (the erased entry was idle, so no slot held it)
-        for (auto &sl : s->slots)
-            if (sl.req && sl.ws_index > lru) --sl.ws_index;
-    }
-    if (s->used + need > s->budget) {
-        *impossible = s->running == 0;  // nothing will ever free memory
-        return -1;
-    }
-    sg_workspace *w = new (std::nothrow) sg_workspace();
-    if (!w) return -1;
-    cudaStream_t st = s->setup_st;
-    w->engines_only = dense;
-    // compact graphs that the device has no room for: wait for those running to
-    // end, then run on the engines
-    bool fits = snap;
-    if (ensure_core(g, *w, W, s->cfg.k_cap, st) != SG_OK ||
-        (snap && ensure_snap(g, *w, co, model, s->cfg.k_cap, st, &fits) != SG_OK) ||
-        (snap && !fits && s->running > 0) ||
-        (!fits && !cc && ensure_workspace(g, *w, W, s->cfg.k_cap, st) != SG_OK) ||
-        (!fits && !cc && heavy_index_enabled(g, W) && ensure_heavy_index(g, *w, W, st) != SG_OK) ||
-        cudaEventRecord(s->setup_ev, st) != cudaSuccess) {
+    const size_t core = core_bytes(g, W, k);
+    while (true) {
+        // the compact graphs' size depends on the cascade, the tiered engines'
+        // arrays only on the graph and W (and LT's masks); a cascade whose
+        // compact graphs pass the budget runs on the engines
+        SrvRoute route = SRV_ENGINES;
+        size_t need = 0, arena = 0;
+        if (rq->c.model == SG_UIC_UNDIRECTED) {
+            route = SRV_COMPONENTS;
+            need = core + cc_workspace_bytes(g, rq->R);
+        } else {
+            arena = snap_bytes(g, co, model);
+            if (!rq->engines && snap_route(g, co, model) && core + arena <= s->budget) route = SRV_COMPACT;
+            need = route == SRV_COMPACT ? core + arena : workspace_bytes(g, W, k);
+            if (route == SRV_ENGINES && co.lt && !g_mask_cache) need += mask_cache_bytes(g, W);
+        }
+        for (size_t i = 0; i < s->pool.size(); ++i) {
+            const SrvWs &e = s->pool[i];
+            if (!e.busy && e.g == g && e.route == route && e.W >= W &&
+                (route == SRV_COMPACT ? e.ws->snap.bytes >= arena : e.bytes >= need))
+                return (int)i;
+        }
+        while (s->used + need > s->budget && srv_evict(s)) {
+        }
+        if (s->used + need > s->budget) {
+            *impossible = s->running == 0;  // nothing will ever free memory
+            return -1;
+        }
+        sg_workspace *w = new (std::nothrow) sg_workspace();
+        if (!w) return -1;
+        cudaStream_t st = s->setup_st;
+        w->engines_only = route == SRV_ENGINES;
+        bool fits = true;
+        if (ensure_core(g, *w, W, k, st) == SG_OK &&
+            (route != SRV_COMPACT || (ensure_snap(g, *w, co, model, k, st, &fits) == SG_OK && fits)) &&
+            (route != SRV_ENGINES || (ensure_workspace(g, *w, W, k, st) == SG_OK &&
+                                      (!heavy_index_enabled(g, W) || ensure_heavy_index(g, *w, W, st) == SG_OK))) &&
+            cudaEventRecord(s->setup_ev, st) == cudaSuccess) {
+            *fresh = true;
+            w->owner_n = g->n;
+            w->device = g->device;
+            s->pool.push_back(SrvWs{g, w, route, W, need, false, ++s->tick});
+            s->used += need;
+            return (int)s->pool.size() - 1;
+        }
+        // The device has less room than the budget says: idle workspaces go
+        // first, then running requests end, then the engines take compact
+        // graphs' place.
         free_workspace(*w, st);
         delete w;
-        *impossible = s->running == 0;
-        return -1;
+        if (srv_evict(s)) continue;
+        if (s->running > 0) {
+            s->starved = true;
+            return -1;
+        }
+        if (route != SRV_COMPACT) {
+            *impossible = true;
+            return -1;
+        }
+        rq->engines = true;
     }
-    *fresh = true;
-    w->owner_n = g->n;
-    w->device = g->device;
-    s->pool.push_back(SrvWs{g, w, W, need, false, ++s->tick});
-    s->used += need;
-    return (int)s->pool.size() - 1;
 }
 
 // Admits queued requests in arrival order while a slot and memory allow.
@@ -320,6 +352,7 @@ void srv_admit(sg_server *s, std::unique_lock<std::mutex> &lock)
                 break;
             }
         if (!free_slot) return;
+        if (s->starved && s->running > 0) return;  // asking again before a request ends is in vain
         SrvRequest *r = s->queue.front();
         bool impossible = false, fresh = false;
         const int wi = srv_workspace(s, r, &impossible, &fresh);

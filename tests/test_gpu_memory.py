@@ -112,3 +112,54 @@ def test_lazy_evaluation_with_little_scratch(sg, times):
             assert len(h.refused) == times and left[0] == 0
             assert (h.largest() > BIG) == (times < 5)
             _same(g.select(100, 12, "wic", 0.0, 5), ref)
+
+
+def _serve(sg, sv, requests, together):
+    """Results of the requests, all submitted at once or one after another."""
+    out, ids = [], []
+    end = time.time() + 120
+
+    def wait(rid, k):
+        while time.time() < end:
+            done, seeds, gains, _ = sg.sg_server_poll(sv, rid, k)
+            if done:
+                return sg.Selection(seeds, gains, None)
+            time.sleep(0.002)
+        raise AssertionError("the server did not answer")
+
+    for q in requests:
+        ids.append((sg.sg_server_submit(sv, *q), q[2]))
+        if not together:
+            out.append(wait(*ids.pop()))
+    return out + [wait(*i) for i in ids]
+
+
+@pytest.mark.parametrize("together", [False, True])
+def test_server_memory_over_mixed_routes(sg, together):
+    """Undirected, compact and dense requests on one graph: what they hold
+    together stays within the budget, in every order."""
+    import torch
+
+    n, s, d = inputs.symmetric(*inputs.er_directed(20000, 60000, 3))
+    cases = [("uic_undirected", 0.05, 2000, 6), ("wic", 0.0, 32, 6), ("uic", 0.1, 64, 6)]
+    refs = {}
+    for model, p, R, k in cases:
+        mode = oracle.COVER if model == "uic_undirected" else oracle.DU
+        refs[model] = oracle.Graph(n, s, d, model, p).select(R, k, 13, mode=mode)
+    budget = 800 << 20
+    g = sg.Graph.from_coo(n, s, d)
+    # what stays with the graph after its first undirected query
+    g.select(1, 1, "uic_undirected", 0.05, 13)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    sv = sg.sg_server_create(3, budget, 64)
+    try:
+        order = [cases[i] for i in (0, 1, 2, 1, 0, 2, 0, 1)]
+        got = _serve(sg, sv, [(g.handle, R, k, model, p, 13) for model, p, R, k in order], together)
+        for (model, *_), res in zip(order, got):
+            _same(res, refs[model])
+        torch.cuda.synchronize()
+        assert free - torch.cuda.mem_get_info()[0] <= budget + (96 << 20)
+    finally:
+        sg.sg_server_destroy(sv)
+        g.close()
