@@ -353,10 +353,12 @@ sg_status sg_select_state(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint6
  * graph at the same time only with workspaces of their own.
  * sg_workspace_create sizes one for queries on g with R <= R_max and
  * k <= k_max (device memory taken through the allocator hooks, cleared;
- * synchronises `stream`).  sg_workspace_bytes reports that size without
- * allocating.  The size is that of the default route under SG_WIC; a query
- * that needs more (a denser cascade, other knobs) adds it when it first runs,
- * or when its batch is captured.  A workspace belongs to the graph it was created for until
+ * synchronises `stream`).  The size is that of the default route under SG_WIC
+ * (of the tiered engines where that is their query); a query that needs more (a
+ * denser cascade, other knobs) adds it when it first runs, or when its batch is
+ * captured.  sg_workspace_bytes reports, without allocating, an upper bound of
+ * that size: the larger of the two routes, since the engines take over where
+ * the default route's memory is refused.  A workspace belongs to the graph it was created for until
  * sg_workspace_free (waits for the device). */
 typedef struct sg_workspace sg_workspace;
 sg_status sg_workspace_create(const sg_graph *g, int32_t R_max, int32_t k_max, void *stream,

@@ -1407,11 +1407,12 @@ sg_status sg_workspace_bytes(const sg_graph *g, int32_t R_max, int32_t k_max, si
         set_error("R_max must satisfy 1 <= R_max < 2^24");
         return SG_EINVAL;
     }
-    // enough for either route
+    // enough for either route: the compact graphs may be refused memory
     const int32_t W = (R_max + 63) / 64;
     Coins co;
     SG_TRY(make_coins(sg_cascade{SG_WIC, 0.0}, 0, R_max, &co));
-    *bytes = std::max(workspace_bytes(g, W, k_max), core_bytes(g, W, k_max) + snap_bytes(g, co, MODEL_WIC));
+    *bytes = workspace_bytes(g, W, k_max);
+    if (snap_route(g, co, MODEL_WIC)) *bytes = std::max(*bytes, core_bytes(g, W, k_max) + snap_bytes(g, co, MODEL_WIC));
     return SG_OK;
 }
 

@@ -148,8 +148,12 @@ __global__ void __launch_bounds__(256) arc_sources_kernel(int n, const int32_t *
 // The compact snapshot graphs serve every directed cascade and LT.  The
 // tiered engines remain for the calls that set one of their knobs (whoever
 // asks for a tier, a landmark count or a cache gets it), for graphs without
-// arcs, and where the graphs would pass SNAP_BYTES_MAX (dense cascades on
-// large graphs: about 100 bytes per live arc and snapshot).
+// arcs, and where the graphs would pass SNAP_BYTES_MAX.  Per place reserved, a
+// snapshot takes 28 bytes for a live arc, 88 for an internal node, 52 for a join
+// and 8 for a tree node, and nodes and joins have as many places as live arcs
+// have, up to n.  Under WIC and LT that is 184 to 200 bytes per live arc (R-MAT
+// 20, R = 256: 21 GiB; a weighted R-MAT 22 passes the limit near R = 175); where
+// the live arcs far outnumber the nodes it comes near 28.
 bool snap_route(const sg_graph *g, const Coins &co, int model)
 {
     const Knobs k = knobs();

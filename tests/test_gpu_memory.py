@@ -163,3 +163,19 @@ def test_server_memory_over_mixed_routes(sg, together):
     finally:
         sg.sg_server_destroy(sv)
         g.close()
+
+
+def test_workspace_bytes_cover_the_workspace(sg):
+    """sg_workspace_bytes is no less than what sg_workspace_create takes, and
+    leaves out compact graphs of a size that is never built (64 GiB)."""
+    n, s, d = inputs.er_directed(3000, 12000, 4)
+    with _Hooks(sg, lambda b: False) as h:
+        with sg.Graph.from_coo(n, s, d) as g:
+            for R in (1, 64, 200, 1000):
+                before = sum(t.numel() for t in h.held.values())
+                ws = sg.sg_workspace_create(g.handle, R, 10)
+                assert sum(t.numel() for t in h.held.values()) - before <= sg.sg_workspace_bytes(g.handle, R, 10)
+                sg.sg_workspace_free(ws)
+            # 190 bytes per place, 3,000 places a snapshot: past 64 GiB from R = 120,000 on
+            small, large = (sg.sg_workspace_bytes(g.handle, R, 10) for R in (64 * 1500, 64 * 3000))
+            assert small < 64 << 30 and large < 64 << 30
