@@ -419,8 +419,9 @@ sg_status sg_set_tuning(const sg_tuning *t);
  * faster.  *out receives the tuning and *out_ms (may be NULL) its time per
  * selection.  With cache_path (may be NULL) a JSON-lines file is read
  * first -- a line whose key (node and arc counts, largest out-degree,
- * model, UIC probability, word count) matches is returned without timing --
- * and a new result is appended.  The process-wide knobs are not changed:
+ * model, UIC probability, word count, revision of the routes it was timed on)
+ * matches is returned without timing -- and a new result is appended, unless
+ * the default route was refused memory while it was timed.  The process-wide knobs are not changed:
  * pass *out to sg_set_tuning, or put it in sg_query.tuning.  The graph's
  * own workspace is released and sized again (its queues for 64 walk
  * groups).  Synchronises `stream`; takes about 20 selections' time.

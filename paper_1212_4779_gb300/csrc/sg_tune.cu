@@ -73,8 +73,13 @@ sg_tuning from_knobs(const Knobs &k)
     return t;
 }
 
+// What a cached line's times were measured on.  Raised when a route changes that
+// the knobs choose between: a line from before the compact graphs would send its
+// query to the engines untimed.
+constexpr int TUNING_REVISION = 2;
+
 // Cache key: the graph's shape (nodes, arcs, largest out-degree), the
-// cascade (model, UIC probability) and the 64-snapshot word count.
+// cascade (model, UIC probability), the 64-snapshot word count and the revision.
 sg_status tuning_key(sg_graph *g, const sg_cascade &c, int32_t W, cudaStream_t st, std::string *out)
 {
     std::vector<int32_t> rp((size_t)g->n + 1);
@@ -83,8 +88,8 @@ sg_status tuning_key(sg_graph *g, const sg_cascade &c, int32_t W, cudaStream_t s
     int32_t dmax = 0;
     for (int64_t v = 0; v < g->n; ++v) dmax = std::max(dmax, rp[(size_t)v + 1] - rp[(size_t)v]);
     char buf[256];
-    snprintf(buf, sizeof buf, "n=%lld m=%lld dmax=%d model=%d p=%.6f W=%d", (long long)g->n, (long long)g->m, dmax,
-             (int)c.model, c.model == SG_WIC ? 0.0 : c.p, (int)W);
+    snprintf(buf, sizeof buf, "n=%lld m=%lld dmax=%d model=%d p=%.6f W=%d rev=%d", (long long)g->n, (long long)g->m, dmax,
+             (int)c.model, c.model == SG_WIC ? 0.0 : c.p, (int)W, TUNING_REVISION);
     *out = buf;
     return SG_OK;
 }
@@ -276,6 +281,8 @@ sg_status sg_autotune(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t 
         rc = SG_ECUDA;
     }
     if (rc == SG_OK) rc = time_knobs(T, best, &best_ms);
+    // compact graphs refused memory: the times say nothing about other days
+    bool refused = g->ws.snap_limit != SIZE_MAX;
     // coordinate descent: each knob over its candidates, others held
     auto try_values = [&](auto setter, const std::vector<int> &vals) {
         for (int v : vals) {
@@ -310,7 +317,8 @@ sg_status sg_autotune(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t 
     if (rc != SG_OK) return rc;
     *out = from_knobs(best);
     if (out_ms) *out_ms = best_ms;
-    if (cache_path) cache_store(cache_path, key, *out, best_ms);
+    refused |= g->ws.snap_limit != SIZE_MAX;
+    if (cache_path && !refused) cache_store(cache_path, key, *out, best_ms);
     return SG_OK;
 }
 
