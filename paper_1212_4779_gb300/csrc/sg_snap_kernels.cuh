@@ -52,6 +52,8 @@ constexpr int SW_ARCS = 96;     // ... and arcs it may scan
 constexpr int SW_U = 4;         // ... several at a time
 constexpr int WK_U = 4;         // arcs in flight per lane
 constexpr int ROUND_ONE = 2;    // tasks per chunk from which a round walks with single threads first
+constexpr int LMK_LONG = 64;    // in-arcs of a join from which warps share their sum ...
+constexpr int LMK_CHUNK = 2048; // ... this many a warp
 constexpr int ROUND_LMK = 512;  // newly covered joins from which a round has a landmark
 constexpr uint32_t CV_CYCLE = 0x80000000u;
 constexpr uint32_t ARC_LEAF = 0x80000000u;  // jarc: the join has no live out-arc (weight 1, nothing below)
@@ -778,13 +780,15 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, int least, i
 // walks start from a copy of R(x)'s bits and total.  Bound by chains of an
 // arc's map, rank and counter accesses (9 ms, R-MAT 20, R = 256); four arcs a
 // thread in stages gave 1.6 % of a selection there and cost 3 % on a dense
-// cascade of 97k nodes.
-__global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
+// cascade of 97k nodes.  32 registers, so that two blocks share an SM (48 took
+// that cascade from 10.5 to 10.7 ms).
+__global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
 {
     __shared__ ExpandShared S;
     __shared__ QueueShared Q;
     __shared__ unsigned long long best;
     __shared__ unsigned int lc, ld;
+    __shared__ int nlong;
     chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
     SnapInfo *info = v.info + r;
@@ -871,17 +875,53 @@ __global__ void __launch_bounds__(SN_T) snap_place_kernel(SnapView v)
         up[i] = p >= 0 ? make_int2(~p, 1) : (j >= 0 ? make_int2(inoff[j], inoff[j + 1] - inoff[j]) : make_int2(0, 0));
     }
     if (tid == 0) ld = 0;
-    // landmark: join arcs below times in-arcs up to two steps above
-    for (int c = tid; c < C; c += T) {
-        const int w = rec[c].w;
-        if (w < 2) continue;
-        unsigned long long up = 0;
-        for (int k = inoff[c]; k < inoff[c + 1]; ++k) {
-            const int j = v.jid[io + ~sn_hi(pj[jin[k].x])];
-            up += 1ull + (j >= 0 ? (unsigned long long)(inoff[j + 1] - inoff[j]) : 0ull);
-        }
-        const unsigned long long sc = min(up * (unsigned long long)w, (1ull << 31) - 1ull);
+    // landmark: join arcs below times in-arcs up to two steps above.  A join
+    // with many in-arcs is left to the warps: with one thread each, the 200,000
+    // in-arcs of one join took 33 ms.
+    auto above2 = [&](int k) -> unsigned long long {
+        const int j = v.jid[io + ~sn_hi(pj[jin[k].x])];
+        return 1ull + (j >= 0 ? (unsigned long long)(inoff[j + 1] - inoff[j]) : 0ull);
+    };
+    auto score = [&](int c, unsigned long long up) {
+        const unsigned long long sc = min(up * (unsigned long long)rec[c].w, (1ull << 31) - 1ull);
         atomicMax(&best, (sc << 32) | (uint32_t)c);
+    };
+    unsigned long long *sums = reinterpret_cast<unsigned long long *>(Q.range);  // of the joins in S.aux
+    if (tid == 0) nlong = 0;
+    __syncthreads();
+    for (int c = tid; c < C; c += T) {
+        if (rec[c].w < 2) continue;
+        if (inoff[c + 1] - inoff[c] > LMK_LONG) {
+            const int q = atomicAdd(&nlong, 1);
+            if (q < SN_T) {
+                S.aux[q] = c;
+                sums[q] = 0;
+                continue;
+            }
+        }
+        unsigned long long up = 0;
+        for (int k = inoff[c]; k < inoff[c + 1]; ++k) up += above2(k);
+        score(c, up);
+    }
+    __syncthreads();
+    {
+        const int nl = min(nlong, SN_T), nw = T >> 5;
+        int before = 0;  // chunks of the joins before this one
+        for (int q = 0; q < nl; ++q) {
+            const int c = S.aux[q], k0 = inoff[c], k1 = inoff[c + 1];
+            const int chunks = (k1 - k0 + LMK_CHUNK - 1) / LMK_CHUNK;
+            for (int h = (wid + nw - before % nw) % nw; h < chunks; h += nw) {
+                const int end = min(k1 - k0, (h + 1) * LMK_CHUNK);
+                unsigned long long up = 0;
+                for (int k = h * LMK_CHUNK + lane; k < end; k += 32) up += above2(k0 + k);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) up += __shfl_xor_sync(SN_FULL, up, o);
+                if (lane == 0) atomicAdd(&sums[q], up);
+            }
+            before += chunks;
+        }
+        __syncthreads();
+        for (int q = tid; q < nl; q += T) score(S.aux[q], sums[q]);
     }
     __syncthreads();
     const int x = best ? (int)(uint32_t)best : -1;
