@@ -288,8 +288,8 @@ sg_status sg_select_celf(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64
  * count, the out-degree sum over the reached (node, snapshot) pairs.
  * A multi-source walk with the coins hashed in registers (no per-query
  * cache is used): one snapshot per block at a time with a visited bit per
- * node in shared memory; bit-sliced, one 64-snapshot word per block, for LT
- * and for graphs of more than 1.7 million nodes.  S: host or
+ * node in shared memory; bit-sliced, one 64-snapshot word per block, for LT,
+ * for graphs of more than 1.7 million nodes and for R > 800 sqrt(n).  S: host or
  * device int32[s_count]; out_total: host or device int64; out_edges: host.
  * Synchronises `stream` before returning; uses up to ~8 GiB of scratch.
  * Errors: SG_EINVAL for a NULL graph/output, s_count < 0, a seed outside

@@ -205,10 +205,21 @@ __global__ void __launch_bounds__(1024) spread_snapshots_kernel(SpreadView a)
 
 }  // namespace
 
+// LT draws per node, not per arc; above 1.7 M nodes the bits do not fit.  A
+// snapshot takes a block a few microseconds however little it reaches, so many
+// snapshots of a small graph go faster 64 at a time.  Six cascades (mean live
+// degree 0.1 to 2.5) from 1, 10 and 100 seeds on uniform and power-law graphs,
+// bit-sliced time over this one's, geometric means:
+//       R =      4,000  20,000  100,000
+//   n =    200    1.26    0.85     0.57
+//   n =  1,000    1.64    1.06     0.75
+//   n =  4,000    2.17    1.28     0.92
+//   n = 16,000    2.74    1.52     1.14
+// so the line lies at R = 800 sqrt(n).
 bool spread_by_snapshot(const sg_graph *g, const Coins &co)
 {
-    // LT draws per node, not per arc; above 1.7 M nodes the bits do not fit
-    return !co.lt && ((size_t)g->n + 127) / 128 * 16 + SPREAD_FIXED <= SPREAD_SMEM;
+    return !co.lt && ((size_t)g->n + 127) / 128 * 16 + SPREAD_FIXED <= SPREAD_SMEM &&
+           (double)co.R * co.R <= 640000.0 * (double)g->n;
 }
 
 sg_status run_spread_snapshots(sg_graph *g, const Coins &co, int model, const int32_t *d_S, int32_t ns,
