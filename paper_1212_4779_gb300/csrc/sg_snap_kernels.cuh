@@ -1583,7 +1583,7 @@ __global__ void __launch_bounds__(SN_T)
 {
     __shared__ ExpandShared S;
     __shared__ QueueShared Q;
-    __shared__ int nnew, tnew, nt0, nt1, last, pleaf;
+    __shared__ int nnew, tnew, nt0, nt1, last, pleaf, around;
     __shared__ unsigned int lw;
     __shared__ unsigned long long best;
     chain_start();
@@ -1621,6 +1621,7 @@ __global__ void __launch_bounds__(SN_T)
         nt0 = 0;
         nt1 = 0;
         pleaf = -1;
+        around = 0;
         lw = 0;
         best = 0;
     }
@@ -1685,6 +1686,77 @@ __global__ void __launch_bounds__(SN_T)
             }
         }
         const int na = DU ? sn_search(S, Q, qi, 0, above, mark_up) : 0;
+        // The round's landmark: the newly covered join with the most arcs
+        // below times in-arcs from uncovered non-ancestors, two steps up.  Where
+        // it lies on a cycle, the nodes above it are looked for before any is
+        // marked as covered, since the way up leads through newly covered ones:
+        // v* may lie above a large component that others reach at joins of their
+        // own (R-MAT 18, p = 0.2, R = 64: a million walks of 36,000 joins each in
+        // round one otherwise).  Elsewhere the few more nodes found so are not
+        // worth the longer way (R-MAT 20, WIC: 2 % of a selection).
+        int nu = na, nl = 0, lj = -1;
+        auto climb = [&]() {
+            if (tid == 0) Q.tail = na;
+            __syncthreads();
+            for (int k = inoff[lj] + tid; k < inoff[lj + 1]; k += T) mark(jin[k].x);
+            nu = sn_search(S, Q, qi, na, above, mark_arc);
+        };
+        if (DU && nd >= ROUND_LMK) {
+            for (int i = tid; i < cw; i += T) lmr[i] = 0;
+            for (int q = tid; q < nd; q += T) qr[q] = 0;
+            __syncthreads();
+            sn_expand_n(
+                S, 0, nd,
+                [&](int q, int &first, int &len) {
+                    const int j = ql[q];
+                    if (rec[j].w < 2) return;
+                    first = inoff[j];
+                    len = inoff[j + 1] - first;
+                },
+                [&](const auto &q, const auto &k) {
+                    constexpr int U = sizeof(q) / sizeof(int);
+                    int i[U], rj[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) i[u] = q[u] >= 0 ? jin[k[u]].x : -1;
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (i[u] >= 0) rj[u] = sn_bit(mk, i[u]) ? -2 : ~sn_hi(v.pj[io + i[u]]);
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (i[u] >= 0 && rj[u] != -2) rj[u] = jid[rj[u]];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (i[u] < 0 || rj[u] == -2 || (rj[u] >= 0 && sn_bit(rel, rj[u]))) continue;
+                        atomicAdd(&qr[q[u]], 1 + (rj[u] >= 0 ? inoff[rj[u] + 1] - inoff[rj[u]] : 0));
+                    }
+                });
+            for (int q = tid; q < nd; q += T) {
+                const unsigned long long a = (unsigned long long)(uint32_t)qr[q];
+                if (a)
+                    atomicMax(&best, (min(a * (unsigned long long)rec[ql[q]].w, (1ull << 31) - 1ull) << 32) |
+                                         (uint32_t)ql[q]);
+            }
+            __syncthreads();
+            lj = best ? (int)(uint32_t)best : -1;
+            if (lj >= 0) {
+                if (tid == 0) {
+                    Q.tail = 0;
+                    lmr[lj >> 5] = 1u << (lj & 31);
+                    sn_push(Q, qr, lj, below(lj));
+                }
+                nl = sn_search(S, Q, qr, 0, below, [&](int k) {
+                    const uint32_t a = jarc[k];
+                    const int j = (int)(a & ~ARC_LEAF);
+                    const uint32_t bit = 1u << (j & 31);
+                    const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
+                    if (!(rel[j >> 5] & bit)) return;  // covered before
+                    if (j == lj) around = 1;
+                    if (!(atomicOr(&lmr[j >> 5], bit) & bit)) sn_push(Q, qr, j, e);
+                });
+                for (int q = tid; q < nl; q += T) atomicAdd(&lw, (unsigned)rec[qr[q]].x);
+                if (around) climb();
+            }
+        }
         // newly covered nodes: the trees of those joins and T(v*)
         // (a node stands once in a list, so its bit is looked up before it is
         // set and the loads of EX_U nodes go out together)
@@ -1767,67 +1839,7 @@ __global__ void __launch_bounds__(SN_T)
             const int j = jid[~sn_hi(v.pj[io + pleaf])];
             if (j >= 0 && !sn_bit(covj, j)) v.rec[jo + j].x -= tnew;
         }
-        // The round's landmark: the newly covered join with the most arcs
-        // below times in-arcs from uncovered non-ancestors, two steps up.
-        int nu = na, nl = 0;
-        if (DU && nd >= ROUND_LMK) {
-            for (int i = tid; i < cw; i += T) lmr[i] = 0;
-            for (int q = tid; q < nd; q += T) qr[q] = 0;
-            __syncthreads();
-            sn_expand_n(
-                S, 0, nd,
-                [&](int q, int &first, int &len) {
-                    const int j = ql[q];
-                    if (rec[j].w < 2) return;
-                    first = inoff[j];
-                    len = inoff[j + 1] - first;
-                },
-                [&](const auto &q, const auto &k) {
-                    constexpr int U = sizeof(q) / sizeof(int);
-                    int i[U], rj[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) i[u] = q[u] >= 0 ? jin[k[u]].x : -1;
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (i[u] >= 0) rj[u] = sn_bit(mk, i[u]) ? -2 : ~sn_hi(v.pj[io + i[u]]);
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (i[u] >= 0 && rj[u] != -2) rj[u] = jid[rj[u]];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (i[u] < 0 || rj[u] == -2) continue;
-                        atomicAdd(&qr[q[u]], 1 + (rj[u] >= 0 ? inoff[rj[u] + 1] - inoff[rj[u]] : 0));
-                    }
-                });
-            for (int q = tid; q < nd; q += T) {
-                const unsigned long long a = (unsigned long long)(uint32_t)qr[q];
-                if (a)
-                    atomicMax(&best, (min(a * (unsigned long long)rec[ql[q]].w, (1ull << 31) - 1ull) << 32) |
-                                         (uint32_t)ql[q]);
-            }
-            __syncthreads();
-            const int lj = best ? (int)(uint32_t)best : -1;
-            if (lj >= 0) {
-                if (tid == 0) {
-                    Q.tail = 0;
-                    lmr[lj >> 5] = 1u << (lj & 31);
-                    sn_push(Q, qr, lj, below(lj));
-                }
-                nl = sn_search(S, Q, qr, 0, below, [&](int k) {
-                    const uint32_t a = jarc[k];
-                    const int j = (int)(a & ~ARC_LEAF);
-                    const uint32_t bit = 1u << (j & 31);
-                    const int2 e = a & ARC_LEAF ? make_int2(0, 0) : below(j);
-                    if (!(rel[j >> 5] & bit)) return;  // covered before
-                    if (!(atomicOr(&lmr[j >> 5], bit) & bit)) sn_push(Q, qr, j, e);
-                });
-                for (int q = tid; q < nl; q += T) atomicAdd(&lw, (unsigned)rec[qr[q]].x);
-                if (tid == 0) Q.tail = na;
-                __syncthreads();
-                for (int k = inoff[lj] + tid; k < inoff[lj + 1]; k += T) mark(jin[k].x);
-                nu = sn_search(S, Q, qi, na, above, mark_arc);
-            }
-        }
+        if (DU && lj >= 0 && !around) climb();
         int ni = 0;
         if (DU) {
             if (tid == 0) Q.tail = nu;
@@ -1844,7 +1856,9 @@ __global__ void __launch_bounds__(SN_T)
         }
         // their ranges are tasks, the joins among them relevant too
         int32_t *task = v.task + io;
+        auto newly = [&](int q) { return q < nu && sn_bit(covi, qi[q]); };  // above the landmark, covered itself
         for (int q = na + tid; q < ni; q += T) {
+            if (newly(q)) continue;
             const int i = qi[q];
             const int j = jid[i];
             if (j >= 0) atomicOr(&rel[j >> 5], 1u << (j & 31));
@@ -1897,6 +1911,7 @@ __global__ void __launch_bounds__(SN_T)
                 rrec[rank2(rel2, j)] = make_int4(covered ? e.x : 0, 0, a.x, a.y);
             };
             for (int q = na + tid; q < ni; q += T) {
+                if (newly(q)) continue;
                 const int i = qi[q], j = jid[i];
                 if (j >= 0) record(j, false);
                 if (v.share[io + i] < 0) rrange[i] = range2((int)sn_lo(v.pj[io + i]), sn_hi(v.acc[io + i]));
@@ -1904,7 +1919,7 @@ __global__ void __launch_bounds__(SN_T)
             sn_expand_n(
                 S, 0, nd + ni - na,
                 [&](int q, int &first, int &len) {
-                    const int j = q < nd ? ql[q] : jid[qi[na + q - nd]];
+                    const int j = q < nd ? ql[q] : newly(na + q - nd) ? -1 : jid[qi[na + q - nd]];
                     if (j < 0) return;
                     if (q < nd) record(j, true);
                     S.aux[tid] = rank2(rel2, j);
