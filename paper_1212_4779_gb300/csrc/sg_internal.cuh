@@ -258,6 +258,8 @@ struct Ctl {
     long long du_total;   // reverse tasks of the current round
 };
 
+constexpr int SN_LMK = 32;  // most landmarks of a snapshot's initial gains
+
 // One snapshot's compact graph (sg_snap_kernels.cuh).
 struct SnapInfo {
     int32_t nI;        // internal nodes: a live out-arc
@@ -267,7 +269,8 @@ struct SnapInfo {
     int32_t N;         // nodes of the trees under internal roots
     int32_t t0, t1;    // closure tasks, from the front / back of the task list
     int32_t f0, f1;    // initial gains: sources that need a walk of their own, likewise
-    int32_t lmk_cnt, lmk_deg;  // nodes the landmark reaches, their out-degree sum
+    int32_t marks;     // landmarks of the initial gains
+    int32_t lmk_cnt, lmk_deg;  // nodes the first (or the round's) landmark reaches, their out-degree sum
     int32_t nrel;      // relevant joins of the round
     int32_t bad;       // the snapshot has more live arcs than reserved
 };
@@ -288,13 +291,15 @@ struct SnapView {
     int32_t *outp, *joinp;                  // ... and set bits before each word
     SnapInfo *info;
     int2 *arc;                              // [R][cap] live arcs in CSR order: (internal source, destination)
-    int32_t *inode, *par, *pend, *share, *jid;  // [R][icap] node id, tree parent, scratch, child with the
+    int32_t *inode, *par, *pend, *share, *jid;  // [R][icap] node id, tree parent, scratch (then landmark), child with the
                                                 // same join range, join id
     uint32_t *deg, *cnt;                    // [R][icap] out-degree sum of T(v); current marginal count
     unsigned long long *acc;                // [R][icap] (arcs from T(v) to joins, |T(v)|)
     unsigned long long *pj, *pn;            // [R][icap] (~root, first position in jarc) / (~root, ... in tn)
     int2 *up;                               // [R][icap] what lies above: (first, count) in jin, or (~parent, 1)
-    int2 *rrange;                           // [R][icap] a round's tasks: (first, count) in rarc
+    int2 *rrange;                           // [R][icap] a round's tasks: (first, count) in rarc; before the rounds:
+    uint32_t *lmi;                          // [R][SN_LMK][jw] what the initial gains' landmarks but the first reach
+    int2 *lmt;                              // [R][SN_LMK] their nodes and out-degree sums
     unsigned long long *cv;                 // [R][icap] closure totals of a walked range
     int32_t *task, *fb, *ilist;             // [R][icap]
     int4 *rec;                              // [R][jcap] join: |T|, out-degree sum, first join arc, join arcs
@@ -307,7 +312,7 @@ struct SnapView {
     int2 *tn;                               // [R][tcap] nodes of the trees, T(v) contiguous: (node, internal or -1)
     uint32_t *covi, *marki;                 // [R][iw] covered / marked internal nodes
     uint32_t *covj, *rel;                   // [R][jw] covered joins, a round's relevant ones
-    uint32_t *lmr, *lmc;                    // [R][jw] landmark's reach, the same by rank among the relevant
+    uint32_t *lmr, *lmc;                    // [R][jw] (first) landmark's reach, the same by rank among the relevant
     uint2 *rel2;                            // [R][jw] word of rel, set bits before it
     int4 *rrec;                             // [R][jcap] relevant joins by rank: weight, -, first arc, arcs
     uint32_t *rarc;                         // [R][cap] arcs to relevant joins, in jarc's order, by rank

@@ -102,7 +102,9 @@ size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base,
     c.take(v.pj, ri);
     c.take(v.pn, ri);
     c.take(v.up, ri);
-    c.take(v.rrange, ri);
+    // the rounds' ranges lie where the initial gains' landmarks were
+    c.take(v.rrange, std::max(ri, (R * SN_LMK * v.jw + 1) / 2));
+    v.lmi = reinterpret_cast<uint32_t *>(v.rrange);
     c.take(v.cv, ri);
     c.take(v.task, ri);
     c.take(v.fb, ri);
@@ -128,6 +130,7 @@ size_t carve(const sg_graph *g, const Coins &co, int model, unsigned char *base,
     c.take(v.cstart, 2 * R + 4);
     c.take(v.wq, wb * WK_W * WK_QG);
     c.take(v.gbm, wb * v.jw);
+    c.take(v.lmt, R * SN_LMK);
     unsigned long long *masks = nullptr;
     if (co.lt) c.take(masks, (size_t)g->m * co.W);
     if (lm) *lm = masks;

@@ -54,6 +54,8 @@ constexpr int WK_U = 4;         // arcs in flight per lane
 constexpr int ROUND_ONE = 2;    // tasks per chunk from which a round walks with single threads first
 constexpr int LMK_LONG = 64;    // in-arcs of a join from which warps share their sum ...
 constexpr int LMK_CHUNK = 2048; // ... this many a warp
+constexpr int LMK_MORE = 512;  // joins of a landmark's component from which another landmark is looked for ...
+constexpr int LMK_FAR = 64;    // ... with at least this part of the first one's score
 constexpr int ROUND_LMK = 512;  // newly covered joins from which a round has a landmark
 constexpr uint32_t CV_CYCLE = 0x80000000u;
 constexpr uint32_t ARC_LEAF = 0x80000000u;  // jarc: the join has no live out-arc (weight 1, nothing below)
@@ -775,9 +777,9 @@ __device__ __forceinline__ void sn_plan(const SnapView &v, int *sh, int least, i
 }
 
 // Join-arc, join in-arc and node lists and join records of one snapshot,
-// then its landmark: a join x with many arcs below it and
-// many above.  Every node that reaches x reaches all of R(x), so those
-// walks start from a copy of R(x)'s bits and total.  Bound by chains of an
+// then its landmarks: joins x with many arcs below and many above.  Every
+// node that reaches x reaches all of R(x), so those walks start from a copy of
+// R(x)'s bits and total.  Bound by chains of an
 // arc's map, rank and counter accesses (9 ms, R-MAT 20, R = 256); four arcs a
 // thread in stages gave 1.6 % of a selection there and cost 3 % on a dense
 // cascade of 97k nodes.  32 registers, so that two blocks share an SM (48 took
@@ -788,7 +790,7 @@ __global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
     __shared__ QueueShared Q;
     __shared__ unsigned long long best;
     __shared__ unsigned int lc, ld;
-    __shared__ int nlong;
+    __shared__ int nlong, inside;
     chain_start();
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = blockDim.x;
     SnapInfo *info = v.info + r;
@@ -874,23 +876,27 @@ __global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
         const int p = v.par[io + i], j = v.jid[io + i];
         up[i] = p >= 0 ? make_int2(~p, 1) : (j >= 0 ? make_int2(inoff[j], inoff[j + 1] - inoff[j]) : make_int2(0, 0));
     }
-    if (tid == 0) ld = 0;
-    // landmark: join arcs below times in-arcs up to two steps above.  A join
+    // landmarks: join arcs below times in-arcs up to two steps above.  A join
     // with many in-arcs is left to the warps: with one thread each, the 200,000
     // in-arcs of one join took 33 ms.
     auto above2 = [&](int k) -> unsigned long long {
         const int j = v.jid[io + ~sn_hi(pj[jin[k].x])];
         return 1ull + (j >= 0 ? (unsigned long long)(inoff[j + 1] - inoff[j]) : 0ull);
     };
+    int32_t *scores = v.fb + io;
     auto score = [&](int c, unsigned long long up) {
         const unsigned long long sc = min(up * (unsigned long long)rec[c].w, (1ull << 31) - 1ull);
+        if (C >= LMK_MORE) scores[c] = (int)sc;
         atomicMax(&best, (sc << 32) | (uint32_t)c);
     };
     unsigned long long *sums = reinterpret_cast<unsigned long long *>(Q.range);  // of the joins in S.aux
     if (tid == 0) nlong = 0;
     __syncthreads();
     for (int c = tid; c < C; c += T) {
-        if (rec[c].w < 2) continue;
+        if (rec[c].w < 2) {
+            if (C >= LMK_MORE) scores[c] = 0;
+            continue;
+        }
         if (inoff[c + 1] - inoff[c] > LMK_LONG) {
             const int q = atomicAdd(&nlong, 1);
             if (q < SN_T) {
@@ -924,14 +930,38 @@ __global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
         for (int q = tid; q < nl; q += T) score(S.aux[q], sums[q]);
     }
     __syncthreads();
-    const int x = best ? (int)(uint32_t)best : -1;
+    // Several large components need a landmark each: while the last one lies in
+    // a component of many joins, the join with the best score among those that
+    // reach none so far is the next.  A node's landmark is the first it reaches.
+    const unsigned long long first = best >> 32;
     const int cw = (C + 31) >> 5, iw = (nI + 31) >> 5;
-    uint32_t *lr = v.lmr + (size_t)r * v.jw, *lu = v.marki + (size_t)r * v.iw;
+    uint32_t *lu = v.marki + (size_t)r * v.iw;
     int32_t *ql = v.jlist + jo, *qi = v.ilist + io;
-    for (int i = tid; i < cw; i += T) lr[i] = 0;
     for (int i = tid; i < iw; i += T) lu[i] = 0;
-    __syncthreads();
-    if (x >= 0) {
+    int from = 0, marks = 0;  // nodes above the landmarks before this one; landmarks
+    for (int l = 0; l < SN_LMK; ++l) {
+        if (l > 0) {
+            __syncthreads();
+            if (tid == 0) best = 0;
+            __syncthreads();
+            for (int c = tid; c < C; c += T) {
+                const unsigned long long sc = (unsigned long long)scores[c];
+                if (sc * LMK_FAR < first || sn_bit(lu, sn_rank(outb, outp, v.jnode[jo + c]))) continue;
+                atomicMax(&best, (sc << 32) | (uint32_t)c);
+            }
+            __syncthreads();
+        }
+        if (!best) break;
+        const int x = (int)(uint32_t)best;
+        uint32_t *lr = l ? v.lmi + ((size_t)r * SN_LMK + l) * v.jw : v.lmr + (size_t)r * v.jw;
+        for (int i = tid; i < cw; i += T) lr[i] = 0;
+        if (tid == 0) {
+            lc = 0;
+            ld = 0;
+            inside = 0;
+            Q.tail = 0;
+        }
+        __syncthreads();
         auto below = [&](int j) {
             const int4 e = rec[j];
             return make_int2(e.z, e.w);
@@ -952,17 +982,36 @@ __global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
             atomicAdd(&lc, (unsigned)e.x);
             atomicAdd(&ld, (unsigned)e.y);
         }
-        if (tid == 0) Q.tail = 0;
+        if (tid == 0) Q.tail = from;
         __syncthreads();
         // U(x): internal nodes that reach x
         auto mark = [&](int i) { mark_path(Q, up, lu, qi, i); };
         for (int k = inoff[x] + tid; k < inoff[x + 1]; k += T) mark(jin[k].x);
-        sn_search(S, Q, qi, 0, [&](int i) { return joins_above(up[i]); }, [&](int k) { mark(jin[k].x); });
+        const int to = sn_search(S, Q, qi, from, [&](int i) { return joins_above(up[i]); }, [&](int k) { mark(jin[k].x); });
+        if (tid == 0) {
+            if (l) {
+                v.lmt[(size_t)r * SN_LMK + l] = make_int2((int)lc, (int)ld);
+            } else {
+                info->lmk_cnt = (int)lc;
+                info->lmk_deg = (int)ld;
+            }
+            S.aux[l] = to;
+        }
+        ++marks;
+        if (to - from < LMK_MORE) break;
+        for (int q = from + tid; q < to; q += T) {
+            const int j = v.jid[io + qi[q]];
+            if (j >= 0 && sn_bit(lr, j)) atomicAdd(&inside, 1);
+        }
+        from = to;
+        __syncthreads();
+        if (inside < LMK_MORE) break;
     }
-    __syncthreads();
-    if (tid == 0) {
-        info->lmk_cnt = (int)lc;
-        info->lmk_deg = (int)ld;
+    if (tid == 0) info->marks = marks;
+    if (marks > 1) {
+        __syncthreads();
+        for (int l = 0; l < marks; ++l)
+            for (int q = (l ? S.aux[l - 1] : 0) + tid; q < S.aux[l]; q += T) v.pend[io + qi[q]] = l;
     }
 }
 
@@ -1032,6 +1081,32 @@ __device__ __forceinline__ bool small_walk(uint32_t *list, int stride, const uin
     }
 }
 
+// What snapshot r's landmark l reaches, and its totals (count, out-degrees).
+__device__ __forceinline__ uint32_t *snap_reach(const SnapView &v, int r, int l)
+{
+    return l ? v.lmi + ((size_t)r * SN_LMK + l) * v.jw : v.lmr + (size_t)r * v.jw;
+}
+__device__ __forceinline__ int2 snap_total(const SnapView &v, int r, int l)
+{
+    return l ? v.lmt[(size_t)r * SN_LMK + l] : make_int2(v.info[r].lmk_cnt, v.info[r].lmk_deg);
+}
+
+// Internal node i's landmark in the initial gains: the bits of what it reaches
+// (NULL: none) and its totals.  lu: nodes that have one, pend: which, with
+// several (one more dependent load for every walk otherwise).
+__device__ __forceinline__ const uint32_t *snap_landmark(const SnapView &v, int r, int i, const uint32_t *lu, size_t io,
+                                                         bool several, unsigned int &cnt, unsigned int &deg)
+{
+    cnt = 0;
+    deg = 0;
+    if (!sn_bit(lu, i)) return nullptr;
+    const int l = several ? v.pend[io + i] : 0;
+    const int2 t = snap_total(v, r, l);
+    cnt = (unsigned)t.x;
+    deg = (unsigned)t.y;
+    return snap_reach(v, r, l);
+}
+
 // The initial gains' ranges by one thread each; those that are too large go
 // to the task lists of the warp walks (in place of all tasks).  R-MAT 20, R =
 // 256: 4.2 ms here and 13.5 ms of warp walks; all ranges by warps took 20 and 7
@@ -1050,18 +1125,19 @@ __global__ void __launch_bounds__(256) snap_small_kernel(SnapView v)
         SnapInfo *info = v.info + r;
         const int nI = info->nI;
         const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
-        const uint32_t *lu = v.marki + (size_t)r * v.iw, *lmr = v.lmr + (size_t)r * v.jw;
+        const uint32_t *lu = v.marki + (size_t)r * v.iw;
+        const bool several = info->marks > 1;
         for (int i = part * 256 + tid; i < nI; i += per * 256) {
             const int wd = sn_hi(v.acc[io + i]);
             if (wd < 2 || v.share[io + i] >= 0) continue;
             const unsigned long long pj = v.pj[io + i];
-            const bool l = sn_bit(lu, i);
-            unsigned int c = l ? (unsigned)info->lmk_cnt : 0u, d = l ? (unsigned)info->lmk_deg : 0u;
+            unsigned int c = 0, d = 0;
+            const uint32_t *l = snap_landmark(v, r, i, lu, io, several, c, d);
             int n;
-            if (small_walk<EDGES>(&list[0][tid], 256, v.jarc + (size_t)r * v.cap, v.rec + jo, l ? lmr : nullptr,
-                                  (int)sn_lo(pj), wd, c, d, n)) {
+            if (small_walk<EDGES>(&list[0][tid], 256, v.jarc + (size_t)r * v.cap, v.rec + jo, l, (int)sn_lo(pj), wd, c,
+                                  d, n)) {
                 const int rj = v.jid[io + ~sn_hi(pj)];
-                bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
+                bool cyc = rj >= 0 && l && sn_bit(l, rj);
                 for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
                 v.cv[io + i] = sn_pack((int)(c | (cyc ? CV_CYCLE : 0u)), d);
             } else if (l) {
@@ -1360,7 +1436,7 @@ __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long lon
     w.gvis = v.gbm + (size_t)blockIdx.x * v.jw;
     w.qg = v.wq + ((size_t)blockIdx.x * WK_W + wid) * WK_QG;
     int q = -1, qbeg = 0, qend = 0;  // (snapshot, segment) at hand: its base is in vis
-    int cnt = 0, lcnt = 0, ldeg = 0;
+    int cnt = 0, lcnt = 0, ldeg = 0, mark = -1;
     size_t io = 0;
     const uint32_t *base = nullptr;
     const int32_t *list = nullptr;
@@ -1377,18 +1453,19 @@ __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long lon
             const int r = q >> 1, seg = q & 1;
             const SnapInfo *in = v.info + r;
             cnt = MODE == 0 || all ? (seg ? in->t1 : in->t0) : (seg ? in->f1 : in->f0);
-            lcnt = seg ? in->lmk_cnt : 0;
-            ldeg = seg ? in->lmk_deg : 0;
+            lcnt = seg && ROUND ? in->lmk_cnt : 0;
+            ldeg = 0;
+            mark = -1;
             io = (size_t)r * v.icap;
             w.count = ROUND ? in->nrel : in->C;
             w.jarc = (ROUND ? v.rarc : v.jarc) + (size_t)r * v.cap;
             w.rec = (ROUND ? v.rrec : v.rec) + (size_t)r * v.jcap;
-            base = seg ? (ROUND ? v.lmc : v.lmr) + (size_t)r * v.jw : nullptr;
+            base = seg && ROUND ? v.lmc + (size_t)r * v.jw : nullptr;
             list = (MODE == 0 || all ? v.task : (MODE == 1 ? v.fb : v.ilist)) + io;
-            w.load(base, lane);
+            if (ROUND || !seg) w.load(base, lane);
         }
         const int k0 = (ch - qbeg) * per, nk = min(cnt - k0, per);
-        int ti = 0, tp = 0, tw = 0, tr = 0;  // the chunk's tasks, one per lane
+        int ti = 0, tp = 0, tw = 0, tr = 0, tl = 0;  // the chunk's tasks, one per lane
         if (lane < nk) {
             ti = list[(q & 1) ? v.icap - 1 - (k0 + lane) : k0 + lane];
             if (ROUND) {
@@ -1400,9 +1477,21 @@ __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long lon
                 tp = (int)sn_lo(pj);
                 tw = sn_hi(v.acc[io + ti]);
                 tr = v.jid[io + ~sn_hi(pj)];
+                if ((q & 1) && v.info[q >> 1].marks > 1) tl = v.pend[io + ti];
             }
         }
         for (int k = 0; k < nk; ++k) {
+            if (!ROUND && (q & 1)) {
+                const int l = __shfl_sync(SN_FULL, tl, k);
+                if (l != mark) {  // another landmark than the last task's
+                    mark = l;
+                    const int2 t = snap_total(v, q >> 1, l);
+                    lcnt = t.x;
+                    ldeg = t.y;
+                    base = snap_reach(v, q >> 1, l);
+                    w.load(base, lane);
+                }
+            }
             const int i = __shfl_sync(SN_FULL, ti, k), rj = __shfl_sync(SN_FULL, tr, k);
             w.template range<EDGES && !ROUND>(__shfl_sync(SN_FULL, tp, k), __shfl_sync(SN_FULL, tw, k), base, lane);
             unsigned int c = w.cnt, d = w.deg;
@@ -1459,9 +1548,10 @@ __global__ void __launch_bounds__(WK_T, 2) snap_walk_kernel(SnapView v, Ctl *ctl
 // is followed to the join's own closure.  Where that closure runs through a
 // cycle (so that it might hold the node's own tree) the node gets a walk of
 // its own, by this thread or, when too large, by a warp (list fb, planned
-// for MODE 1 by the last block).
+// for MODE 1 by the last block).  Bound by loads in flight: five blocks an SM
+// (four, 57 registers: LT on 60k nodes 146 -> 198 us).
 template <bool EDGES>
-__global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl, long long *s)
+__global__ void __launch_bounds__(256, EDGES ? 4 : 5) snap_resolve_kernel(SnapView v, Ctl *ctl, long long *s)
 {
     __shared__ uint32_t list[SW_CAP][256];
     __shared__ int sh[33];
@@ -1476,7 +1566,7 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
         const int nI = info->nI;
         const size_t io = (size_t)r * v.icap, jo = (size_t)r * v.jcap;
         const uint32_t *jarc = v.jarc + (size_t)r * v.cap;
-        const uint32_t *lu = v.marki + (size_t)r * v.iw, *lmr = v.lmr + (size_t)r * v.jw;
+        const uint32_t *lu = v.marki + (size_t)r * v.iw;
         const uint32_t *outb = v.outb + (size_t)r * v.n32;
         const int32_t *outp = v.outp + (size_t)r * v.n32;
         for (int i = part * 256 + tid; i < nI; i += per * 256) {
@@ -1520,14 +1610,11 @@ __global__ void __launch_bounds__(256) snap_resolve_kernel(SnapView v, Ctl *ctl,
             }
             if (walk) {
                 const unsigned long long pj = v.pj[io + i];
-                const bool l = sn_bit(lu, i);
-                c = l ? (unsigned)info->lmk_cnt : 0u;
-                d = l ? (unsigned)info->lmk_deg : 0u;
+                const uint32_t *l = snap_landmark(v, r, i, lu, io, info->marks > 1, c, d);
                 int n;
-                if (small_walk<EDGES>(&list[0][tid], 256, jarc, v.rec + jo, l ? lmr : nullptr, (int)sn_lo(pj),
-                                      sn_hi(a), c, d, n)) {
+                if (small_walk<EDGES>(&list[0][tid], 256, jarc, v.rec + jo, l, (int)sn_lo(pj), sn_hi(a), c, d, n)) {
                     const int rj = v.jid[io + ~sn_hi(pj)];
-                    bool cyc = rj >= 0 && l && sn_bit(lmr, rj);
+                    bool cyc = rj >= 0 && l && sn_bit(l, rj);
                     for (int k = 0; k < n; ++k) cyc |= (int)(list[k][tid] & ~ARC_LEAF) == rj;
                     if (!cyc) {
                         c += sn_lo(a);

@@ -58,3 +58,26 @@ def test_a_round_over_a_component(sg, p, R):
     reaches (16,000 arcs a walk otherwise, 24 M a snapshot)."""
     work = _check(sg, _component_under_sources(2000, 16000, 1500, 1800), p, R, 4)
     assert sum(work[1]) < 1000000 * R, work
+
+
+def _components(count, n, m):
+    """`count` random digraphs of n nodes, each below a node of its own."""
+    s, d = [], []
+    for c in range(count):
+        _, a, b = inputs.er_directed(n, m, 20 + c)
+        at = c * (n + 1)
+        s += [a + at, [at + n]]
+        d += [b + at, [at + c % n]]
+    return count * (n + 1), np.concatenate(s).astype(np.int32), np.concatenate(d).astype(np.int32)
+
+
+@pytest.mark.parametrize("count,n,p,R,bound", [
+    (1, 700, 1.0, 2, 2000), (2, 700, 1.0, 65, 4000), (3, 1200, 0.9, 64, 100000),
+    (32, 600, 1.0, 1, 200000), (34, 600, 1.0, 3, 14000000),  # more than there are landmarks: two walk in full
+    (5, 400, 1.0, 3, 20000000),                              # components below the size that calls for another
+])
+def test_gains_over_several_components(sg, count, n, p, R, bound):
+    """Every large component has a landmark: a node's walk starts from what the
+    landmark reaches (8 n arcs for each of the n nodes otherwise)."""
+    work = _check(sg, _components(count, n, 8 * n), p, R, 3)
+    assert sum(work[0]) < bound * R, work
