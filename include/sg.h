@@ -273,8 +273,9 @@ sg_status sg_set_mask_cache(int32_t enable);
  * is queued again.  *out_evals (may be NULL) receives the number of such
  * evaluations (the initial gains not counted).  Outputs as sg_select (host
  * or device); stats (may be NULL): init and forward snapshot-edge counts
- * (reverse 0), ms_init, ms_rounds, ms_total.  Synchronises `stream` once per
- * evaluation and per round (not capturable).  Uses the graph's default
+ * (reverse 0), ms_init, ms_rounds, ms_total; work_keys and work_elems leave
+ * the evaluations out.  Synchronises `stream` once per evaluation and per round
+ * (default: once per launch of up to 16 evaluations; not capturable).  Uses the graph's default
  * workspace, like sg_select.  Errors: as sg_select. */
 sg_status sg_select_celf(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t seed, void *stream,
                          int32_t *out_seeds, int64_t *out_gains, int64_t *out_evals, sg_stats *stats);
@@ -421,10 +422,10 @@ sg_status sg_set_tuning(const sg_tuning *t);
  * first -- a line whose key (node and arc counts, largest out-degree,
  * model, UIC probability, word count, revision of the routes it was timed on)
  * matches is returned without timing -- and a new result is appended, unless
- * the default route was refused memory while it was timed.  The process-wide knobs are not changed:
- * pass *out to sg_set_tuning, or put it in sg_query.tuning.  The graph's
- * own workspace is released and sized again (its queues for 64 walk
- * groups).  Synchronises `stream`; takes about 20 selections' time.
+ * the default route was refused memory while it was timed.  The process-wide
+ * knobs are not changed: pass *out to sg_set_tuning, or put it in
+ * sg_query.tuning.  The graph's own workspace is released and sized again (its
+ * queues for 64 walk groups).  Synchronises `stream`; takes about 20 selections' time.
  * Errors: as sg_select; SG_EINTERNAL if two settings gave different
  * results. */
 sg_status sg_autotune(sg_graph *g, int32_t R, int32_t k, sg_cascade c, uint64_t seed, void *stream,

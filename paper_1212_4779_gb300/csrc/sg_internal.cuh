@@ -98,7 +98,7 @@ void clear_error();
 // has passed chain_next or is done: late, so that waiting blocks do not hold
 // the places of another stream's kernels.  15k nodes, R = 100, k = 50, UIC:
 // 2.20 -> 1.93 ms; with chain_next as the second statement 1.98 ms, but
-// requests on four streams took 129 ms in place of 113.
+// requests on eight streams took 129 ms in place of 113.
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -291,8 +291,8 @@ struct SnapView {
     int32_t *outp, *joinp;                  // ... and set bits before each word
     SnapInfo *info;
     int2 *arc;                              // [R][cap] live arcs in CSR order: (internal source, destination)
-    int32_t *inode, *par, *pend, *share, *jid;  // [R][icap] node id, tree parent, scratch (then landmark), child with the
-                                                // same join range, join id
+    int32_t *inode, *par, *pend, *share, *jid;  // [R][icap] node id, tree parent, scratch (then which landmark),
+                                                // child with the same join range, join id
     uint32_t *deg, *cnt;                    // [R][icap] out-degree sum of T(v); current marginal count
     unsigned long long *acc;                // [R][icap] (arcs from T(v) to joins, |T(v)|)
     unsigned long long *pj, *pn;            // [R][icap] (~root, first position in jarc) / (~root, ... in tn)

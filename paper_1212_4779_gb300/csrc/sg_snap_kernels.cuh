@@ -987,7 +987,8 @@ __global__ void __launch_bounds__(SN_T, 2) snap_place_kernel(SnapView v)
         // U(x): internal nodes that reach x
         auto mark = [&](int i) { mark_path(Q, up, lu, qi, i); };
         for (int k = inoff[x] + tid; k < inoff[x + 1]; k += T) mark(jin[k].x);
-        const int to = sn_search(S, Q, qi, from, [&](int i) { return joins_above(up[i]); }, [&](int k) { mark(jin[k].x); });
+        auto above = [&](int i) { return joins_above(up[i]); };
+        const int to = sn_search(S, Q, qi, from, above, [&](int k) { mark(jin[k].x); });
         if (tid == 0) {
             if (l) {
                 v.lmt[(size_t)r * SN_LMK + l] = make_int2((int)lc, (int)ld);

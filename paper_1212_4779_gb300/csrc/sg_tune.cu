@@ -88,8 +88,8 @@ sg_status tuning_key(sg_graph *g, const sg_cascade &c, int32_t W, cudaStream_t s
     int32_t dmax = 0;
     for (int64_t v = 0; v < g->n; ++v) dmax = std::max(dmax, rp[(size_t)v + 1] - rp[(size_t)v]);
     char buf[256];
-    snprintf(buf, sizeof buf, "n=%lld m=%lld dmax=%d model=%d p=%.6f W=%d rev=%d", (long long)g->n, (long long)g->m, dmax,
-             (int)c.model, c.model == SG_WIC ? 0.0 : c.p, (int)W, TUNING_REVISION);
+    snprintf(buf, sizeof buf, "n=%lld m=%lld dmax=%d model=%d p=%.6f W=%d rev=%d", (long long)g->n, (long long)g->m,
+             dmax, (int)c.model, c.model == SG_WIC ? 0.0 : c.p, (int)W, TUNING_REVISION);
     *out = buf;
     return SG_OK;
 }
