@@ -1927,7 +1927,20 @@ __global__ void __launch_bounds__(SN_T)
             const int j = jid[~sn_hi(v.pj[io + pleaf])];
             if (j >= 0 && !sn_bit(covj, j)) v.rec[jo + j].x -= tnew;
         }
-        if (DU && lj >= 0 && !around) climb();
+        int32_t *task = v.task + io;
+        if (DU && lj >= 0) {
+            if (!around) {
+                climb();
+            } else {  // covered nodes leave the list
+                for (int q = na + tid; q < nu; q += T)
+                    if (!sn_bit(covi, qi[q])) task[atomicAdd(&nt0, 1)] = qi[q];
+                __syncthreads();
+                nu = na + nt0;
+                for (int q = na + tid; q < nu; q += T) qi[q] = task[q - na];
+                __syncthreads();
+                if (tid == 0) nt0 = 0;
+            }
+        }
         int ni = 0;
         if (DU) {
             if (tid == 0) Q.tail = nu;
@@ -1943,10 +1956,7 @@ __global__ void __launch_bounds__(SN_T)
             ni = sn_search(S, Q, qi, nu, above, mark_arc);
         }
         // their ranges are tasks, the joins among them relevant too
-        int32_t *task = v.task + io;
-        auto newly = [&](int q) { return q < nu && sn_bit(covi, qi[q]); };  // above the landmark, covered itself
         for (int q = na + tid; q < ni; q += T) {
-            if (newly(q)) continue;
             const int i = qi[q];
             const int j = jid[i];
             if (j >= 0) atomicOr(&rel[j >> 5], 1u << (j & 31));
@@ -1999,7 +2009,6 @@ __global__ void __launch_bounds__(SN_T)
                 rrec[rank2(rel2, j)] = make_int4(covered ? e.x : 0, 0, a.x, a.y);
             };
             for (int q = na + tid; q < ni; q += T) {
-                if (newly(q)) continue;
                 const int i = qi[q], j = jid[i];
                 if (j >= 0) record(j, false);
                 if (v.share[io + i] < 0) rrange[i] = range2((int)sn_lo(v.pj[io + i]), sn_hi(v.acc[io + i]));
@@ -2007,7 +2016,7 @@ __global__ void __launch_bounds__(SN_T)
             sn_expand_n(
                 S, 0, nd + ni - na,
                 [&](int q, int &first, int &len) {
-                    const int j = q < nd ? ql[q] : newly(na + q - nd) ? -1 : jid[qi[na + q - nd]];
+                    const int j = q < nd ? ql[q] : jid[qi[na + q - nd]];
                     if (j < 0) return;
                     if (q < nd) record(j, true);
                     S.aux[tid] = rank2(rel2, j);
