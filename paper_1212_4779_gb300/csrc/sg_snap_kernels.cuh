@@ -1424,7 +1424,7 @@ __device__ __forceinline__ int find_chunk(const int32_t *start, int count, int t
 // time.)  Each warp keeps its bits in shared memory (in global memory, one
 // warp per block, when they are more than that holds) and undoes a small
 // walk's bits one by one instead of clearing all.  R-MAT 20, R = 256: 13.5 ms
-// (MODE 0, 0.8 G join arcs), 19 ms (MODE 2, all rounds, 7 of them the first).
+// (MODE 0, 0.8 G join arcs), 18 ms (MODE 2, all rounds, 6 of them the first).
 template <int MODE, bool EDGES, bool SH>
 __device__ __forceinline__ void walk_tasks(const SnapView &v, Ctl *ctl, long long *s, int area)
 {
