@@ -353,6 +353,7 @@ void srv_admit(sg_server *s, std::unique_lock<std::mutex> &lock)
             }
         if (!free_slot) return;
         if (s->starved && s->running > 0) return;  // asking again before a request ends is in vain
+        s->starved = false;
         SrvRequest *r = s->queue.front();
         bool impossible = false, fresh = false;
         const int wi = srv_workspace(s, r, &impossible, &fresh);

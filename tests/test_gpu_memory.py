@@ -134,18 +134,25 @@ def _serve(sg, sv, requests, together):
     return out + [wait(*i) for i in ids]
 
 
-@pytest.mark.parametrize("together", [False, True])
-def test_server_memory_over_mixed_routes(sg, together):
-    """Undirected, compact and dense requests on one graph: what they hold
-    together stays within the budget, in every order."""
-    import torch
-
+@pytest.fixture(scope="module")
+def mixed():
+    """A symmetric graph, requests of three routes on it, their results."""
     n, s, d = inputs.symmetric(*inputs.er_directed(20000, 60000, 3))
     cases = [("uic_undirected", 0.05, 2000, 6), ("wic", 0.0, 32, 6), ("uic", 0.1, 64, 6)]
     refs = {}
     for model, p, R, k in cases:
         mode = oracle.COVER if model == "uic_undirected" else oracle.DU
         refs[model] = oracle.Graph(n, s, d, model, p).select(R, k, 13, mode=mode)
+    return (n, s, d), cases, refs
+
+
+@pytest.mark.parametrize("together", [False, True])
+def test_server_memory_over_mixed_routes(sg, mixed, together):
+    """Undirected, compact and dense requests on one graph: what they hold
+    together stays within the budget, in every order."""
+    import torch
+
+    (n, s, d), cases, refs = mixed
     budget = 800 << 20
     g = sg.Graph.from_coo(n, s, d)
     # what stays with the graph after its first undirected query
